@@ -105,6 +105,111 @@ def choose_plan(n: int) -> Tuple[int, ...]:
     return tuple(sorted(best[1], reverse=True))
 
 
+# ---------------------------------------------------------------------------
+# Geometry of the FP32 passes: N = R0 R1 R2, the R1 R2-point sub-transforms on
+# groups of 8, 16 or 32 lanes, R0 of them per transform (R0 = 1 for the lengths
+# one group holds).
+# ---------------------------------------------------------------------------
+_FACTOR_COST = {2: 2.0, 3: 5.0, 5: 7.0, 7: 10.0}   # operations per point of one prime factor
+R0_MAX = 42
+
+
+def _dft_cost(r: int) -> float:
+    c = 7.0   # the exchange around the butterfly
+    for p in (2, 3, 5, 7):
+        while r % p == 0:
+            c += _FACTOR_COST[p]
+            r //= p
+    return c
+
+
+def lanes_for(r1: int, r2: int) -> int:
+    m = max(r1, r2)
+    return 8 if m <= 8 else 16 if m <= 16 else 32
+
+
+def candidate_geos(n: int) -> List[Tuple[int, int, int]]:
+    """Factors (R0, R1, R2) by estimated cost: operations per point of each
+    stage, over the share of the lanes it keeps busy (stage 2 runs on R2 of
+    the group's lanes, stage 3 on R1)."""
+    out = []
+    for r1 in range(2, 33):
+        for r2 in range(2, 33):
+            if n % (r1 * r2):
+                continue
+            r0 = n // (r1 * r2)
+            if r0 > R0_MAX or (r0 == 1 and n > 1024) or (r0 > 1 and n <= 1024):
+                continue
+            g = lanes_for(r1, r2)
+            cost = _dft_cost(r1) * g / r2 + _dft_cost(r2) * g / r1
+            if r0 > 1:
+                cost += _dft_cost(r0) + (0 if r0 <= 21 else 3 if r0 <= 32 else 8)
+            cost += 1.0 * (max(r1, r2) > 24) + 0.5 * (r2 % 2)
+            out.append((round(cost, 6), abs(r1 - r2), r2, (r0, r1, r2)))
+    if not out:
+        raise ValueError(f"no block geometry for {n}")
+    return [x[-1] for x in sorted(out)]
+
+
+def choose_geo(n: int) -> Tuple[int, int, int]:
+    return candidate_geos(n)[0]
+
+
+def layout_elems(r: Sequence[int]) -> int:
+    """Complex elements of shared memory of one transform (Lay in fft_core.cuh)."""
+    r0, r1, r2 = r
+    vec = r2 % 2 == 0
+    s1 = r2 if not vec or (r2 // 2) % 2 else r2 + 2
+    s0 = r1 * s1
+    s0 = (s0 | 1) if not vec else s0 if (s0 // 2) % 2 else s0 + 2
+    return (r0 * s0 + 7) // 16 * 16 + 8
+
+
+def pass_smem(r: Sequence[int], nt: int) -> int:
+    """Shared-memory bytes of a pass with nt transforms per block (PassCfg)."""
+    r0, r1, _ = r
+    w1 = (r0 * ((r1 + 1) // 2 * 2) + 7) // 8 * 8 if r0 > 1 else 0
+    return 8 * (w1 + nt * layout_elems(r))
+
+
+def pass_shape(r: Sequence[int], nt: int, extra: int = 0) -> List[int]:
+    """[transforms per block, threads, resident blocks per SM] of one pass:
+    the thread count whose rounds waste least among those with 12 to 40
+    points per thread; resident blocks by shared memory (extra: bytes beside
+    the working set) and by the registers the largest radix needs."""
+    r0, r1, r2 = r
+    n, g = r0 * r1 * r2, lanes_for(r1, r2)
+    if r0 == 1:
+        th = max(32, min(128, nt * g))
+        nt = th // g
+    else:
+        best = None
+        for w in range(1, 25):
+            t = 32 * w
+            if not 12 <= n * nt / t <= 36:
+                continue
+            u1, ub, gr = r1 * r2 * nt, r0 * nt, w * (32 // g)
+            waste = -(-u1 // t) * t / u1 + 2.0 * (-(-ub // gr) * gr / ub)
+            key = (round(waste, 3) + (0.4 if t > 512 else 0.0), -w)
+            if best is None or key < best[0]:
+                best = (key, t)
+        th = best[1]
+    smem = pass_smem(r, nt) + extra
+    regs = max(64, 2 * max(r) + 32)
+    by_smem = (228 * 1024) // (smem + 1024)
+    by_regs = 65536 // (th * (regs + 7) // 8 * 8)
+    return [nt, th, max(1, min(by_smem, by_regs, 16))]
+
+
+def geo_plan(r: Sequence[int]) -> dict:
+    """Pass shapes of a geometry before any measurement."""
+    n = r[0] * r[1] * r[2]
+    two = 8 if r[0] == 1 else 2 if n <= 5120 else 1
+    pm_nt = 4 if r[0] == 1 else 2 if n <= 2560 else 1
+    return dict(r=list(r), p1=pass_shape(r, two), p2=pass_shape(r, two), p3=pass_shape(r, two),
+                pm=pass_shape(r, pm_nt, 8 * pm_nt * n), grp=2 if n > 5120 else 1)
+
+
 TUNED_JSON = os.path.join(HERE, "tuned_plans.json")
 
 
@@ -137,7 +242,7 @@ def plan_table_entry(n: int) -> dict:
             break
     return dict(radices=list(r), threads=t, f1=f, f3=f, smem=smem,
                 upb=[PF_UNITS] * 3, minb=[1, 1, 1], kstage=True, tt=0, pf=[1, 1, 1], db=[0, 0, 0],
-                batch=True)
+                batch=True, geo=geo_plan(choose_geo(n)))
 
 
 def plan_table() -> Dict[int, dict]:
@@ -161,6 +266,8 @@ def plan_table() -> Dict[int, dict]:
                      late=list(t.get("late", DEFAULT_LATE)))
             if e["tt"]:
                 e["threads"] = e["tt"]
+            if "geo" in t:
+                e["geo"] = dict(t["geo"])
         table[n] = e
     return table
 
@@ -175,38 +282,27 @@ _SIZE_TU = """// generated by paper_1907_02891_gb300/build.py -- one supported F
 namespace lpk {{
 namespace {{
 constexpr int kN = {n};
-using P = Plan<kN, Seq<{seq}>, {tt}>;   // threads per transform (0 = one butterfly each)
-constexpr int kF1 = {f1}, kF3 = {f3};
-constexpr int kSmem = P::SMEM_BYTES;
-constexpr long long kMaxSmem = 227 * 1024;
-// tuned parameters of the prefetching kernels: work units per block and
-// minimum resident blocks per SM (register cap) per pass; spectrum staging
-constexpr int kUPB1 = {upb1}, kUPB2 = {upb2}, kUPB3 = {upb3};
-constexpr int kMINB1 = {minb1}, kMINB2 = {minb2}, kMINB3 = {minb3};
-constexpr bool kKSTAGE = {kstage};
-constexpr bool kPF1 = {pf1}, kPF2 = {pf2}, kPF3 = {pf3};   // prefetching form allowed per pass
-constexpr bool kDB1 = {db1}, kDB2 = {db2}, kDB3 = {db3};   // double-buffered exchange per pass
-// forward row pass / one-spectrum column pass: the next kernel launches as
-// this one's blocks exit instead of once they have all started
-constexpr bool kLATE1 = {late1}, kLATE2 = {late2};
-// several spectra: the batched column kernel (forward column parked in global
-// memory, one product + inverse per spectrum) or one single-spectrum pass per
-// spectrum (forward transform repeated)
+using Ge = Geo<kN, {geo}>;
+// shape of each pass: transforms per block, threads, resident blocks
+using C1 = PassCfg<Ge, {p1}, {late1}>;
+using C2 = PassCfg<Ge, {p2}, {late2}>;
+using C3 = PassCfg<Ge, {p3}, {late3}>;
+using CM = PassCfg<Ge, {pm}, {late2}>;   // several spectra or classes
+// the passes over several spectra or classes keep one parked column (set)
+// beside their working sets: in shared memory where that fits, else in
+// global memory; kGrp groups share the parked column
+constexpr int kMaxSmem = 227 * 1024;
+constexpr int kParkB = 8 * CM::NT * kN;
+constexpr bool kParkG = kParkB + CM::SMEM > kMaxSmem;
+constexpr int kSmemG = kParkB + CM::SMEM + ({grp} - 1) * 8 * CM::WORK;
+constexpr int kGrp = !kParkG && kSmemG <= kMaxSmem && CM::TH * {grp} <= 1024 ? {grp} : 1;
+constexpr int kSmemM = kGrp > 1 ? kSmemG : (kParkG ? 0 : kParkB) + CM::SMEM;
+constexpr int kSmemC = (kParkG ? 0 : kParkB) + CM::SMEM;
+// several spectra: the batched column kernel (one forward transform, one
+// product + inverse per spectrum) or one single-spectrum pass per spectrum
 constexpr bool kBatch = {batch};
-// the batched column kernel parks its forward column in shared memory where
-// it fits next to the exchange buffer, else in global memory
-constexpr bool kParkG = P::SMEM_BYTES + 8 * kN > kMaxSmem;
-constexpr int kSmemM = kParkG ? kSmem : kSmem + 8 * kN;
-constexpr int kX1 = kDB1 ? 2 : 1, kX2 = kDB2 ? 2 : 1, kX3 = kDB3 ? 2 : 1;
-// one-unit-per-block column kernel: spectrum column staged in shared memory
-// (where the staging fits next to the exchange buffer)
-constexpr bool kKST2 = {kst2};
-constexpr bool kKstOk(bool kreal)
-{{
-    return kKST2 && (long long)kX2 * kSmem + (kreal ? 4 : 8) * ((kN + 3) / 4 * 4) <= kMaxSmem;
-}}
-constexpr int kKst(bool kreal) {{ return kKstOk(kreal) ? (kreal ? 4 : 8) * ((kN + 3) / 4 * 4) : 0; }}
 // split-precision tensor-core column pass (0 shared bytes: not available)
+using P = Plan<kN, Seq<{seq}>>;
 using TP = TcPlan<P, kN>;
 constexpr bool kTC = TP::FITS;
 constexpr int kTcSmem = kTC ? TP::SMEM_BYTES : 0;
@@ -217,77 +313,58 @@ cudaError_t attr(K k, int bytes)
     return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
 }}
 
-// blocks of a prefetching launch: each block takes upb units
-inline int persistent_grid(int units, int upb) {{ return (units + upb - 1) / upb; }}
-
 cudaError_t set_attrs()
 {{
     cudaError_t e;
-    if ((e = attr(p1_rows<P, kN, kF1, kLATE1>, kF1 * kSmem)) != cudaSuccess) return e;
-    if ((e = attr(p2_cols<P, kN, true, false, kMINB2, kDB2, kKstOk(true), false, kLATE2>, kX2 * kSmem + kKst(true))) != cudaSuccess) return e;
-    if ((e = attr(p2_cols<P, kN, false, false, kMINB2, kDB2, kKstOk(false), false, kLATE2>, kX2 * kSmem + kKst(false))) != cudaSuccess) return e;
-    if ((e = attr(p2_cols<P, kN, true, true, 1, false, false, kParkG>, kSmemM)) != cudaSuccess) return e;
-    if ((e = attr(p2_cols<P, kN, false, true, 1, false, false, kParkG>, kSmemM)) != cudaSuccess) return e;
-    if ((e = attr(p2_multiclass<P, kN, true>, kSmem)) != cudaSuccess) return e;
-    if ((e = attr(p2_multiclass<P, kN, false>, kSmem)) != cudaSuccess) return e;
-    if ((e = attr(p3_rows<P, kN, kF3>, kF3 * kSmem)) != cudaSuccess) return e;
+    if ((e = attr(p1_rows<C1>, C1::SMEM)) != cudaSuccess) return e;
+    if ((e = attr(p2_cols<C2, true>, C2::SMEM)) != cudaSuccess) return e;
+    if ((e = attr(p2_cols<C2, false>, C2::SMEM)) != cudaSuccess) return e;
+    if ((e = attr(p2_cols_multi<CM, kGrp, kParkG, true>, kSmemM)) != cudaSuccess) return e;
+    if ((e = attr(p2_cols_multi<CM, kGrp, kParkG, false>, kSmemM)) != cudaSuccess) return e;
+    if ((e = attr(p2_multiclass<CM, kParkG, true>, kSmemC)) != cudaSuccess) return e;
+    if ((e = attr(p2_multiclass<CM, kParkG, false>, kSmemC)) != cudaSuccess) return e;
     if constexpr (kTC) {{
         if ((e = attr(p2_cols_tc<P, kN, true>, kTcSmem)) != cudaSuccess) return e;
         if ((e = attr(p2_cols_tc<P, kN, false>, kTcSmem)) != cudaSuccess) return e;
     }}
-    if ((e = attr(p1_rows_pf<P, kN, kUPB1, kMINB1, kDB1, kLATE1>, (int)kMaxSmem)) != cudaSuccess) return e;
-    if ((e = attr(p2_cols_pf<P, kN, true, kUPB2, kMINB2, kKSTAGE, kDB2, kLATE2>, (int)kMaxSmem)) != cudaSuccess) return e;
-    if ((e = attr(p2_cols_pf<P, kN, false, kUPB2, kMINB2, kKSTAGE, kDB2, kLATE2>, (int)kMaxSmem)) != cudaSuccess) return e;
-    return attr(p3_rows_pf<P, kN, kUPB3, kMINB3, kDB3>, (int)kMaxSmem);
+    return attr(p3_rows<C3>, C3::SMEM);
 }}
 
 cudaError_t p1(const P1Args& a, cudaStream_t s)
 {{
-    const long long sm = kX1 * kSmem + p1_stage_bytes(a.Wst);
-    if (kPF1 && sm <= kMaxSmem)
-        return launch_pdl(p1_rows_pf<P, kN, kUPB1, kMINB1, kDB1, kLATE1>, dim3(persistent_grid(a.npairs - a.pair0, kUPB1)),
-                          dim3(P::T), sm, s, a);
-    return launch_pdl(p1_rows<P, kN, kF1, kLATE1>, dim3((a.npairs - a.pair0 + kF1 - 1) / kF1), dim3(P::T * kF1),
-                      kF1 * kSmem, s, a);
+    return launch_pdl(p1_rows<C1>, dim3((a.npairs - a.pair0 + C1::NT - 1) / C1::NT), dim3(C1::TH), C1::SMEM, s, a);
 }}
 
 cudaError_t p2(const P2Args& a, bool kreal, cudaStream_t s)
 {{
-    const bool multi = a.nspec > 1;
-    const long long sm = kX2 * kSmem + p2_stage_bytes(a.ldT, a.ldK, kreal, kKSTAGE);
-    if (!multi) {{
-        const dim3 gpf(persistent_grid(a.ncols, kUPB2));
-        if (kPF2 && sm <= kMaxSmem)
-            return kreal ? launch_pdl(p2_cols_pf<P, kN, true, kUPB2, kMINB2, kKSTAGE, kDB2, kLATE2>, gpf, dim3(P::T), sm, s, a)
-                         : launch_pdl(p2_cols_pf<P, kN, false, kUPB2, kMINB2, kKSTAGE, kDB2, kLATE2>, gpf, dim3(P::T), sm, s, a);
-        return kreal ? launch_pdl(p2_cols<P, kN, true, false, kMINB2, kDB2, kKstOk(true), false, kLATE2>, dim3(a.ncols), dim3(P::T),
-                                  kX2 * kSmem + kKst(true), s, a)
-                     : launch_pdl(p2_cols<P, kN, false, false, kMINB2, kDB2, kKstOk(false), false, kLATE2>, dim3(a.ncols), dim3(P::T),
-                                  kX2 * kSmem + kKst(false), s, a);
+    if (a.nspec == 1) {{
+        const dim3 g((a.ncols + C2::NT - 1) / C2::NT);
+        return kreal ? launch_pdl(p2_cols<C2, true>, g, dim3(C2::TH), C2::SMEM, s, a)
+                     : launch_pdl(p2_cols<C2, false>, g, dim3(C2::TH), C2::SMEM, s, a);
     }}
     if (kBatch && (!kParkG || a.park)) {{
-        return kreal ? launch_pdl(p2_cols<P, kN, true, true, 1, false, false, kParkG>, dim3(a.ncols), dim3(P::T), kSmemM, s, a)
-                     : launch_pdl(p2_cols<P, kN, false, true, 1, false, false, kParkG>, dim3(a.ncols), dim3(P::T), kSmemM, s, a);
-    }} else {{
-        // one single-spectrum pass per spectrum (no room to park the forward
-        // column, or the plan measured this faster)
-        for (int i = 0; i < a.nspec; ++i) {{
-            P2Args b = a;
-            b.K[0] = a.K[i];
-            b.nspec = 1;
-            b.U = a.U + (long long)i * a.specU;
-            b.u_elems = a.u_elems - (long long)i * a.specU;
-            cudaError_t e = p2(b, kreal, s);
-            if (e != cudaSuccess) return e;
-        }}
-        return cudaSuccess;
+        const dim3 g((a.ncols + CM::NT - 1) / CM::NT);
+        return kreal ? launch_pdl(p2_cols_multi<CM, kGrp, kParkG, true>, g, dim3(CM::TH * kGrp), kSmemM, s, a)
+                     : launch_pdl(p2_cols_multi<CM, kGrp, kParkG, false>, g, dim3(CM::TH * kGrp), kSmemM, s, a);
     }}
+    // one single-spectrum pass per spectrum (the plan measured this faster)
+    for (int i = 0; i < a.nspec; ++i) {{
+        P2Args b = a;
+        b.K[0] = a.K[i];
+        b.nspec = 1;
+        b.U = a.U + (long long)i * a.specU;
+        b.u_elems = a.u_elems - (long long)i * a.specU;
+        cudaError_t e = p2(b, kreal, s);
+        if (e != cudaSuccess) return e;
+    }}
+    return cudaSuccess;
 }}
 
 cudaError_t p2m(const P2MArgs& a, bool kreal, cudaStream_t s)
 {{
-    return kreal ? launch_pdl(p2_multiclass<P, kN, true>, dim3(a.ncols), dim3(P::T), kSmem, s, a)
-                 : launch_pdl(p2_multiclass<P, kN, false>, dim3(a.ncols), dim3(P::T), kSmem, s, a);
+    const dim3 g((a.a.ncols + CM::NT - 1) / CM::NT);
+    return kreal ? launch_pdl(p2_multiclass<CM, kParkG, true>, g, dim3(CM::TH), kSmemC, s, a)
+                 : launch_pdl(p2_multiclass<CM, kParkG, false>, g, dim3(CM::TH), kSmemC, s, a);
 }}
 
 // persistent grid of the tensor-core column pass: resident blocks per SM
@@ -331,16 +408,11 @@ cudaError_t p2tc(const P2TcArgs& a, bool kreal, cudaStream_t s)
 
 cudaError_t p3(const P3Args& a, int nspec, cudaStream_t s)
 {{
-    const long long sm = kX3 * kSmem + p3_stage_bytes(a.ncols);
-    if (kPF3 && sm <= kMaxSmem)
-        return launch_pdl(p3_rows_pf<P, kN, kUPB3, kMINB3, kDB3>, dim3(persistent_grid(a.npairs - a.pair0, kUPB3), nspec),
-                          dim3(P::T), sm, s, a);
-    return launch_pdl(p3_rows<P, kN, kF3>, dim3((a.npairs - a.pair0 + kF3 - 1) / kF3, nspec), dim3(P::T * kF3),
-                      kF3 * kSmem, s, a);
+    return launch_pdl(p3_rows<C3>, dim3((a.npairs - a.pair0 + C3::NT - 1) / C3::NT, nspec), dim3(C3::TH), C3::SMEM, s, a);
 }}
 }}  // namespace
 
-extern const SizeKernels kSize_{n} = {{kN, {ns}, {{{rad6}}}, P::T, kF1, kF3, kSmem, kBatch ? 1 : 0,
+extern const SizeKernels kSize_{n} = {{kN, {{{geo}}}, Ge::VK, {ns}, {{{rad6}}}, kBatch ? 1 : 0, kParkG ? 1 : 0, kParkG ? 1 : 0,
                                        set_attrs, p1, p2, p2m, p3,
                                        kTC ? TP::THREADS : 0, kTcSmem, p2tc}};
 }}  // namespace lpk
@@ -370,6 +442,17 @@ def _write_if_changed(path: str, text: str) -> None:
         fh.write(text)
 
 
+def size_tu(n: int, p: dict) -> str:
+    """Translation unit of one length with plan p."""
+    r, g = list(p["radices"]), p["geo"]
+    late = p.get("late", DEFAULT_LATE)
+    return _SIZE_TU.format(n=n, seq=", ".join(map(str, r)), ns=len(r), rad6=", ".join(map(str, r + [0] * (6 - len(r)))),
+                           geo=", ".join(map(str, g["r"])), grp=g["grp"],
+                           **{k: ", ".join(map(str, g[k])) for k in ("p1", "p2", "p3", "pm")},
+                           batch=_b(p.get("batch", True)), packed=int(bool(p.get("packed", False))),
+                           late1=_b(late[0]), late2=_b(late[1]), late3=_b(late[2]))
+
+
 def generate(sizes: Sequence[int] = ()) -> List[str]:
     """Write one translation unit per supported length (all, or `sizes`)
     and the registry of the lengths written; returns their paths.  A
@@ -383,18 +466,7 @@ def generate(sizes: Sequence[int] = ()) -> List[str]:
     os.makedirs(gen, exist_ok=True)
     files = []
     for n, p in table.items():
-        r = list(p["radices"])
-        text = _SIZE_TU.format(n=n, seq=", ".join(map(str, r)), f1=p["f1"], f3=p["f3"], ns=len(r),
-                               tt=p.get("tt", 0),
-                               upb1=p["upb"][0], upb2=p["upb"][1], upb3=p["upb"][2],
-                               minb1=p["minb"][0], minb2=p["minb"][1], minb3=p["minb"][2],
-                               kstage="true" if p["kstage"] else "false",
-                               pf1=_b(p["pf"][0]), pf2=_b(p["pf"][1]), pf3=_b(p["pf"][2]),
-                               db1=_b(p["db"][0]), db2=_b(p["db"][1]), db3=_b(p["db"][2]),
-                               batch=_b(p.get("batch", True)),
-                               kst2=_b(p.get("kst2", False)), packed=int(bool(p.get("packed", False))),
-                               late1=_b(p.get("late", DEFAULT_LATE)[0]), late2=_b(p.get("late", DEFAULT_LATE)[1]),
-                               rad6=", ".join(map(str, r + [0] * (6 - len(r)))))
+        text = size_tu(n, p)
         path = os.path.join(gen, f"size_{n}.cu")
         _write_if_changed(path, text)
         files.append(path)

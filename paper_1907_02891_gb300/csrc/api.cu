@@ -76,6 +76,15 @@ extern "C" int lp_supported_size(int n)
     return best;
 }
 
+// Order of a spectrum's columns: the FP32 passes read the frequencies in
+// stage-3 run order (Geo::kpos), the tensor-core pass in natural order.
+static SpecOrder spectrum_order(int ny, lp_precision prec)
+{
+    const SizeKernels* k = find_size(ny);
+    if (!k || prec != LP_PREC_FP32) return SpecOrder{0, 0, 0, 0};
+    return SpecOrder{k->geo[0], k->geo[1], k->geo[2], k->vk};
+}
+
 extern "C" int lp_split_supported(int n)
 {
     const SizeKernels* k = find_size(n);
@@ -221,6 +230,24 @@ static void fill_chain_tables(const int* r, int ns, std::vector<float2>& host, s
     }
 }
 
+// the block transform's twiddle tables (BlkTw): w1, then w2
+static size_t block_w1_entries(const int* g) { return (size_t)g[0] * ((g[1] + 1) / 2 * 2); }
+static size_t block_table_entries(const int* g) { return block_w1_entries(g) + (size_t)g[0] * g[1] * g[2]; }
+
+static void fill_block_tables(const int* g, float2* t)
+{
+    const long r0 = g[0], r1 = g[1], r2 = g[2], n = r0 * r1 * r2, r1p = (r1 + 1) / 2 * 2;
+    auto put = [&t](long a, long len) {
+        const double th = 2.0 * M_PI * (double)(a % len) / (double)len;
+        *t++ = make_float2((float)std::cos(th), (float)-std::sin(th));
+    };
+    for (long m = 0; m < r0; ++m)
+        for (long l = 0; l < r1p; ++l) put(l * m, r0 * r1);
+    for (long m = 0; m < r0; ++m)
+        for (long k = 0; k < r1; ++k)
+            for (long i = 0; i < r2; ++i) put(i * (m + r0 * k), n);
+}
+
 // BF16 of x, round to nearest even (finite inputs)
 static uint16_t bf16_rn(float x)
 {
@@ -326,7 +353,8 @@ lp_status lp_get_plan(lp_ctx* ctx, int N, const PlanRec** out)
     const size_t nf = chain_table_entries(fwd, ns), nr = chain_table_entries(rev, ns);
     // one device block: twiddle tables, then (256-byte aligned) the split
     // DFT matrices of the tensor-core column pass where this length has one
-    const size_t tw_bytes = (nf + nr + 1) * sizeof(float2);
+    const size_t nblk = block_table_entries(k->geo);
+    const size_t tw_bytes = (nf + nr + nblk + 1) * sizeof(float2);
     const size_t tc_off = (tw_bytes + 255) / 256 * 256;
     // (matrices of the forward stages -- the inverse chain runs in the
     // conjugate domain on the same ones --, then the step factors of the
@@ -337,10 +365,11 @@ lp_status lp_get_plan(lp_ctx* ctx, int N, const PlanRec** out)
     const size_t total = k->tc_smem > 0 ? tc_off + (tcf + tsf + tsr + 15) / 16 * 16 : tw_bytes;
     std::vector<unsigned char> host(total, 0);
     float2* htw = reinterpret_cast<float2*>(host.data());
-    std::vector<float2> tw(nf + nr + 1);
+    std::vector<float2> tw(nf + nr + nblk + 1);
     size_t of[6] = {0}, orv[6] = {0};
     fill_chain_tables(fwd, ns, tw, 0, of);
     fill_chain_tables(rev, ns, tw, nf, orv);
+    fill_block_tables(k->geo, tw.data() + nf + nr);
     std::memcpy(htw, tw.data(), tw.size() * sizeof(float2));
     if (k->tc_smem > 0) {
         fill_tc_mats(fwd, ns, -1, reinterpret_cast<uint16_t*>(host.data() + tc_off));
@@ -363,6 +392,8 @@ lp_status lp_get_plan(lp_ctx* ctx, int N, const PlanRec** out)
         rec->fwd.p[s] = s < ns ? rec->tw + of[s] : nullptr;
         rec->rev.p[s] = s < ns ? rec->tw + orv[s] : nullptr;
     }
+    rec->blk.w1 = rec->tw + nf + nr;
+    rec->blk.w2 = rec->blk.w1 + block_w1_entries(k->geo);
     if (k->tc_smem > 0) rec->tc_tables = static_cast<char*>(d) + tc_off;
     *out = rec.get();
     ctx->plans.emplace(N, std::move(rec));
@@ -643,7 +674,7 @@ extern "C" lp_status lp_kernel_spectrum(lp_ctx* ctx, const double* K, int hk, in
     e = cudaMemcpyAsync(spec->kcopy, K, spec->kbytes, cudaMemcpyDeviceToDevice, st);
     if (e == cudaSuccess) e = cudaMemsetAsync(dptr, 0, bytes, st);
     if (e == cudaSuccess)
-        e = psf_spectrum_build(K, hk, wk, Ny, Nx, is_real, dptr, ldK, (double2*)scratch,
+        e = psf_spectrum_build(K, hk, wk, Ny, Nx, is_real, dptr, ldK, spectrum_order(Ny, prec), (double2*)scratch,
                                (double2*)(scratch + w1), (double2*)(scratch + 2 * w1),
                                (double2*)(scratch + 2 * w1 + w2), st);
     cudaFreeAsync(scratch, st);
@@ -699,6 +730,12 @@ extern "C" lp_status lp_spectrum_copy(const lp_spectrum* s, float* dst, size_t d
         return lp_fail(LP_ERR_INVALID, "lp_spectrum_copy: destination holds %zu floats, need %zu",
                        dst_floats, ncols * s->ny * per);
     DeviceGuard dg(s->ctx->device);
+    const SpecOrder o = spectrum_order(s->ny, s->prec);
+    if (o.r0 > 0) {
+        CUDA_TRY(spectrum_copy_natural(s->data, s->ldK, s->ny, (int)ncols, s->is_real, o, dst,
+                                       static_cast<cudaStream_t>(stream)));
+        return LP_OK;
+    }
     CUDA_TRY(cudaMemcpy2DAsync(dst, (size_t)s->ny * per * 4, s->data, (size_t)s->ldK * per * 4,
                                (size_t)s->ny * per * 4, ncols, cudaMemcpyDeviceToDevice,
                                static_cast<cudaStream_t>(stream)));
@@ -854,15 +891,15 @@ static void map_dims(int h, int w, int ny, int nx, int hk, int wk, lp_outmode mo
     d->batch = (k && k->batch) ? 1 : 0;
 }
 
-size_t lp_park_bytes(const MapDims& d) { return 8ull * (size_t)d.ncols * (size_t)d.ny; }
+// (whole blocks of columns: the passes park up to kUCB columns side by side)
+size_t lp_park_bytes(const MapDims& d) { return 8ull * (size_t)d.ncolsU * (size_t)d.ny; }
 
 // the batched column pass parks its forward column spectra in the workspace
 // where they do not fit shared memory next to the exchange buffer
 static inline bool uses_park(const MapDims& d, int nchunk)
 {
     const SizeKernels* k = find_size(d.ny);
-    const bool global_park = k && (long long)k->smem_bytes + 8ll * d.ny > 227ll * 1024;
-    return nchunk > 1 && d.batch && global_park && d.prec == (int)LP_PREC_FP32;
+    return nchunk > 1 && d.batch && k && k->park_multi && d.prec == (int)LP_PREC_FP32;
 }
 
 size_t lp_workspace_bytes(const MapDims& d, int n)
@@ -955,32 +992,18 @@ static lp_status launch_rows_forward(lp_ctx* ctx, const PlanRec* px, const float
     a1.ldl = ldl;
     a1.H = h;
     a1.W = w;
-    a1.Wst = (w + 3) / 4 * 4;
-    a1.vec16 = ((reinterpret_cast<uintptr_t>(L) & 15) == 0 && ldl % 4 == 0 && w % 4 == 0) ? 1 : 0;
     a1.T = T;
     a1.ldT = d.ldT;
     a1.pair0 = pair0;
     a1.npairs = pair1;
     a1.ncols = d.ncols;
-    a1.tw = px->fwd;
+    a1.tw = px->blk;
     a1.err = ctx->d_err;
     a1.t_elems = t_extent(ctx, d);
     const int tok = lp_pass_begin(ctx, 0, st);
     CUDA_TRY(px->k->p1(a1, st));
     lp_pass_end(ctx, tok, st);
     return LP_OK;
-}
-
-// Column distance of the column pass's T prefetch: about one wave of
-// resident blocks (three per SM), computed once per context.
-static int prefetch_ahead(lp_ctx* ctx)
-{
-    if (ctx->sms == 0) {
-        int sms = 0;
-        if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ctx->device) != cudaSuccess) sms = 0;
-        ctx->sms = sms > 0 ? sms : -1;
-    }
-    return ctx->sms > 0 ? 3 * ctx->sms : 0;
 }
 
 // column pass for spectra [base, base+cnt) into U (cnt blocks of ncols x ldU)
@@ -1008,10 +1031,10 @@ static lp_status launch_columns(lp_ctx* ctx, const PlanRec* py, const lp_spectru
             b.Hout = d.Hout;
             b.HoutPad = (int)d.ldU;
             b.ncols = d.ncols;
-            b.twf = py->fwd;
-            b.twi = py->rev;
+            b.tw = py->blk;
+            a2.twf = py->fwd;
+            a2.twi = py->rev;
             b.park = nullptr;
-            b.ahead = 0;
             b.err = ctx->d_err;
             b.t_elems = t_extent(ctx, d);
             b.u_elems = (long long)d.ncolsU * d.ldU;
@@ -1048,10 +1071,8 @@ static lp_status launch_columns(lp_ctx* ctx, const PlanRec* py, const lp_spectru
         a2.Hout = d.Hout;
         a2.HoutPad = (int)d.ldU;
         a2.ncols = d.ncols;
-        a2.twf = py->fwd;
-        a2.twi = py->rev;
+        a2.tw = py->blk;
         a2.park = park;
-        a2.ahead = prefetch_ahead(ctx);
         a2.err = ctx->d_err;
         a2.t_elems = t_extent(ctx, d);
         a2.u_elems = (long long)(cnt - k0) * d.ncolsU * d.ldU;
@@ -1081,7 +1102,7 @@ static lp_status launch_rows_inverse(lp_ctx* ctx, const PlanRec* px, const MapDi
     a3.c0 = d.c0;
     a3.Wout = d.Wout;
     a3.ncols = d.ncols;
-    a3.tw = px->rev;
+    a3.tw = px->blk;
     a3.err = ctx->d_err;
     a3.u_elems = (long long)cnt * d.ncolsU * d.ldU;
     const int tok = lp_pass_begin(ctx, 2, st);
@@ -1467,8 +1488,8 @@ extern "C" lp_status lp_map_multiclass(lp_ctx* ctx, const float* const* L, int T
     const size_t tbytes = 8ull * (size_t)d.ncolsT * d.ldT;
     const size_t ubytes = 8ull * (size_t)d.ncolsU * d.ldU;
     void* ws = nullptr;
-    if ((st = lp_get_workspace(ctx, s, (size_t)T * tbytes + ubytes + lp_park_bytes(d) + 512, &ws)) != LP_OK)
-        return st;
+    const size_t sums = py->k->park_class ? lp_park_bytes(d) : 0;  // Eq. (4)'s sums, where not in shared memory
+    if ((st = lp_get_workspace(ctx, s, (size_t)T * tbytes + ubytes + sums + 512, &ws)) != LP_OK) return st;
     float2* Tb = static_cast<float2*>(ws);
     float2* U = Tb + (size_t)T * d.ncolsT * d.ldT;
     float2* accb = park_of(d, U, 1);
@@ -1480,14 +1501,12 @@ extern "C" lp_status lp_map_multiclass(lp_ctx* ctx, const float* const* L, int T
         a1.ldl = ldl;
         a1.H = h;
         a1.W = w;
-        a1.Wst = (w + 3) / 4 * 4;
-        a1.vec16 = ((reinterpret_cast<uintptr_t>(L[t]) & 15) == 0 && ldl % 4 == 0 && w % 4 == 0) ? 1 : 0;
         a1.T = Tb + (size_t)t * d.ncolsT * d.ldT;
         a1.ldT = d.ldT;
         a1.pair0 = 0;
         a1.npairs = npairs;
         a1.ncols = d.ncols;
-        a1.tw = px->fwd;
+        a1.tw = px->blk;
         a1.err = ctx->d_err;
         a1.t_elems = t_extent(ctx, d);
         CUDA_TRY(px->k->p1(a1, s));
@@ -1504,26 +1523,30 @@ extern "C" lp_status lp_map_multiclass(lp_ctx* ctx, const float* const* L, int T
     for (int i = 0; i < kMaxSpectraPerLaunch; ++i) {
         a2.T[i] = i < T ? Tb + (size_t)i * d.ncolsT * d.ldT : nullptr;
         a2.K[i] = i < T ? spectra[i]->data : nullptr;
+        a2.a.K[i] = nullptr;
     }
-    a2.ldT = d.ldT;
-    a2.H = h;
-    a2.ldK = s0->ldK;
     a2.nclass = T;
-    a2.U = U;
-    a2.ldU = d.ldU;
-    a2.r0 = d.r0;
-    a2.Hout = d.Hout;
-    a2.HoutPad = (int)d.ldU;
-    a2.ncols = d.ncols;
-    a2.twf = py->fwd;
-    a2.twi = py->rev;
-    a2.acc = accb;
-    a2.err = ctx->d_err;
-    a2.t_elems = t_extent(ctx, d);
-    a2.k_elems = k_extent(spectra[0]);
-    for (int t = 1; t < T; ++t) a2.k_elems = std::min(a2.k_elems, k_extent(spectra[t]));
-    a2.u_elems = (long long)d.ncolsU * d.ldU;
-    a2.acc_elems = (long long)d.ncols * d.ny;
+    P2Args& b2 = a2.a;
+    b2.T = nullptr;
+    b2.ldT = d.ldT;
+    b2.H = h;
+    b2.ldK = s0->ldK;
+    b2.nspec = 1;
+    b2.U = U;
+    b2.ldU = d.ldU;
+    b2.specU = 0;
+    b2.r0 = d.r0;
+    b2.Hout = d.Hout;
+    b2.HoutPad = (int)d.ldU;
+    b2.ncols = d.ncols;
+    b2.tw = py->blk;
+    b2.park = sums ? accb : nullptr;
+    b2.err = ctx->d_err;
+    b2.t_elems = t_extent(ctx, d);
+    b2.k_elems = k_extent(spectra[0]);
+    for (int t = 1; t < T; ++t) b2.k_elems = std::min(b2.k_elems, k_extent(spectra[t]));
+    b2.u_elems = (long long)d.ncolsU * d.ldU;
+    b2.park_elems = (long long)(sums / 8);
     {
         const cudaError_t e = py->k->p2m(a2, all_real, s);
         if (e != cudaSuccess) return lp_fail(LP_ERR_CUDA, "lp_map_multiclass: %s", cudaGetErrorString(e));
@@ -1540,7 +1563,7 @@ extern "C" lp_status lp_map_multiclass(lp_ctx* ctx, const float* const* L, int T
     a3.c0 = d.c0;
     a3.Wout = d.Wout;
     a3.ncols = d.ncols;
-    a3.tw = px->rev;
+    a3.tw = px->blk;
     a3.err = ctx->d_err;
     a3.u_elems = (long long)d.ncolsU * d.ldU;
     CUDA_TRY(px->k->p3(a3, 1, s));

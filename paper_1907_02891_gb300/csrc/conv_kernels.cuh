@@ -40,9 +40,9 @@ namespace lpk {
 // with ld the (even) number of rows stored per column.  The row passes,
 // which handle all columns of one row pair, then move 16 CB contiguous
 // bytes per column block instead of 16 scattered ones; the column pass
-// reads / writes a column at a 16 CB-byte stride.  Measured at 4704^2 for
-// T: row pass 74 -> 58 us, column pass 68 -> 70 us with CB = 2 (with 4 / 8:
-// 55.5 / 53.7 and 74 / 80 us).  The CB-1 columns past the last one that
+// reads / writes a column at a 16 CB-byte stride.  Measured at 4704^2 with
+// blocks of 1 / 2 / 4 / 8 for T: row pass 73 / 43.4 / 40.0 / 37.0 us; column
+// pass, T and U alike, 51.6 / 55.0 / 67.1 / 86.0 us.  The CB-1 columns past the last one that
 // padding adds to a partial last block are allocated and never touched.
 template <int CB>
 __host__ __device__ constexpr long long blk_cols_alloc(long long ncols) { return (ncols + CB - 1) / CB * CB; }
@@ -56,10 +56,9 @@ template <int CB>
 __host__ __device__ __forceinline__ long long blk_row(int r) { return (long long)(r >> 1) * (2 * CB) + (r & 1); }
 
 constexpr int kTCB = 2;  // T: written by the forward row pass, read by the column pass
-// U: written by the column pass, read by the inverse row pass.  Measured
-// (column / inverse row pass, us), blocks of 1 / 2 / 4:
-//   4704^2:   70.3 / 72.4 / 75.5  and  59.7 / 57.0 / 54.9
-//   17280^2:  1049 / 1142 / 1145  and  1225 / 994 / 851
+// U: written by the column pass, read by the inverse row pass.  Measured at
+// 4704^2, blocks of 1 / 2 / 4 / 8 (T in blocks of 2 for 2 and 4): inverse row
+// pass 56.2 / 45.9 / 39.6 / 37.3 us, column pass 51.6 / 55.0 / 59.7 / 86.0 us.
 constexpr int kUCB = 4;
 __host__ __device__ constexpr long long t_cols_alloc(long long ncols) { return blk_cols_alloc<kTCB>(ncols); }
 __host__ __device__ constexpr long long u_cols_alloc(long long ncols) { return blk_cols_alloc<kUCB>(ncols); }
@@ -87,14 +86,12 @@ struct P1Args {
     const float* L;
     long long ldl;
     int H, W;
-    int Wst;    // staged row length (floats): W rounded up to a multiple of 4
-    int vec16;  // rows can be copied in 16-byte pieces (aligned base, ldl % 4 == 0, W % 4 == 0)
     float2* T;
     long long ldT;
     int pair0;   // first row pair of this launch (pairs pair0 .. npairs-1)
     int npairs;  // ceil(H/2)
     int ncols;   // Nx/2 + 1
-    TwChain tw;  // forward chain of the row plan
+    BlkTw tw;    // of the row length
     int* err;            // device status word (debug builds: bounds checks)
     long long t_elems;   // float2 elements of the T buffer
 };
@@ -113,9 +110,8 @@ struct P2Args {
     int Hout;         // kept rows
     int HoutPad;      // 2 ceil(Hout/2): rows written (the extra one is zero)
     int ncols;
-    TwChain twf, twi;  // forward and reversed chains of the column plan
+    BlkTw tw;          // of the column length
     float2* park;      // batched pass: forward column spectra, N per column
-    int ahead;         // column distance of the T prefetch into L2 (0: none)
     int* err;              // device status word (debug builds: bounds checks)
     long long t_elems;     // float2 elements of the T buffer
     long long u_elems;     // float2 elements of U from a.U on (all spectra of the launch)
@@ -134,7 +130,7 @@ struct P3Args {
     int c0;  // first kept column (mod Nx)
     int Wout;
     int ncols;
-    TwChain tw;  // reversed chain of the row plan
+    BlkTw tw;  // of the row length
     int* err;           // device status word (debug builds: bounds checks)
     long long u_elems;  // float2 elements of U from a.U on (all spectra of the launch)
 };
@@ -215,57 +211,39 @@ __device__ __forceinline__ bool p3_unit_ok(const P3Args& a, int pair, int sidx)
 #endif
 }
 
-template <int N, class FwdSeq, int TT_ = 0>
+// Radix order of a length's self-sorting chain (the tensor-core column pass).
+template <int N, class FwdSeq>
 struct Plan {
     using Fwd = FwdSeq;
     using Inv = Reverse<FwdSeq>;
     static_assert(SeqInfo<Fwd>::product == N, "radices must multiply to N");
     static constexpr int R0 = SeqInfo<Fwd>::first;   // first forward radix
     static constexpr int RL = SeqInfo<Fwd>::last;    // last forward radix
-    // threads per transform: one butterfly per thread in every stage by
-    // default (N / smallest radix, rounded up to whole warps); fewer threads
-    // own several butterflies in the stages with more butterflies
-    static constexpr int T = TT_ > 0 ? TT_ : ((N / SeqInfo<Fwd>::min_r) + 31) / 32 * 32;
-    // shared memory (complex elements) of one transform: the larger padded
-    // extent of the forward and the reversed chain, rounded up to an even
-    // count so that staging areas placed after it start on a 16-byte
-    // boundary (as cp.async of 16 bytes requires)
-    static constexpr int SMEM_ELEMS = ((ChainExtent<Fwd>::value > ChainExtent<Inv>::value
-                                            ? ChainExtent<Fwd>::value
-                                            : ChainExtent<Inv>::value) + 1) / 2 * 2;
-    static constexpr int SMEM_BYTES = 8 * SMEM_ELEMS;
-    static_assert(T <= 1024, "too many threads per transform");
-    using FwdChain = Chain<N, -1, 1, 0, T, Fwd>;
-    using InvChain = Chain<N, +1, 1, 0, T, Inv>;
-    // double-buffered chains: the inverse continues the forward's buffer
-    // alternation (it follows the forward's exchanges in the column pass)
-    static constexpr int NEX = SeqInfo<Fwd>::stages - 1;   // exchanges per chain
-    using FwdChainDB = Chain<N, -1, 1, 0, T, Fwd, true, 0>;
-    using InvChainDB = Chain<N, +1, 1, 0, T, Inv, true, NEX % 2>;
-    static constexpr int E0 = FwdChain::E;                    // forward first stage
-    static constexpr int EL = Chain<N, -1, N / RL, 0, T, Seq<RL>>::E;  // forward last stage
-    static constexpr int EI = InvChain::E;                    // inverse first stage (= EL)
-    static constexpr int EJ = Chain<N, +1, N / R0, 0, T, Seq<R0>>::E;  // inverse last stage
 };
 
 // Programmatic dependent launch.  The pass kernels are launched with the
 // programmatic-stream-serialization attribute and begin with pdl_begin():
-// the trigger lets the next kernel on the stream start launching once every
-// block of this grid has started (its blocks then wait in their own
-// pdl_begin), and the wait holds this grid until the previous grid on the
-// stream has completed with its memory visible -- so no pass touches global
-// memory before its predecessor is done, while the launch latency of each
-// pass overlaps the tail of the one before.  Without the attribute (or after
-// a non-kernel operation) the wait returns at once.  With LATE the block
-// does not trigger, so the next kernel launches only as this grid's blocks
-// exit: measured faster for the forward row pass at three resident blocks
-// per SM (the next pass's early blocks otherwise share its last wave's SMs),
-// a plan knob per pass.
+// the wait holds this grid until the previous grid on the stream has
+// completed with its memory visible, and the trigger after it lets the next
+// kernel on the stream start launching once every block of this grid has got
+// so far (its blocks then wait in their own pdl_begin) -- so no pass touches
+// its predecessor's results before they are there, everything older is
+// complete when a block starts, and the launch latency of each pass overlaps
+// the tail of the one before.  Without the attribute (or after a non-kernel
+// operation) the wait returns at once.  With LATE the block does not
+// trigger, so the next kernel launches only as this grid's blocks exit:
+// measured faster for the forward row pass at three resident blocks per SM
+// (the next pass's early blocks otherwise share its last wave's SMs), a plan
+// knob per pass.
+//
+// What the previous grid wrote (L, T, U) is read by plain loads or TMA, never
+// by __ldg: a non-coherent load may be moved above the wait, its data being
+// constant as far as the compiler knows.
 template <bool LATE = false>
 __device__ __forceinline__ void pdl_begin()
 {
-    if constexpr (!LATE) asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
     asm volatile("griddepcontrol.wait;\n" ::: "memory");
+    if constexpr (!LATE) asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
 }
 
 template <class... KArgs, class... Args>
@@ -285,542 +263,642 @@ inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, s
     return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
 }
 
-// P2's spectrum product on the forward column's last-stage outputs (thread
-// t, butterfly j = t + e T holds frequencies j + m N/RL).
-template <class P, int N, bool KREAL, bool STAGED>
-__device__ __forceinline__ void spectrum_product(float2 (&f)[P::EL][P::RL], int t, const void* kcol,
-                                                 const float* kst)
+
+// ---------------------------------------------------------------------------
+// A pass kernel's shape: geometry of the length, NT transforms per block (row
+// pairs or columns), TH threads (per group in the batched column pass),
+// minimum resident blocks per SM (register cap), late launch trigger.
+// ---------------------------------------------------------------------------
+template <class Ge_, int NT_, int TH_, int MINB_, bool LATE_>
+struct PassCfg {
+    using Ge = Ge_;
+    using La = Lay<Ge_>;
+    static constexpr int NT = NT_, TH = TH_, MINB = MINB_;
+    static constexpr bool LATE = LATE_;
+    static_assert(TH % 32 == 0 && TH <= 1024, "whole warps");
+    static constexpr int WORK = NT * La::ELEMS;          // float2 of one working set
+    static constexpr int SMEM = 8 * (Ge::W1 + WORK);     // w1, then the working set
+    static constexpr int U1 = Ge::N1 * NT;               // stage-1 butterflies
+    static constexpr int E1 = (U1 + TH - 1) / TH;
+    static constexpr int GROUPS = TH / 32 * Ge::GPW;     // sub-transforms in flight
+    static constexpr int UB = Ge::R0 * NT;               // sub-transforms
+    static constexpr int EB = (UB + GROUPS - 1) / GROUPS;
+    static constexpr int US = Ge::R0 * Ge::R1 * NT;      // stage-3 runs
+    static constexpr int ES = (US + TH - 1) / TH;
+};
+
+// shared memory of the FP32 passes (namespace scope, so that functions that
+// are not inlined address it as shared memory)
+extern __shared__ __align__(16) float2 lp_dsmem[];
+
+// ---------------------------------------------------------------------------
+// Row passes.  A transform packs two real rows, z = a + i b, so the half
+// spectra of a and b need each frequency k = m + R0 (k1 + R1 k2) together
+// with N - k.  That partner lies in sub-transform R0 - m (m = 0: in itself),
+// at k1' = R1 - 1 - k1, k2' = R2 - 1 - k2 (m = 0: k1' = (R1 - k1) mod R1, and
+// for k1 = 0 the run's own element (R2 - k2) mod R2).  Where a sub-transform
+// takes half a warp or less, a warp handles m and R0 - m side by side (RowSub)
+// and the partners are exchanged by shuffles, each lane handing over the
+// upper half of its run; else a sweep through shared memory combines them.
+// ---------------------------------------------------------------------------
+template <class C>
+struct RowSub {
+    using Ge = typename C::Ge;
+    static constexpr int R0 = Ge::R0, G = Ge::G;
+    static constexpr bool SHUFFLE = R0 == 1;
+    static constexpr int LANES = R0 == 1 ? G : 2 * G;             // lanes of a unit
+    static constexpr int PU = R0 == 1 ? 1 : R0 / 2 + R0 % 2;      // units of a transform: {m, R0 - m}, {0, R0 / 2}
+    static constexpr int UNITS = PU * C::NT;
+    static constexpr int FLIGHT = SHUFFLE ? C::TH / LANES : 1;
+    static constexpr int ROUNDS = (UNITS + FLIGHT - 1) / FLIGHT;
+    int tr, m, li, partner;  // transform, sub-transform, lane in the group, partner's lane in the warp
+    bool live, origin;       // origin: the run k1 = 0 of m = 0
+    __device__ __forceinline__ RowSub(int t, int round)
+    {
+        const int q = t / LANES + round * FLIGHT;
+        li = t % G;
+        tr = C::NT == 1 ? 0 : q / PU;
+        const int pu = q - tr * PU, half = R0 == 1 ? 0 : (t / G) & 1;
+        live = ROUNDS * FLIGHT == UNITS || q < UNITS;
+        bool self;
+        if (R0 == 1) {
+            m = 0;
+            self = true;
+        } else if (pu == 0) {
+            m = half ? R0 / 2 : 0;
+            if (R0 % 2 && half) live = false;  // odd R0: sub-transform 0 has the warp's half for itself
+            self = true;
+        } else {
+            m = half ? R0 - pu : pu;
+            self = false;
+        }
+        const int kp = m == 0 ? (li == 0 ? 0 : Ge::R1 - li) : Ge::R1 - 1 - li;
+        const int lane = t & 31;
+        partner = ((lane - li) ^ (self ? 0 : G)) + (li < Ge::R1 ? kp : li);
+        origin = m == 0 && li == 0;
+    }
+};
+
+// {2 X_a[c], 2 X_b[c]} of the packed transform's Z[c] and Z[N - c]
+__device__ __forceinline__ float4 split_rows(float2 zc, float2 zm)
 {
-    constexpr int RL = P::RL, NBL = N / RL;
+    float4 o;
+    o.x = zc.x + zm.x;       // 2 X_a = Z[c] + conj Z[N-c]
+    o.y = zc.y - zm.y;
+    o.z = zc.y + zm.y;       // 2 X_b = -i (Z[c] - conj Z[N-c])
+    o.w = -(zc.x - zm.x);
+    return o;
+}
+// Z[c] and Z[N - c] from the half spectra {A, B} of c
+__device__ __forceinline__ float2 join_lo(float4 q) { return make_float2(q.x - q.w, q.y + q.z); }
+__device__ __forceinline__ float2 join_hi(float4 q) { return make_float2(q.x + q.w, q.z - q.y); }
+
+// ---------------------------------------------------------------------------
+// P1: row R2C of two packed rows per transform, NT transforms per block.
+// ---------------------------------------------------------------------------
+struct RowInput {
+    const float *pa, *pb;
+    int wa, wb;  // columns to read of each row (0: none)
+    __device__ __forceinline__ RowInput(const P1Args& a, int pair)
+    {
+        const int ra = 2 * pair;
+        pa = a.L + (long long)ra * a.ldl;
+        pb = pa + a.ldl;
+        wa = pair < a.npairs && ra < a.H ? a.W : 0;
+        wb = pair < a.npairs && ra + 1 < a.H ? a.W : 0;
+    }
+    __device__ __forceinline__ float2 operator()(int col) const
+    {
+        return make_float2(col < wa ? pa[col] : 0.f, col < wb ? pb[col] : 0.f);
+    }
+};
+
+template <class C>
+__global__ void __launch_bounds__(C::TH, C::MINB) p1_rows(const __grid_constant__ P1Args a)
+{
+    pdl_begin<C::LATE>();
+    using Ge = typename C::Ge;
+    using La = typename C::La;
+    using RS = RowSub<C>;
+    constexpr int R0 = Ge::R0, R1 = Ge::R1, R2 = Ge::R2, N1 = Ge::N1, UR = R0 * R1;
+    const int pair0 = a.pair0 + blockIdx.x * C::NT;
+    for (int tr = 0; tr < C::NT; ++tr)
+        if (pair0 + tr < a.npairs && !p1_unit_ok(a, pair0 + tr)) return;  // (whole block: before any barrier)
+    const int t = threadIdx.x;
+    float2* work = lp_dsmem + Ge::W1;
+    if constexpr (R0 > 1) {
+        load_w1<Ge>(lp_dsmem, a.tw.w1, t, C::TH);
+#pragma unroll 1
+        for (int e = 0; e < C::E1; ++e) {
+            const int u = t + e * C::TH;
+            if (C::E1 * C::TH != C::U1 && u >= C::U1) break;
+            const int tr = C::NT == 1 ? 0 : u / N1;
+            const int j = u - tr * N1;
+            const RowInput in(a, pair0 + tr);
+            float2 v[R0];
 #pragma unroll
-    for (int e = 0; e < P::EL; ++e) {
-        const int j = t + e * P::T;
-        if (j >= NBL) continue;
+            for (int q = 0; q < R0; ++q) v[q] = in(j + q * N1);
+            Dft<R0, -1, float2>::run(v);
+            float2* w = work + tr * La::ELEMS + stage1_addr<Ge>(j);
 #pragma unroll
-        for (int m = 0; m < RL; ++m) {
-            const int u = j + m * NBL;
-            if constexpr (KREAL) {
-                const float k = STAGED ? kst[u] : __ldg(static_cast<const float*>(kcol) + u);
-                f[e][m] = cscale(f[e][m], k);
+            for (int m = 0; m < R0; ++m) w[m * La::S0] = v[m];
+        }
+        __syncthreads();
+    }
+    const long long ldq = a.ldT / 2;
+    float4* Tq = reinterpret_cast<float4*>(a.T);
+    if constexpr (RS::SHUFFLE) {
+#pragma unroll 1
+        for (int e = 0; e < RS::ROUNDS; ++e) {
+            const RS s(t, e);
+            float2* b = work + s.tr * La::ELEMS + s.m * La::S0;
+            if (s.live && s.li < R2) {
+                float2 x[R1];
+                if constexpr (R0 > 1) {
+#pragma unroll
+                    for (int l = 0; l < R1; ++l) x[l] = b[s.li + l * La::S1];
+                } else {
+                    const RowInput in(a, pair0 + s.tr);
+#pragma unroll
+                    for (int l = 0; l < R1; ++l) x[l] = in(s.li + l * R2);
+                }
+                stage2_fwd<Ge>(x, b, s.m, s.li, lp_dsmem, a.tw.w2);
+            }
+            __syncwarp();
+            float2 f[R2];
+            if (s.live && s.li < R1) {
+                load_run<Ge>(f, b, s.li);
+                Dft<R2, -1, float2>::run(f);
+            }
+            const int pair = pair0 + s.tr;
+            const bool store = s.live && s.li < R1 && pair < a.npairs;
+            const int u = s.m + R0 * s.li;
+            float4* dst = Tq + t_index4(u, pair, ldq);
+#pragma unroll
+            for (int k = 0; k <= R2 / 2; ++k) {
+                float2 zm;
+                constexpr int last = R2 - 1;
+                zm.x = __shfl_sync(0xffffffffu, f[last - k].x, s.partner);
+                zm.y = __shfl_sync(0xffffffffu, f[last - k].y, s.partner);
+                if (s.origin) zm = f[k == 0 ? 0 : R2 - k];
+                const int c = u + k * UR;
+                if (store && (k < R2 / 2 || c < a.ncols)) {
+                    const float4 o = split_rows(f[k], zm);
+                    if constexpr (UR % kTCB == 0) dst[k * (UR / kTCB) * (ldq * kTCB)] = o;
+                    else Tq[t_index4(c, pair, ldq)] = o;
+                }
+            }
+        }
+    } else {
+        const int li = t % Ge::G;
+#pragma unroll 1
+        for (int e = 0; e < C::EB; ++e) {
+            const int q = t / Ge::G + e * C::GROUPS;
+            const bool live = C::EB * C::GROUPS == C::UB || q < C::UB;
+            const int tr = C::NT == 1 ? 0 : q / R0;
+            const int m = q - tr * R0;
+            float2* b = work + tr * La::ELEMS + m * La::S0;
+            if (live && li < R2) {
+                float2 x[R1];
+#pragma unroll
+                for (int l = 0; l < R1; ++l) x[l] = b[li + l * La::S1];
+                stage2_fwd<Ge>(x, b, m, li, lp_dsmem, a.tw.w2);
+            }
+            __syncwarp();
+            if (live && li < R1) {
+                float2 f[R2];
+                load_run<Ge>(f, b, li);
+                Dft<R2, -1, float2>::run(f);
+                store_run<Ge>(f, b, li);
+            }
+        }
+        __syncthreads();
+        // The run u = m + R0 k1 holds the frequencies c = u + R0 R1 k2, its
+        // partners N - c are the run R0 R1 - u backwards, so both addresses
+        // are a base plus a constant.
+#pragma unroll 1
+        for (int e = 0; e < C::ES; ++e) {
+            const int v = t + e * C::TH;
+            if (C::ES * C::TH != C::US && v >= C::US) break;
+            const int tr = v % C::NT, u = v / C::NT;
+            const int pair = pair0 + tr;
+            if (pair >= a.npairs) continue;
+            const int up = u == 0 ? 0 : UR - u;
+            const float2* z = work + tr * La::ELEMS + (u % R0) * La::S0 + (u / R0) * La::S1;
+            const float2* zp = work + tr * La::ELEMS + (up % R0) * La::S0 + (up / R0) * La::S1;
+            float4* dst = Tq + t_index4(u, pair, ldq);
+            auto put = [&](int k, float2 zc, float2 zm) {
+                if constexpr (UR % kTCB == 0) dst[k * (UR / kTCB) * (ldq * kTCB)] = split_rows(zc, zm);
+                else Tq[t_index4(u + k * UR, pair, ldq)] = split_rows(zc, zm);
+            };
+            if (La::VEC && u > 0) {
+                // R2 even: k2 < R2 / 2, two at a time
+#pragma unroll
+                for (int k = 0; k < R2 / 2; k += 2) {
+                    const float4 c2 = *reinterpret_cast<const float4*>(z + k);
+                    const float4 p2 = *reinterpret_cast<const float4*>(zp + (R2 - 2 - k));
+                    put(k, make_float2(c2.x, c2.y), make_float2(p2.z, p2.w));
+                    if (k + 1 < R2 / 2) put(k + 1, make_float2(c2.z, c2.w), make_float2(p2.x, p2.y));
+                }
             } else {
-                const float2 k = STAGED ? reinterpret_cast<const float2*>(kst)[u]
-                                        : __ldg(static_cast<const float2*>(kcol) + u);
-                f[e][m] = cmul(f[e][m], k);
+#pragma unroll
+                for (int k = 0; k <= R2 / 2; ++k)
+                    if (k < R2 / 2 || u + k * UR < a.ncols)
+                        put(k, z[k], zp[u > 0 ? R2 - 1 - k : k == 0 ? 0 : R2 - k]);
             }
         }
     }
-}
-
-// P2's inverse-output store: rows of the crop window of column Uc.
-template <class P, int N>
-__device__ __forceinline__ void store_column(const float2 (&o)[P::EJ][P::R0], int t, float2* Uc,
-                                             int r0, int Hout, int HoutPad)
-{
-    constexpr int R0 = P::R0, NB0 = N / R0;
-#pragma unroll
-    for (int e = 0; e < P::EJ; ++e) {
-        const int j = t + e * P::T;
-        if (j >= NB0) continue;
-#pragma unroll
-        for (int m = 0; m < R0; ++m) {
-            int rr = j + m * NB0 - r0;
-            if (rr < 0) rr += N;
-            if (rr < Hout) Uc[u_row(rr)] = o[e][m];
-        }
-    }
-    if (HoutPad != Hout && t == 0) Uc[u_row(Hout)] = make_float2(0.f, 0.f);
-}
-
-// P1's split of the packed transform Z (in shared memory, natural order)
-// into the half spectra of rows a and b: {2 X_a[c], 2 X_b[c]} -> T[c][pair].
-template <int N, int T>
-__device__ __forceinline__ void unpack_rows(const float2* sm, int t, int ncols, float4* Tq, long long ldq,
-                                            int pair)
-{
-    for (int c = t; c < ncols; c += T) {
-        const int cm = (c == 0) ? 0 : N - c;
-        const float2 zc = sm[c], zm = sm[cm];
-        float4 o;
-        o.x = zc.x + zm.x;       // 2 X_a = Z[c] + conj Z[N-c]
-        o.y = zc.y - zm.y;
-        o.z = zc.y + zm.y;       // 2 X_b = -i (Z[c] - conj Z[N-c])
-        o.w = -(zc.x - zm.x);
-        Tq[t_index4(c, pair, ldq)] = o;
-    }
-}
-
-// P1/P3 hand the last stage's outputs to shared memory in natural order.
-template <class P, int N, int E, int R>
-__device__ __forceinline__ void to_smem_natural(const float2 (&z)[E][R], int t, float2* sm)
-{
-    constexpr int NBL = N / R;
-    __syncthreads();
-#pragma unroll
-    for (int e = 0; e < E; ++e) {
-        const int j = t + e * P::T;
-        if (j >= NBL) continue;
-#pragma unroll
-        for (int m = 0; m < R; ++m) sm[j + m * NBL] = z[e][m];
-    }
-    __syncthreads();
-}
-
-// P3's first-stage input: Z[k] = A[k] + i B[k] from the stored half spectra
-// q = {A, B} of k (k <= N/2) or of N-k (Hermitian extension).
-__device__ __forceinline__ float2 packed_inverse_input(float4 q, bool lo, bool vb)
-{
-    if (!vb) {
-        q.z = 0.f;
-        q.w = 0.f;
-    }
-    return lo ? make_float2(q.x - q.w, q.y + q.z) : make_float2(q.x + q.w, q.z - q.y);
-}
-
-// P3's final store: real part -> row a, imaginary part -> row b, crop columns.
-template <class P, int N>
-__device__ __forceinline__ void store_rows(const float2 (&o)[P::EJ][P::R0], int t, float* oa, float* ob,
-                                           bool vb, int c0, int Wout)
-{
-    constexpr int RJ = P::R0, NBJ = N / RJ;
-#pragma unroll
-    for (int e = 0; e < P::EJ; ++e) {
-        const int j = t + e * P::T;
-        if (j >= NBJ) continue;
-#pragma unroll
-        for (int m = 0; m < RJ; ++m) {
-            int cc = j + m * NBJ - c0;
-            if (cc < 0) cc += N;
-            if (cc < Wout) {
-                oa[cc] = o[e][m].x;
-                if (vb) ob[cc] = o[e][m].y;
-            }
-        }
-    }
-}
-
-// ---------------------------------------------------------------------------
-// P1: row R2C of two packed rows per transform, F transforms per block.
-// ---------------------------------------------------------------------------
-template <class P, int N, int F, bool LATE = false>
-__global__ void __launch_bounds__(P::T * F) p1_rows(const P1Args a)
-{
-    pdl_begin<LATE>();
-    extern __shared__ float2 smem2[];
-    constexpr int T = P::T;
-    constexpr int R0 = P::R0, NB0 = N / R0;
-    const int f = threadIdx.x / T;
-    const int t = threadIdx.x - f * T;
-    float2* sm = smem2 + f * P::SMEM_ELEMS;
-    const int pair = a.pair0 + blockIdx.x * F + f;
-    const int ra = 2 * pair, rb = ra + 1;
-    const bool live = pair < a.npairs && p1_unit_ok(a, pair);
-    const bool va = live && ra < a.H, vb = live && rb < a.H;
-    const float* La = a.L + (long long)ra * a.ldl;
-    const float* Lb = a.L + (long long)rb * a.ldl;
-
-    float2 v[P::E0][R0];
-#pragma unroll
-    for (int e = 0; e < P::E0; ++e) {
-        const int j = t + e * T;
-        if (j >= NB0) continue;
-#pragma unroll
-        for (int m = 0; m < R0; ++m) {
-            const int col = j + m * NB0;
-            const bool in = col < a.W;
-            v[e][m].x = (in && va) ? __ldg(La + col) : 0.f;
-            v[e][m].y = (in && vb) ? __ldg(Lb + col) : 0.f;
-        }
-    }
-    P::FwdChain::run(v, t, sm, a.tw, [&](float2(&z)[P::EL][P::RL], int tt) {
-        to_smem_natural<P, N>(z, tt, sm);
-        if (live) unpack_rows<N, T>(sm, tt, a.ncols, reinterpret_cast<float4*>(a.T), a.ldT / 2, pair);
-    });
 }
 
 // ---------------------------------------------------------------------------
 // P2: per column forward FFT, spectrum product, inverse FFT, row crop.
 // ---------------------------------------------------------------------------
-// One spectrum of the batched column pass: the forward column is parked in
-// F (natural order); product with spectrum s, inverse, store.  Not inlined:
-// as a loop body it would let the compiler keep the whole inverse's
-// constants and indices live across iterations.
-template <class P, int N, bool KREAL>
-__device__ __noinline__ void p2_spectrum_pass(const P2Args& a, int c, int s, const float2* F, float2* sm)
+// Stage 1 of NT columns from T (rows >= H are the zero padding) into sm.
+// Consecutive lanes take the block's columns, then rows, so that the pieces
+// of a column block of T are read together.
+template <class C>
+__device__ __forceinline__ void column_stage1(const float2* T, long long ldT, int H, int c0, int ncols,
+                                              float2* sm, int t, int th)
 {
-    constexpr int RL = P::RL, NBL = N / RL;
-    const int t = threadIdx.x;
-    float2 g[P::EL][RL];
+    using Ge = typename C::Ge;
+    using La = typename C::La;
+    constexpr int R0 = Ge::R0, N1 = Ge::N1, NT = C::NT;
+#pragma unroll 1
+    for (int u = t; u < C::U1; u += th) {
+        const int cl = u % NT, j = u / NT;
+        const int c = c0 + cl;
+        const float2* col = t_column(T, ldT, c);
+        float2 v[R0];
 #pragma unroll
-    for (int e = 0; e < P::EL; ++e) {
-        const int j = t + e * P::T;
-        if (j >= NBL) continue;
+        for (int q = 0; q < R0; ++q) {
+            const int row = j + q * N1;
+            const long long off = (N1 % 2 == 0) ? t_row(j) + q * t_row_step<N1>() : t_row(row);
+            v[q] = (row < H && (NT == 1 || c < ncols)) ? col[off] : make_float2(0.f, 0.f);
+        }
+        Dft<R0, -1, float2>::run(v);
+        float2* w = sm + cl * La::ELEMS + stage1_addr<Ge>(j);
 #pragma unroll
-        for (int m = 0; m < RL; ++m) g[e][m] = F[j + m * NBL];
+        for (int m = 0; m < R0; ++m) w[m * La::S0] = v[m];
     }
-    const long long kw = KREAL ? 1 : 2;
-    spectrum_product<P, N, KREAL, false>(g, t, static_cast<const float*>(a.K[s]) + (long long)c * a.ldK * kw,
-                                         nullptr);
-    float2* Uc = u_column(a.U + (long long)s * a.specU, a.ldU, c);
-    P::InvChain::run(g, t, sm, a.twi, [&](float2(&o)[P::EJ][P::R0], int tt) {
-        store_column<P, N>(o, tt, Uc, a.r0, a.Hout, a.HoutPad);
-    });
 }
 
-__device__ __forceinline__ void cp_async4(void* smem, const void* gmem);
-__device__ __forceinline__ void cp_async16(void* smem, const void* gmem);
-// bulk prefetch of [p, p + bytes) into L2 (p 16-byte aligned, bytes a
-// multiple of 16)
-__device__ __forceinline__ void l2_prefetch(const void* p, unsigned bytes)
+// Inverse stage 1 of NT columns: rows of the crop window to U.
+template <class C>
+__device__ __forceinline__ void column_out(const P2Args& a, float2* U, int c0, const float2* sm, int t)
 {
-    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;\n" ::"l"(p), "r"(bytes) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit();
-__device__ __forceinline__ void cp_async_wait_all();
-
-// KST (one spectrum): the block's spectrum column is copied into shared
-// memory (after the exchange buffer) with cp.async at the start, so its
-// load latency overlaps the forward transform instead of stalling the
-// product.
-// PARKG (several spectra): the forward column is parked in global memory
-// (a.park) instead of shared memory, for lengths whose exchange buffer and
-// parked column do not fit shared memory together.
-template <class P, int N, bool KREAL, bool MULTI, int MINB = 1, bool DB = false, bool KST = false,
-          bool PARKG = false, bool LATE = false>
-__global__ void __launch_bounds__(P::T, MINB) p2_cols(const __grid_constant__ P2Args a)
-{
-    pdl_begin<LATE>();
-    static_assert(!(DB && MULTI), "the batched column pass is single-buffered");
-    static_assert(!(KST && MULTI), "spectrum staging is for one spectrum");
-    using Fwd = typename std::conditional<DB, typename P::FwdChainDB, typename P::FwdChain>::type;
-    using Inv = typename std::conditional<DB, typename P::InvChainDB, typename P::InvChain>::type;
-    extern __shared__ float2 smem2[];
-    constexpr int R0 = P::R0, NB0 = N / R0;
-    constexpr int RL = P::RL, NBL = N / RL;
-    float2* sm = smem2;
-    const int c = blockIdx.x;
-    const int t = threadIdx.x;
-    constexpr int KW = KREAL ? 1 : 2;  // floats per spectrum value
-    if (!p2_column_ok(a, c, N, KW)) return;  // (whole block: before any barrier)
-    const float2* col = t_column(a.T, a.ldT, c);
-    float* kst = reinterpret_cast<float*>(smem2 + (DB ? 2 : 1) * P::SMEM_ELEMS);
-    if constexpr (!MULTI && !KST) {
-        // the spectrum column is needed after the forward transform: one bulk
-        // prefetch into L2 now (no shared memory, no barrier) shortens its
-        // load latency at the product
-        if (t == 0) l2_prefetch(static_cast<const float*>(a.K[0]) + (long long)c * a.ldK * KW, 16u * ((N * KW + 3) / 4));
-        // the T columns of a block that starts about one wave of resident
-        // blocks later (a.ahead columns on), so that its first loads hit L2;
-        // the even column of each pair prefetches the pair's block
-        const int cn = c + a.ahead;
-        if (t == 32 && a.ahead > 0 && (cn & 1) == 0 && cn < a.ncols)
-            l2_prefetch(t_column(a.T, a.ldT, cn), (unsigned)(16 * a.ldT));
-    }
-    if constexpr (KST) {
-        // ldK is a multiple of 32, so the column start is 16-byte aligned
-        const float* src = static_cast<const float*>(a.K[0]) + (long long)c * a.ldK * KW;
-        for (int q = t; q < (N * KW + 3) / 4; q += P::T) cp_async16(kst + 4 * q, src + 4 * q);
-        cp_async_commit();
-    }
-
-    float2 v[P::E0][R0];
+    using Ge = typename C::Ge;
+    using La = typename C::La;
+    constexpr int R0 = Ge::R0, N1 = Ge::N1, NT = C::NT;
+#pragma unroll 1
+    for (int u = t; u < C::U1; u += C::TH) {
+        const int cl = u % NT, j = u / NT;
+        const int c = c0 + cl;
+        const float2* w = sm + cl * La::ELEMS + stage1_addr<Ge>(j);
+        float2 v[R0];
 #pragma unroll
-    for (int e = 0; e < P::E0; ++e) {
-        const int j = t + e * P::T;
-        if (j >= NB0) continue;
+        for (int m = 0; m < R0; ++m) v[m] = w[m * La::S0];
+        Dft<R0, 1, float2>::run(v);
+        if (NT > 1 && c >= a.ncols) continue;
+        float2* Uc = u_column(U, a.ldU, c);
 #pragma unroll
-        for (int m = 0; m < R0; ++m) {
-            const int row = j + m * NB0;
-            const long long off = (NB0 % 2 == 0) ? t_row(j) + m * t_row_step<NB0>() : t_row(row);
-            v[e][m] = row < a.H ? __ldg(col + off) : make_float2(0.f, 0.f);
+        for (int q = 0; q < R0; ++q) {
+            int rr = j + q * N1 - a.r0;
+            if (rr < 0) rr += Ge::N;
+            if (rr < a.Hout) Uc[u_row(rr)] = v[q];
         }
     }
-    Fwd::run(v, t, sm, a.twf, [&](float2(&fz)[P::EL][RL], int tt) {
-        if constexpr (MULTI) {
-            // parked forward column, in shared memory after the exchange
-            // buffer, or in global memory (L2-resident while the block runs);
-            // each thread reads back only the elements it wrote, so no
-            // barrier orders the park
-            float2* F = PARKG ? a.park + (size_t)c * N : smem2 + P::SMEM_ELEMS;
+}
+
+// the zero row that completes the last row pair when Hout is odd
+template <class C>
+__device__ __forceinline__ void column_pad(const P2Args& a, float2* U, int c0, int t)
+{
+    if (a.HoutPad != a.Hout && t < C::NT && c0 + t < a.ncols)
+        u_column(U, a.ldU, c0 + t)[u_row(a.Hout)] = make_float2(0.f, 0.f);
+}
+
+// Spectrum values of frequencies (m, k1, 0..R2-1) of one column (stored in
+// the order Geo::kpos).
+template <class Ge, bool KREAL>
+__device__ __forceinline__ void load_spectrum(typename std::conditional<KREAL, float, float2>::type (&k)[Ge::R2],
+                                              const void* kcol, int m, int k1)
+{
+    constexpr int R2 = Ge::R2, VK = Ge::VK;
+    if constexpr (KREAL) {
+        const float* p = static_cast<const float*>(kcol) + Ge::kpos(m, k1, 0);
 #pragma unroll
-            for (int e = 0; e < P::EL; ++e) {
-                const int j = tt + e * P::T;
-                if (j >= NBL) continue;
-#pragma unroll
-                for (int m = 0; m < RL; ++m) F[j + m * NBL] = fz[e][m];
-            }
-            for (int s = 0; s < a.nspec; ++s) p2_spectrum_pass<P, N, KREAL>(a, c, s, F, sm);
-        } else {
-            if constexpr (KST) {
-                cp_async_wait_all();
-                __syncthreads();  // every thread's share of the column has landed
-            }
-            spectrum_product<P, N, KREAL, KST>(fz, tt, static_cast<const float*>(a.K[0]) + (long long)c * a.ldK * KW,
-                                               kst);
-            float2* Uc = u_column(a.U, a.ldU, c);
-            Inv::run(fz, tt, sm, a.twi, [&](float2(&o)[P::EJ][R0], int t2) {
-                store_column<P, N>(o, t2, Uc, a.r0, a.Hout, a.HoutPad);
-            }, P::SMEM_ELEMS);
-        }
-    }, P::SMEM_ELEMS);
-}
-
-// ---------------------------------------------------------------------------
-// P3: row C2R of two packed rows per transform, F transforms per block,
-// blockIdx.y selects the spectrum.
-// ---------------------------------------------------------------------------
-template <class P, int N, int F>
-__global__ void __launch_bounds__(P::T * F) p3_rows(const P3Args a)
-{
-    pdl_begin();
-    extern __shared__ float2 smem2[];
-    constexpr int T = P::T;
-    constexpr int RI = P::RL, NBI = N / RI;
-    const int f = threadIdx.x / T;
-    const int t = threadIdx.x - f * T;
-    float2* sm = smem2 + f * P::SMEM_ELEMS;
-    const int pair = a.pair0 + blockIdx.x * F + f;
-    const int sidx = blockIdx.y;
-    const int ra = 2 * pair, rb = ra + 1;
-    const float4* Uq = reinterpret_cast<const float4*>(a.U + (long long)sidx * a.specU);
-    const long long ldq = a.ldU / 2;
-    const bool live = pair < a.npairs && p3_unit_ok(a, pair, sidx);
-    const bool vb = rb < a.Hout;
-
-    float2 v[P::EI][RI];
-#pragma unroll
-    for (int e = 0; e < P::EI; ++e) {
-        const int j = t + e * T;
-        if (j >= NBI) continue;
-#pragma unroll
-        for (int m = 0; m < RI; ++m) {
-            const int k = j + m * NBI;
-            const bool lo = k < a.ncols;
-            float4 q = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (live) q = __ldg(Uq + u_index4(lo ? k : N - k, pair, ldq));
-            v[e][m] = packed_inverse_input(q, lo, vb);
-        }
-    }
-    P::InvChain::run(v, t, sm, a.tw, [&](float2(&o)[P::EJ][P::R0], int tt) {
-        if (live) {
-            float* oa = a.out[sidx] + (long long)ra * a.ldo;
-            store_rows<P, N>(o, tt, oa, oa + a.ldo, vb, a.c0, a.Wout);
-        }
-    });
-}
-
-// ---------------------------------------------------------------------------
-// Prefetching variants.  Each block handles UPB work units (u, u + gridDim.x,
-// ...); while it transforms one unit, the input of the next one is copied
-// into a shared-memory staging area with cp.async (16-byte pieces where
-// aligned), so global-memory latency overlaps the butterflies instead of
-// stalling them.  cp.async.wait_group is a hardware wait: no spin loop is
-// involved.  Units are unrolled at compile time: a loop back-edge makes the
-// compiler keep about 70 more registers live per thread.
-// ---------------------------------------------------------------------------
-__device__ __forceinline__ void cp_async16(void* smem, const void* gmem)
-{
-    const unsigned s = (unsigned)__cvta_generic_to_shared(smem);
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(s), "l"(gmem) : "memory");
-}
-__device__ __forceinline__ void cp_async4(void* smem, const void* gmem)
-{
-    const unsigned s = (unsigned)__cvta_generic_to_shared(smem);
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(s), "l"(gmem) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
-__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;\n" ::: "memory"); }
-
-// staging bytes of the prefetching kernels (host and device agree on these)
-__host__ __device__ constexpr long long p1_stage_bytes(int Wst) { return 8ll * Wst; }
-__host__ __device__ constexpr long long p2_stage_bytes(long long ldT, long long ldK, bool kreal, bool kstage)
-{
-    return 8ll * ldT + (kstage ? (kreal ? 4ll : 8ll) * ldK : 0ll);
-}
-__host__ __device__ constexpr long long p3_stage_bytes(int ncols) { return 16ll * ncols; }
-
-template <class P, int N, int UPB, int MINB, bool DB = false, bool LATE = false>
-__global__ void __launch_bounds__(P::T, MINB) p1_rows_pf(const P1Args a)
-{
-    pdl_begin<LATE>();
-    extern __shared__ float2 smem2[];
-    constexpr int T = P::T;
-    constexpr int R0 = P::R0, NB0 = N / R0;
-    constexpr int NBUF = DB ? 2 : 1;
-    using Fwd = typename std::conditional<DB, typename P::FwdChainDB, typename P::FwdChain>::type;
-    float2* sm = smem2;
-    float* st = reinterpret_cast<float*>(smem2 + NBUF * P::SMEM_ELEMS);  // rows a, b: 2 x Wst floats
-    const int Wst = a.Wst;
-
-    auto prefetch = [&](int pair) {
-        if (pair >= a.npairs || !p1_unit_ok(a, pair)) return;
-        const int t = threadIdx.x;
-        for (int r = 0; r < 2; ++r) {
-            const int row = 2 * pair + r;
-            if (row >= a.H) continue;
-            const float* src = a.L + (long long)row * a.ldl;
-            float* dst = st + r * Wst;
-            if (a.vec16) {
-                for (int q = t; q < (a.W >> 2); q += T) cp_async16(dst + 4 * q, src + 4 * q);
+        for (int i = 0; i < R2; i += VK) {
+            const float* q = p + i * Ge::R1;
+            if constexpr (VK == 4) {
+                const float4 x = __ldg(reinterpret_cast<const float4*>(q));
+                k[i] = x.x;
+                k[i + 1] = x.y;
+                k[i + 2] = x.z;
+                k[i + 3] = x.w;
+            } else if constexpr (VK == 2) {
+                const float2 x = __ldg(reinterpret_cast<const float2*>(q));
+                k[i] = x.x;
+                k[i + 1] = x.y;
             } else {
-                for (int i = t; i < a.W; i += T) cp_async4(dst + i, src + i);
+                k[i] = __ldg(q);
             }
         }
-        cp_async_commit();
-    };
-    auto unit = [&](int pair) {
-        cp_async_wait_all();
-        __syncthreads();
-        const int t = threadIdx.x;
-        const bool vb = 2 * pair + 1 < a.H;
-        float2 v[P::E0][R0];
+    } else {
+        const float2* p = static_cast<const float2*>(kcol) + Ge::kpos(m, k1, 0);
 #pragma unroll
-        for (int e = 0; e < P::E0; ++e) {
-            const int j = t + e * T;
-            if (j >= NB0) continue;
+        for (int i = 0; i < R2; i += VK) {
+            const float2* q = p + i * Ge::R1;
+            if constexpr (VK >= 2) {
 #pragma unroll
-            for (int m = 0; m < R0; ++m) {
-                const int col = j + m * NB0;
-                const bool in = col < a.W;
-                v[e][m].x = in ? st[col] : 0.f;
-                v[e][m].y = (in && vb) ? st[Wst + col] : 0.f;
+                for (int h = 0; h < VK; h += 2) {
+                    const float4 x = __ldg(reinterpret_cast<const float4*>(q + h));
+                    k[i + h] = make_float2(x.x, x.y);
+                    k[i + h + 1] = make_float2(x.z, x.w);
+                }
+            } else {
+                k[i] = __ldg(q);
             }
         }
-        __syncthreads();  // staging consumed
-        prefetch(pair + gridDim.x);
-        Fwd::run(v, t, sm, a.tw, [&](float2(&z)[P::EL][P::RL], int tt) {
-            to_smem_natural<P, N>(z, tt, sm);
-            unpack_rows<N, T>(sm, tt, a.ncols, reinterpret_cast<float4*>(a.T), a.ldT / 2, pair);
-        }, P::SMEM_ELEMS);
-    };
-    prefetch(a.pair0 + blockIdx.x);
-    sfor<0, UPB>([&](auto I) {
-        const int pair = a.pair0 + blockIdx.x + decltype(I)::value * gridDim.x;
-        if (pair < a.npairs && p1_unit_ok(a, pair)) unit(pair);
-    });
+    }
 }
 
-// single spectrum; T column staged, K^ column staged when KSTAGE (else read
-// directly at the product)
-template <class P, int N, bool KREAL, int UPB, int MINB, bool KSTAGE, bool DB = false, bool LATE = false>
-__global__ void __launch_bounds__(P::T, MINB) p2_cols_pf(const P2Args a)
+template <bool KREAL, int R>
+__device__ __forceinline__ void spectrum_product(float2 (&f)[R],
+                                                 const typename std::conditional<KREAL, float, float2>::type (&k)[R])
 {
-    pdl_begin<LATE>();
-    extern __shared__ float2 smem2[];
-    constexpr int T = P::T;
-    constexpr int R0 = P::R0, NB0 = N / R0;
-    constexpr int RL = P::RL;
-    constexpr int KW = KREAL ? 1 : 2;                    // floats per K^ element
-    constexpr int NBUF = DB ? 2 : 1;
-    using Fwd = typename std::conditional<DB, typename P::FwdChainDB, typename P::FwdChain>::type;
-    using Inv = typename std::conditional<DB, typename P::InvChainDB, typename P::InvChain>::type;
-    float2* sm = smem2;
-    float2* tst = smem2 + NBUF * P::SMEM_ELEMS;          // ldT complex
-    float* kst = reinterpret_cast<float*>(tst + a.ldT);  // ldK floats or complex
-
-    auto prefetch_t = [&](int c) {
-        if (c >= a.ncols || !p2_column_ok(a, c, N, KW)) return;
-        const float4* src = reinterpret_cast<const float4*>(a.T);
-        const long long ldq = a.ldT >> 1;
-        for (int q = threadIdx.x; q < (int)ldq; q += T) cp_async16(tst + 2 * q, src + t_index4(c, q, ldq));
-        cp_async_commit();
-    };
-    auto prefetch_k = [&](int c) {
-        if constexpr (!KSTAGE) return;
-        if (c >= a.ncols || !p2_column_ok(a, c, N, KW)) return;
-        const float* src = static_cast<const float*>(a.K[0]) + (long long)c * a.ldK * KW;
-        for (int q = threadIdx.x; q < (int)((a.ldK * KW) >> 2); q += T) cp_async16(kst + 4 * q, src + 4 * q);
-        cp_async_commit();
-    };
-
-    auto unit = [&](int c) {
-        cp_async_wait_all();
-        __syncthreads();
-        const int t = threadIdx.x;
-        float2 v[P::E0][R0];
 #pragma unroll
-        for (int e = 0; e < P::E0; ++e) {
-            const int j = t + e * T;
-            if (j >= NB0) continue;
-#pragma unroll
-            for (int m = 0; m < R0; ++m) {
-                const int row = j + m * NB0;
-                v[e][m] = row < a.H ? tst[row] : make_float2(0.f, 0.f);
-            }
-        }
-        __syncthreads();
-        prefetch_t(c + gridDim.x);
-        Fwd::run(v, t, sm, a.twf, [&](float2(&fz)[P::EL][RL], int tt) {
-            spectrum_product<P, N, KREAL, KSTAGE>(
-                fz, tt, static_cast<const float*>(a.K[0]) + (long long)c * a.ldK * KW, kst);
-            if constexpr (KSTAGE) {
-                __syncthreads();  // K^ staging consumed
-                prefetch_k(c + gridDim.x);
-            }
-            float2* Uc = u_column(a.U, a.ldU, c);
-            Inv::run(fz, tt, sm, a.twi, [&](float2(&o)[P::EJ][R0], int t2) {
-                store_column<P, N>(o, t2, Uc, a.r0, a.Hout, a.HoutPad);
-            }, P::SMEM_ELEMS);
-        }, P::SMEM_ELEMS);
-    };
-    prefetch_t(blockIdx.x);
-    prefetch_k(blockIdx.x);
-    sfor<0, UPB>([&](auto I) {
-        const int c = blockIdx.x + decltype(I)::value * gridDim.x;
-        if (c < a.ncols && p2_column_ok(a, c, N, KW)) unit(c);
-    });
+    for (int i = 0; i < R; ++i) {
+        if constexpr (KREAL) f[i] = cscale(f[i], k[i]);
+        else f[i] = cmul(f[i], k[i]);
+    }
 }
 
-template <class P, int N, int UPB, int MINB, bool DB = false>
-__global__ void __launch_bounds__(P::T, MINB) p3_rows_pf(const P3Args a)
+// Where R0 = 1 a column is one sub-transform: rows li + l R2 of T, read by
+// stage 2 itself.
+template <class Ge>
+__device__ __forceinline__ void column_direct(float2 (&x)[Ge::R1], const float2* T, long long ldT, int H, int c,
+                                              int li)
 {
-    pdl_begin();
-    extern __shared__ float2 smem2[];
-    constexpr int T = P::T;
-    constexpr int RI = P::RL, NBI = N / RI;
-    constexpr int NBUF = DB ? 2 : 1;
-    using Inv = typename std::conditional<DB, typename P::InvChainDB, typename P::InvChain>::type;
-    float2* sm = smem2;
-    float4* ust = reinterpret_cast<float4*>(smem2 + NBUF * P::SMEM_ELEMS);  // ncols x {A, B}
-    const int sidx = blockIdx.y;
-    const float4* Uq = reinterpret_cast<const float4*>(a.U + (long long)sidx * a.specU);
-    const long long ldq = a.ldU / 2;
+    const float2* col = t_column(T, ldT, c);
+#pragma unroll
+    for (int l = 0; l < Ge::R1; ++l) {
+        const int row = li + l * Ge::R2;
+        x[l] = row < H ? col[t_row(row)] : make_float2(0.f, 0.f);
+    }
+}
+template <class Ge>
+__device__ __forceinline__ void column_direct_out(const float2 (&x)[Ge::R1], const P2Args& a, float2* U, int c, int li)
+{
+    float2* Uc = u_column(U, a.ldU, c);
+#pragma unroll
+    for (int l = 0; l < Ge::R1; ++l) {
+        int rr = li + l * Ge::R2 - a.r0;
+        if (rr < 0) rr += Ge::N;
+        if (rr < a.Hout) Uc[u_row(rr)] = x[l];
+    }
+}
 
-    auto prefetch = [&](int pair) {
-        if (pair >= a.npairs || !p3_unit_ok(a, pair, sidx)) return;
-        for (int k = threadIdx.x; k < a.ncols; k += T) cp_async16(ust + k, Uq + u_index4(k, pair, ldq));
-        cp_async_commit();
-    };
-
-    auto unit = [&](int pair) {
-        cp_async_wait_all();
+// One spectrum.
+template <class C, bool KREAL>
+__global__ void __launch_bounds__(C::TH, C::MINB) p2_cols(const __grid_constant__ P2Args a)
+{
+    pdl_begin<C::LATE>();
+    using Ge = typename C::Ge;
+    using La = typename C::La;
+    constexpr int R0 = Ge::R0, R1 = Ge::R1, R2 = Ge::R2, NT = C::NT;
+    const int c0 = blockIdx.x * NT;
+    const int t = threadIdx.x;
+    float2* work = lp_dsmem + Ge::W1;
+    for (int cl = 0; cl < NT; ++cl)
+        if (c0 + cl < a.ncols && !p2_column_ok(a, c0 + cl, Ge::N, KREAL ? 1 : 2)) return;
+    if constexpr (R0 > 1) {
+        load_w1<Ge>(lp_dsmem, a.tw.w1, t, C::TH);
+        column_stage1<C>(a.T, a.ldT, a.H, c0, a.ncols, work, t, C::TH);
         __syncthreads();
-        const int t = threadIdx.x;
-        const int ra = 2 * pair, rb = ra + 1;
-        const bool vb = rb < a.Hout;
-        float2 v[P::EI][RI];
+    }
+    const int li = t % Ge::G;
+#pragma unroll 1
+    for (int e = 0; e < C::EB; ++e) {
+        const int q = t / Ge::G + e * C::GROUPS;
+        const int cl = q % NT, m = q / NT;
+        const int c = c0 + cl;
+        const bool live = (C::EB * C::GROUPS == C::UB || q < C::UB) && (NT == 1 || c < a.ncols);
+        float2* b = work + cl * La::ELEMS + m * La::S0;
+        if (live && li < R2) {
+            float2 x[R1];
+            if constexpr (R0 > 1) {
 #pragma unroll
-        for (int e = 0; e < P::EI; ++e) {
-            const int j = t + e * T;
-            if (j >= NBI) continue;
+                for (int l = 0; l < R1; ++l) x[l] = b[li + l * La::S1];
+            } else {
+                column_direct<Ge>(x, a.T, a.ldT, a.H, c, li);
+            }
+            stage2_fwd<Ge>(x, b, m, li, lp_dsmem, a.tw.w2);
+        }
+        typename std::conditional<KREAL, float, float2>::type k[R2];
+        if (live && li < R1)
+            load_spectrum<Ge, KREAL>(k, static_cast<const float*>(a.K[0]) + (long long)c * a.ldK * (KREAL ? 1 : 2), m, li);
+        __syncwarp();
+        if (live && li < R1) {
+            float2 f[R2];
+            load_run<Ge>(f, b, li);
+            Dft<R2, -1, float2>::run(f);
+            spectrum_product<KREAL>(f, k);
+            Dft<R2, 1, float2>::run(f);
+            store_run<Ge>(f, b, li);
+        }
+        __syncwarp();
+        if (live && li < R2) {
+            float2 x[R1];
+            stage2_inv<Ge>(x, b, m, li, lp_dsmem, a.tw.w2);
+            if constexpr (R0 > 1) {
 #pragma unroll
-            for (int m = 0; m < RI; ++m) {
-                const int k = j + m * NBI;
-                const bool lo = k < a.ncols;
-                v[e][m] = packed_inverse_input(ust[lo ? k : N - k], lo, vb);
+                for (int l = 0; l < R1; ++l) b[li + l * La::S1] = x[l];
+            } else {
+                column_direct_out<Ge>(x, a, a.U, c, li);
             }
         }
+    }
+    if constexpr (R0 > 1) {
         __syncthreads();
-        prefetch(pair + gridDim.x);
-        Inv::run(v, t, sm, a.tw, [&](float2(&o)[P::EJ][P::R0], int tt) {
-            float* oa = a.out[sidx] + (long long)ra * a.ldo;
-            store_rows<P, N>(o, tt, oa, oa + a.ldo, vb, a.c0, a.Wout);
-        }, P::SMEM_ELEMS);
-    };
-    prefetch(a.pair0 + blockIdx.x);
-    sfor<0, UPB>([&](auto I) {
-        const int pair = a.pair0 + blockIdx.x + decltype(I)::value * gridDim.x;
-        if (pair < a.npairs && p3_unit_ok(a, pair, sidx)) unit(pair);
-    });
+        column_out<C>(a, a.U, c0, work, t);
+    }
+    column_pad<C>(a, a.U, c0, t);
+}
+
+// ---------------------------------------------------------------------------
+// Several spectra (lp_map, n > 1) and several source classes (Sec. 2.2
+// Eq. (4)): the frequencies of a column are parked in the order the threads
+// of stage 3 hold them -- run (m, k1) of column cl, elements k2 -- in shared
+// memory, or in global memory (PARKG) for the lengths that leave no room.
+// Every element is read back by the thread that wrote it or after a barrier.
+// ---------------------------------------------------------------------------
+template <class C>
+__device__ __forceinline__ void park_store(float2* F, int run, const float2 (&f)[C::Ge::R2])
+{
+    constexpr int R2 = C::Ge::R2, RUNS = C::US;
+    if constexpr (R2 % 2 == 0) {
+        float4* p = reinterpret_cast<float4*>(F) + run;
+#pragma unroll
+        for (int k = 0; k < R2; k += 2)
+            p[(k / 2) * RUNS] = make_float4(f[k].x, f[k].y, f[k + 1].x, f[k + 1].y);
+    } else {
+#pragma unroll
+        for (int k = 0; k < R2; ++k) F[k * RUNS + run] = f[k];
+    }
+}
+template <class C>
+__device__ __forceinline__ void park_load(float2 (&f)[C::Ge::R2], const float2* F, int run)
+{
+    constexpr int R2 = C::Ge::R2, RUNS = C::US;
+    if constexpr (R2 % 2 == 0) {
+        const float4* p = reinterpret_cast<const float4*>(F) + run;
+#pragma unroll
+        for (int k = 0; k < R2; k += 2) {
+            const float4 q = p[(k / 2) * RUNS];
+            f[k] = make_float2(q.x, q.y);
+            f[k + 1] = make_float2(q.z, q.w);
+        }
+    } else {
+#pragma unroll
+        for (int k = 0; k < R2; ++k) f[k] = F[k * RUNS + run];
+    }
+}
+
+// barrier of one group of TH threads (the whole block where there is one group)
+template <int TH, int GRP>
+__device__ __forceinline__ void group_sync(int grp)
+{
+    if constexpr (GRP == 1) __syncthreads();
+    else asm volatile("barrier.cta.sync %0, %1;\n" ::"r"(grp + 1), "n"(TH) : "memory");
+}
+
+// Forward transform of columns c0.. of T by all `th` threads of the block,
+// each frequency run handed to `sink(cl, m, k1, f)`.
+template <class C, class Sink>
+__device__ __forceinline__ void columns_forward(const float2* T, long long ldT, int H, int c0, int ncols,
+                                                BlkTw tw, float2* sm, int t, int th, Sink&& sink)
+{
+    using Ge = typename C::Ge;
+    using La = typename C::La;
+    constexpr int R0 = Ge::R0, R1 = Ge::R1, R2 = Ge::R2, NT = C::NT;
+    if constexpr (R0 > 1) {
+        column_stage1<C>(T, ldT, H, c0, ncols, sm, t, th);
+        __syncthreads();
+    }
+    const int li = t % Ge::G;
+    const int groups = th / Ge::G;
+#pragma unroll 1
+    for (int q0 = 0; q0 < C::UB; q0 += groups) {
+        const int q = t / Ge::G + q0;
+        const int cl = q % NT, m = q / NT;
+        const bool live = q < C::UB && (NT == 1 || c0 + cl < ncols);
+        float2* b = sm + cl * La::ELEMS + m * La::S0;
+        if (live && li < R2) {
+            float2 x[R1];
+            if constexpr (R0 > 1) {
+#pragma unroll
+                for (int l = 0; l < R1; ++l) x[l] = b[li + l * La::S1];
+            } else {
+                column_direct<Ge>(x, T, ldT, H, c0 + cl, li);
+            }
+            stage2_fwd<Ge>(x, b, m, li, lp_dsmem, tw.w2);
+        }
+        __syncwarp();
+        if (live && li < R1) {
+            float2 f[R2];
+            load_run<Ge>(f, b, li);
+            Dft<R2, -1, float2>::run(f);
+            sink(cl, m, li, f);
+        }
+    }
+}
+
+// Inverse of columns c0.. by the TH threads of one group (thread t of it):
+// `source(cl, m, k1, f)` gives each frequency run (live columns only).
+template <class C, int GRP, class Source>
+__device__ __forceinline__ void columns_inverse(const P2Args& a, float2* U, int c0, float2* sm, int t, int grp,
+                                                Source&& source)
+{
+    using Ge = typename C::Ge;
+    using La = typename C::La;
+    constexpr int R0 = Ge::R0, R1 = Ge::R1, R2 = Ge::R2, NT = C::NT;
+    const int li = t % Ge::G;
+#pragma unroll 1
+    for (int e = 0; e < C::EB; ++e) {
+        const int q = t / Ge::G + e * C::GROUPS;
+        const int cl = q % NT, m = q / NT;
+        const bool live = (C::EB * C::GROUPS == C::UB || q < C::UB) && (NT == 1 || c0 + cl < a.ncols);
+        float2* b = sm + cl * La::ELEMS + m * La::S0;
+        if (live && li < R1) {
+            float2 f[R2];
+            source(cl, m, li, f);
+            Dft<R2, 1, float2>::run(f);
+            store_run<Ge>(f, b, li);
+        }
+        __syncwarp();
+        if (live && li < R2) {
+            float2 x[R1];
+            stage2_inv<Ge>(x, b, m, li, lp_dsmem, a.tw.w2);
+            if constexpr (R0 > 1) {
+#pragma unroll
+                for (int l = 0; l < R1; ++l) b[li + l * La::S1] = x[l];
+            } else {
+                column_direct_out<Ge>(x, a, U, c0 + cl, li);
+            }
+        }
+        if constexpr (R0 == 1) __syncwarp();
+    }
+    if constexpr (R0 > 1) {
+        group_sync<C::TH, GRP>(grp);
+        column_out<C>(a, U, c0, sm, t);
+    }
+    column_pad<C>(a, U, c0, t);
+}
+
+// One spectrum of the batched pass.  Not inlined: as a loop body it would
+// let the compiler keep constants and addresses of the whole inverse live
+// across iterations.
+template <class C, int GRP, bool PARKG, bool KREAL>
+__device__ __noinline__ void p2_spectrum_pass(const P2Args& a, int c0, int s, int work, int t, int grp)
+{
+    using Ge = typename C::Ge;
+    constexpr int R2 = Ge::R2;
+    const float2* F = PARKG ? a.park + (size_t)c0 * Ge::N : lp_dsmem + Ge::W1 + GRP * C::WORK;
+    columns_inverse<C, GRP>(a, a.U + (long long)s * a.specU, c0, lp_dsmem + Ge::W1 + work, t, grp,
+                            [&](int cl, int m, int k1, float2(&f)[R2]) {
+                                typename std::conditional<KREAL, float, float2>::type k[R2];
+                                load_spectrum<Ge, KREAL>(k, static_cast<const float*>(a.K[s]) +
+                                                                (long long)(c0 + cl) * a.ldK * (KREAL ? 1 : 2), m, k1);
+                                park_load<C>(f, F, (cl * Ge::R0 + m) * Ge::R1 + k1);
+                                spectrum_product<KREAL>(f, k);
+                            });
+}
+
+// Several spectra: GRP groups of TH threads take the spectra in turn, each
+// with a working set of its own beside the one parked column (set).
+template <class C, int GRP, bool PARKG, bool KREAL>
+__global__ void __launch_bounds__(C::TH * GRP, C::MINB) p2_cols_multi(const __grid_constant__ P2Args a)
+{
+    pdl_begin<C::LATE>();
+    using Ge = typename C::Ge;
+    constexpr int NT = C::NT;
+    const int c0 = blockIdx.x * NT;
+    for (int cl = 0; cl < NT; ++cl)
+        if (c0 + cl < a.ncols && !p2_column_ok(a, c0 + cl, Ge::N, KREAL ? 1 : 2)) return;
+    float2* F = PARKG ? a.park + (size_t)c0 * Ge::N : lp_dsmem + Ge::W1 + GRP * C::WORK;
+    load_w1<Ge>(lp_dsmem, a.tw.w1, threadIdx.x, C::TH * GRP);
+    columns_forward<C>(a.T, a.ldT, a.H, c0, a.ncols, a.tw, lp_dsmem + Ge::W1, threadIdx.x, C::TH * GRP,
+                       [&](int cl, int m, int k1, float2(&f)[Ge::R2]) {
+                           park_store<C>(F, (cl * Ge::R0 + m) * Ge::R1 + k1, f);
+                       });
+    __syncthreads();
+    const int grp = GRP == 1 ? 0 : threadIdx.x / C::TH;
+    const int t = GRP == 1 ? threadIdx.x : threadIdx.x % C::TH;
+#pragma unroll 1
+    for (int s = grp; s < a.nspec; s += GRP) {
+        p2_spectrum_pass<C, GRP, PARKG, KREAL>(a, c0, s, grp * C::WORK, t, grp);
+        if constexpr (Ge::R0 > 1) group_sync<C::TH, GRP>(grp);  // the working set has been read
+    }
 }
 
 // ---------------------------------------------------------------------------
@@ -829,111 +907,251 @@ __global__ void __launch_bounds__(P::T, MINB) p3_rows_pf(const P3Args a)
 // and accumulated; one inverse transform follows.
 // ---------------------------------------------------------------------------
 struct P2MArgs {
+    P2Args a;  // output side, twiddles, ncols; T and K unused
     const float2* T[kMaxSpectraPerLaunch];
-    long long ldT;
-    int H;
     const void* K[kMaxSpectraPerLaunch];
-    long long ldK;
     int nclass;
-    float2* U;
-    long long ldU;
-    int r0, Hout, HoutPad;
-    int ncols;
-    TwChain twf, twi;
-    float2* acc;  // the sums of the products, N per column (global memory)
-    int* err;             // device status word (debug builds: bounds checks)
-    long long t_elems;    // float2 elements of each class's T buffer
-    long long k_elems;    // spectrum values of each spectrum
-    long long u_elems;    // float2 elements of U
-    long long acc_elems;  // float2 elements of the sums
 };
 
 // multiclass unit: column c of every class's T, of every spectrum, of U and of the sums
-__device__ __forceinline__ bool p2m_column_ok(const P2MArgs& a, int c, int n)
+__device__ __forceinline__ bool p2m_column_ok(const P2MArgs& m, int c, int n, int kw)
 {
-#if LP_DEBUG
-    return lp_checked(a.err, c >= 0 && c < a.ncols && a.H <= a.ldT && n <= a.ldK && a.HoutPad <= a.ldU &&
-                                 2 * t_index4(c, 0, a.ldT / 2) + t_row((int)a.ldT - 1) < a.t_elems &&
-                                 (long long)(c + 1) * a.ldK <= a.k_elems &&
-                                 2 * u_index4(c, 0, a.ldU / 2) + u_row(a.HoutPad - 1) < a.u_elems &&
-                                 (long long)(c + 1) * n <= a.acc_elems);
-#else
-    (void)a;
-    (void)c;
-    (void)n;
-    return true;
-#endif
+    return p2_column_ok(m.a, c, n, kw);
 }
 
-// One class of the Eq. (4) column pass: forward transform of the class's
-// column, product with its spectrum, summed into ACC (natural order; the
-// first class writes it).  Each thread adds only to the elements it owns
-// (j + m N/RL), so the sum needs no barrier.  Not inlined, for the same
-// reason as p2_spectrum_pass.
-template <class P, int N, bool KREAL>
-__device__ __noinline__ void p2_class_pass(const P2MArgs& a, int c, int q, float2* ACC, float2* sm)
+// One class: forward transform of the class's columns, product with its
+// spectrum, summed into F (the first class writes it).  Each thread adds only
+// to elements it owns, so the sum needs no barrier.
+template <class C, bool PARKG, bool KREAL>
+__device__ __noinline__ void p2_class_pass(const P2MArgs& M, int c0, int q)
 {
-    constexpr int R0 = P::R0, NB0 = N / R0;
-    constexpr int RL = P::RL, NBL = N / RL;
-    const int t = threadIdx.x;
-    const float2* col = t_column(a.T[q], a.ldT, c);
-    float2 v[P::E0][R0];
+    using Ge = typename C::Ge;
+    constexpr int R2 = Ge::R2;
+    const P2Args& a = M.a;
+    float2* F = PARKG ? a.park + (size_t)c0 * Ge::N : lp_dsmem + Ge::W1 + C::WORK;
+    columns_forward<C>(M.T[q], a.ldT, a.H, c0, a.ncols, a.tw, lp_dsmem + Ge::W1, threadIdx.x, C::TH,
+                       [&](int cl, int m, int k1, float2(&f)[R2]) {
+                           typename std::conditional<KREAL, float, float2>::type k[R2];
+                           load_spectrum<Ge, KREAL>(k, static_cast<const float*>(M.K[q]) +
+                                                           (long long)(c0 + cl) * a.ldK * (KREAL ? 1 : 2), m, k1);
+                           spectrum_product<KREAL>(f, k);
+                           const int run = (cl * Ge::R0 + m) * Ge::R1 + k1;
+                           if (q > 0) {
+                               float2 s[R2];
+                               park_load<C>(s, F, run);
 #pragma unroll
-    for (int e = 0; e < P::E0; ++e) {
-        const int j = t + e * P::T;
-        if (j >= NB0) continue;
-#pragma unroll
-        for (int m = 0; m < R0; ++m) {
-            const int row = j + m * NB0;
-            const long long off = (NB0 % 2 == 0) ? t_row(j) + m * t_row_step<NB0>() : t_row(row);
-            v[e][m] = row < a.H ? __ldg(col + off) : make_float2(0.f, 0.f);
-        }
+                               for (int i = 0; i < R2; ++i) f[i] = cadd(s[i], f[i]);
+                           }
+                           park_store<C>(F, run, f);
+                       });
+}
+
+template <class C, bool PARKG, bool KREAL>
+__global__ void __launch_bounds__(C::TH, C::MINB) p2_multiclass(const __grid_constant__ P2MArgs M)
+{
+    pdl_begin<C::LATE>();
+    using Ge = typename C::Ge;
+    constexpr int NT = C::NT;
+    const P2Args& a = M.a;
+    const int c0 = blockIdx.x * NT;
+    for (int cl = 0; cl < NT; ++cl)
+        if (c0 + cl < a.ncols && !p2m_column_ok(M, c0 + cl, Ge::N, KREAL ? 1 : 2)) return;
+    const float2* F = PARKG ? a.park + (size_t)c0 * Ge::N : lp_dsmem + Ge::W1 + C::WORK;
+    load_w1<Ge>(lp_dsmem, a.tw.w1, threadIdx.x, C::TH);
+#pragma unroll 1
+    for (int q = 0; q < M.nclass; ++q) {
+        p2_class_pass<C, PARKG, KREAL>(M, c0, q);
+        __syncthreads();  // the working set has been read
     }
-    P::FwdChain::run(v, t, sm, a.twf, [&](float2(&fz)[P::EL][RL], int tt) {
-        const long long kw = KREAL ? 1 : 2;
-        spectrum_product<P, N, KREAL, false>(fz, tt, static_cast<const float*>(a.K[q]) + (long long)c * a.ldK * kw,
-                                             nullptr);
+    // (groups of one round are the same in both directions: TH threads, one
+    // group; every run is read back by the thread that summed it)
+    columns_inverse<C, 1>(a, a.U, c0, lp_dsmem + Ge::W1, threadIdx.x, 0, [&](int cl, int m, int k1, float2(&f)[Ge::R2]) {
+        park_load<C>(f, F, (cl * Ge::R0 + m) * Ge::R1 + k1);
+    });
+}
+
+// ---------------------------------------------------------------------------
+// P3: row C2R of two packed rows per transform, NT transforms per block,
+// blockIdx.y selects the spectrum.  P1 backwards.
+// ---------------------------------------------------------------------------
+template <class C>
+__global__ void __launch_bounds__(C::TH, C::MINB) p3_rows(const __grid_constant__ P3Args a)
+{
+    pdl_begin<C::LATE>();
+    using Ge = typename C::Ge;
+    using La = typename C::La;
+    using RS = RowSub<C>;
+    constexpr int R0 = Ge::R0, R1 = Ge::R1, R2 = Ge::R2, N1 = Ge::N1, N = Ge::N, UR = R0 * R1;
+    const int pair0 = a.pair0 + blockIdx.x * C::NT;
+    const int sidx = blockIdx.y;
+    for (int tr = 0; tr < C::NT; ++tr)
+        if (pair0 + tr < a.npairs && !p3_unit_ok(a, pair0 + tr, sidx)) return;
+    const int t = threadIdx.x;
+    float2* work = lp_dsmem + Ge::W1;
+    const long long ldq = a.ldU / 2;
+    const float4* Uq = reinterpret_cast<const float4*>(a.U + (long long)sidx * a.specU);
+    auto store2 = [&](int tr, int col, float2 o) {
+        const int pair = pair0 + tr;
+        int cc = col - a.c0;
+        if (cc < 0) cc += N;
+        if (cc < a.Wout && pair < a.npairs) {
+            float* oa = a.out[sidx] + (long long)(2 * pair) * a.ldo + cc;
+            oa[0] = o.x;
+            if (2 * pair + 1 < a.Hout) oa[a.ldo] = o.y;
+        }
+    };
+    // lane li of sub-transform m at b: inverse stage 2, kept in place or (R0 = 1) stored
+    auto finish = [&](int tr, int m, int li, float2* b) {
+        float2 x[R1];
+        stage2_inv<Ge>(x, b, m, li, lp_dsmem, a.tw.w2);
+        if constexpr (R0 > 1) {
 #pragma unroll
-        for (int e = 0; e < P::EL; ++e) {
-            const int j = tt + e * P::T;
-            if (j >= NBL) continue;
+            for (int l = 0; l < R1; ++l) b[li + l * La::S1] = x[l];
+        } else {
 #pragma unroll
-            for (int m = 0; m < RL; ++m) {
-                float2& acc = ACC[j + m * NBL];
-                acc = q == 0 ? fz[e][m] : cadd(acc, fz[e][m]);
+            for (int l = 0; l < R1; ++l) store2(tr, li + l * R2, x[l]);
+        }
+    };
+    if constexpr (R0 > 1) load_w1<Ge>(lp_dsmem, a.tw.w1, t, C::TH);
+    if constexpr (RS::SHUFFLE) {
+        if constexpr (R0 > 1) __syncthreads();  // w1
+#pragma unroll 1
+        for (int e = 0; e < RS::ROUNDS; ++e) {
+            const RS s(t, e);
+            float2* b = work + s.tr * La::ELEMS + s.m * La::S0;
+            const int pair = pair0 + s.tr;
+            const bool load = s.live && s.li < R1 && pair < a.npairs;
+            const bool vb = 2 * pair + 1 < a.Hout;
+            const int u = s.m + R0 * s.li;
+            const float4* src = Uq + u_index4(u, pair, ldq);
+            float4 q[R2 / 2 + 1];
+#pragma unroll
+            for (int k = 0; k <= R2 / 2; ++k) {
+                const int c = u + k * UR;
+                q[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+                if (load && (k < R2 / 2 || c < a.ncols)) {
+                    if constexpr (UR % kUCB == 0) q[k] = src[k * (UR / kUCB) * (ldq * kUCB)];
+                    else q[k] = Uq[u_index4(c, pair, ldq)];
+                }
+                if (!vb) q[k].z = q[k].w = 0.f;
+            }
+            // own lower half; the upper half from the partner (the origin
+            // run holds its own, one element further on)
+            float2 f[R2];
+#pragma unroll
+            for (int k = 0; k < R2 / 2; ++k) f[k] = join_lo(q[k]);
+#pragma unroll
+            for (int k = 0; k < (R2 + 1) / 2; ++k) {
+                float2 h = join_hi(q[k]);
+                h.x = __shfl_sync(0xffffffffu, h.x, s.partner);
+                h.y = __shfl_sync(0xffffffffu, h.y, s.partner);
+                if (k == R2 / 2) {  // R2 odd: the middle element, whichever side of N / 2 it is on
+                    f[k] = u + k * UR < a.ncols ? join_lo(q[k]) : h;
+                } else {
+                    const float2 own = (R2 % 2 == 0 && k + 1 == R2 / 2) ? join_lo(q[R2 / 2]) : join_hi(q[k + 1]);
+                    f[R2 - 1 - k] = s.origin ? own : h;
+                }
+            }
+            if (s.live && s.li < R1) {
+                Dft<R2, 1, float2>::run(f);
+                store_run<Ge>(f, b, s.li);
+            }
+            __syncwarp();
+            if (s.live && s.li < R2) finish(s.tr, s.m, s.li, b);
+        }
+    } else {
+#pragma unroll 1
+        for (int e = 0; e < C::ES; ++e) {
+            const int v = t + e * C::TH;
+            if (C::ES * C::TH != C::US && v >= C::US) break;
+            const int tr = v % C::NT, u = v / C::NT;
+            const int pair = pair0 + tr;
+            if (pair >= a.npairs) continue;
+            const bool vb = 2 * pair + 1 < a.Hout;
+            const int up = u == 0 ? 0 : UR - u;
+            float2* z = work + tr * La::ELEMS + (u % R0) * La::S0 + (u / R0) * La::S1;
+            float2* zp = work + tr * La::ELEMS + (up % R0) * La::S0 + (up / R0) * La::S1;
+            const float4* src = Uq + u_index4(u, pair, ldq);
+            float4 q[R2 / 2 + 1];
+#pragma unroll
+            for (int k = 0; k <= R2 / 2; ++k) {
+                const int c = u + k * UR;
+                if (k == R2 / 2 && c >= a.ncols) break;
+                if constexpr (UR % kUCB == 0) q[k] = src[k * (UR / kUCB) * (ldq * kUCB)];
+                else q[k] = Uq[u_index4(c, pair, ldq)];
+                if (!vb) q[k].z = q[k].w = 0.f;
+            }
+            if (La::VEC && u > 0) {
+#pragma unroll
+                for (int k = 0; k < R2 / 2; k += 2) {
+                    const float2 l0 = join_lo(q[k]), h0 = join_hi(q[k]);
+                    if (k + 1 < R2 / 2) {
+                        const float2 l1 = join_lo(q[k + 1]), h1 = join_hi(q[k + 1]);
+                        *reinterpret_cast<float4*>(z + k) = make_float4(l0.x, l0.y, l1.x, l1.y);
+                        *reinterpret_cast<float4*>(zp + (R2 - 2 - k)) = make_float4(h1.x, h1.y, h0.x, h0.y);
+                    } else {
+                        z[k] = l0;
+                        zp[R2 - 1 - k] = h0;
+                    }
+                }
+            } else {
+#pragma unroll
+                for (int k = 0; k <= R2 / 2; ++k) {
+                    const int c = u + k * UR;
+                    if (k == R2 / 2 && c >= a.ncols) break;
+                    z[k] = join_lo(q[k]);
+                    if (k == 0 ? u != 0 : (k != R2 / 2 || 2 * c != N)) zp[u > 0 ? R2 - 1 - k : R2 - k] = join_hi(q[k]);
+                }
             }
         }
-    });
-}
-
-template <class P, int N, bool KREAL>
-__global__ void __launch_bounds__(P::T) p2_multiclass(const __grid_constant__ P2MArgs a)
-{
-    pdl_begin();
-    extern __shared__ float2 smem2[];
-    constexpr int RL = P::RL, NBL = N / RL;
-    float2* sm = smem2;
-    const int c = blockIdx.x;
-    const int t = threadIdx.x;
-    if (!p2m_column_ok(a, c, N)) return;  // (whole block: before any barrier)
-    // the sums live in global memory (L2-resident while the block runs), so
-    // shared memory holds one exchange buffer at every length; every
-    // element of ACC is owned by one thread (j + m N/RL), which writes it for
-    // the first class, adds to it for the others and reads it back below
-    float2* ACC = a.acc + (size_t)c * N;
-    for (int q = 0; q < a.nclass; ++q) p2_class_pass<P, N, KREAL>(a, c, q, ACC, sm);
-    float2 acc[P::EL][RL];
-#pragma unroll
-    for (int e = 0; e < P::EL; ++e) {
-        const int j = t + e * P::T;
-        if (j >= NBL) continue;
-#pragma unroll
-        for (int m = 0; m < RL; ++m) acc[e][m] = ACC[j + m * NBL];
+        __syncthreads();
+        const int li = t % Ge::G;
+#pragma unroll 1
+        for (int e = 0; e < C::EB; ++e) {
+            const int q = t / Ge::G + e * C::GROUPS;
+            const bool live = C::EB * C::GROUPS == C::UB || q < C::UB;
+            const int tr = C::NT == 1 ? 0 : q / R0;
+            const int m = q - tr * R0;
+            float2* b = work + tr * La::ELEMS + m * La::S0;
+            if (live && li < R1) {
+                float2 f[R2];
+                load_run<Ge>(f, b, li);
+                Dft<R2, 1, float2>::run(f);
+                store_run<Ge>(f, b, li);
+            }
+            __syncwarp();
+            if (live && li < R2) finish(tr, m, li, b);
+        }
     }
-    float2* Uc = u_column(a.U, a.ldU, c);
-    P::InvChain::run(acc, t, sm, a.twi, [&](float2(&o)[P::EJ][P::R0], int tt) {
-        store_column<P, N>(o, tt, Uc, a.r0, a.Hout, a.HoutPad);
-    });
+    if constexpr (R0 > 1) {
+        __syncthreads();
+#pragma unroll 1
+        for (int e = 0; e < C::E1; ++e) {
+            const int u = t + e * C::TH;
+            if (C::E1 * C::TH != C::U1 && u >= C::U1) break;
+            const int tr = C::NT == 1 ? 0 : u / N1;
+            const int j = u - tr * N1;
+            const float2* w = work + tr * La::ELEMS + stage1_addr<Ge>(j);
+            float2 v[R0];
+#pragma unroll
+            for (int m = 0; m < R0; ++m) v[m] = w[m * La::S0];
+            Dft<R0, 1, float2>::run(v);
+            const int pair = pair0 + tr;
+            if (pair >= a.npairs) continue;
+            const bool vb = 2 * pair + 1 < a.Hout;
+            float* oa = a.out[sidx] + (long long)(2 * pair) * a.ldo;
+            float* ob = oa + a.ldo;
+#pragma unroll
+            for (int q = 0; q < R0; ++q) {
+                int cc = j + q * N1 - a.c0;
+                if (cc < 0) cc += N;
+                if (cc < a.Wout) {
+                    oa[cc] = v[q].x;
+                    if (vb) ob[cc] = v[q].y;
+                }
+            }
+        }
+    }
 }
 
 }  // namespace lpk

@@ -1,24 +1,19 @@
 // Device building blocks of the FFT path: compile-time trigonometry,
-// in-register DFTs of small radices, and Stockham stage chains that exchange
-// data through padded structure-of-arrays shared memory.
+// in-register DFTs of small radices, and block transforms that exchange data
+// in place through shared memory.
 //
 // The transform computed is the DFT of Sec. 2.3 Eq. (10) (0-based indices),
 // F[k] = sum_n f[n] exp(DIR * i 2 pi k n / N), DIR = -1 forward, +1 inverse
 // (unnormalised both ways), evaluated by the Cooley-Tukey factorisation the
-// paper cites for FFTs (Sec. 2.3): N = R_0 R_1 ... R_{S-1}, one radix-R_s
-// butterfly stage per factor, in the self-sorting (Stockham) arrangement so
-// that the output comes out in natural order without a bit-reversal pass.
-//
-// Stage s of a chain, with Ns = R_0 ... R_{s-1} and butterfly index
-// j in [0, N/R_s):
+// paper cites for FFTs (Sec. 2.3), one butterfly stage per factor of N: in
+// place, three factors at most, for the FP32 passes (block transforms
+// below), and in the self-sorting (Stockham) order, stage s of
+// N = R_0 R_1 ... R_{S-1}, for the tensor-core column pass and the FP64
+// spectrum build: with Ns = R_0 ... R_{s-1} and butterfly j in [0, N/R_s)
 //   inputs   x[j + m N/R_s],                      m = 0..R_s-1
 //   twiddle  x_m *= exp(DIR i 2 pi (j mod Ns) m / (Ns R_s))
 //   DFT of size R_s in registers
 //   outputs  y[(j div Ns) Ns R_s + (j mod Ns) + m Ns]
-// In the last stage Ns = N / R_{S-1}, so thread j holds y[j + m N/R_{S-1}]:
-// exactly the set the first stage of a chain with the same radix reads.  The
-// convolution kernels use that to multiply by the PSF spectrum between the
-// forward and the inverse column transform without touching shared memory.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -377,125 +372,160 @@ template <> struct SeqInfo<Seq<>> {
 };
 
 // ---------------------------------------------------------------------------
-// Shared-memory exchange layout.  Complex values are stored interleaved
-// (one 64-bit access per element).  The exchange after a stage with group
-// size P = Ns * R inserts q padding elements after every group of P:
-//   padded(i) = i + q * (i / P).
-// The next stage reads x[j + m NB'] with NB' = N / R' a multiple of P, so
-// both sides stay "per-thread base + compile-time offset".  q is chosen so
-// that the 16 threads of each 64-bit access phase hit distinct bank pairs:
-// an odd element stride when Ns = 1, and consecutive banks across groups
-// (Ns R + q = Ns mod 16) otherwise.
+// Block transforms: N = R0 R1 R2 (R0 = 1: two factors), in place in shared
+// memory.  With N1 = R1 R2, input n = j + N1 q (j < N1, q < R0), j = i + R2 l
+// (i < R2, l < R1), and frequency k = m + R0 (k1 + R1 k2):
+//
+//   stage 1   for each j: DFT of size R0 over q -> m
+//   stage 2   for each m, i: times exp(-i 2 pi l m / (R0 R1)), DFT of size R1
+//             over l -> k1, times exp(-i 2 pi i (m + R0 k1) / N)
+//   stage 3   for each m, k1: DFT of size R2 over i -> k2
+//
+// (decimation in frequency; the inverse runs the mirror image, decimation in
+// time, with the conjugate twiddles).  Element (m, l, i) sits at
+// m S0 + l S1 + i, and every butterfly writes where it read: stage 2 leaves
+// k1 in l's place, stage 3 leaves k2 in i's place.  So an exchange needs no
+// second buffer and no barrier before its writes, and the R1 R2-point
+// sub-transform of one m (stages 2 and 3) stays within one group of G lanes
+// of a warp (8, 16 or 32, the smallest that holds max(R1, R2)): its exchange
+// is ordered by __syncwarp alone.  Only the exchange between stage 1 and the
+// sub-transforms crosses warps, which leaves one block barrier per transform
+// where the self-sorting order needs two per exchange.
+//
+// Twiddles: the factor exp(-i 2 pi (i + R2 l) m / N) between stages 1 and 2
+// is split into its l part, R0 R1 values that a block keeps in shared memory
+// (w1; the lanes of a group read one address), and its i part, which is the
+// same for the whole butterfly and joins the table of stage 2's outputs (w2,
+// N values).  The passes are bound by shared-memory and L1 bandwidth: a
+// table of stage 1 of its own would add 8 bytes per point and direction.
 // ---------------------------------------------------------------------------
-__host__ __device__ constexpr int pad_q(int Ns, int R)
-{
-    return Ns == 1 ? ((R % 2 == 0) ? 1 : 0) : (((Ns * (1 - R)) % 16) + 16) % 16;
-}
-
-// elements of shared memory one chain's exchanges touch
-template <int... Rs>
-__host__ __device__ constexpr int chain_extent()
-{
-    constexpr int S = sizeof...(Rs);
-    const int r[S] = {Rs...};
-    int n = 1;
-    for (int s = 0; s < S; ++s) n *= r[s];
-    int ext = n, Ns = 1;
-    for (int s = 0; s + 1 < S; ++s) {
-        const int P = Ns * r[s], q = pad_q(Ns, r[s]);
-        const int e = (n - 1) + q * ((n - 1) / P) + 1;
-        ext = e > ext ? e : ext;
-        Ns = P;
-    }
-    return ext;
-}
-template <class S> struct ChainExtent;
-template <int... Rs> struct ChainExtent<Seq<Rs...>> {
-    static constexpr int value = chain_extent<Rs...>();
-};
-
-// ---------------------------------------------------------------------------
-// Stage chain in FP32.  TT threads cooperate on one transform; in a stage
-// with NB = N/R butterflies, thread t owns butterflies j = t + e TT for
-// e < E = ceil(NB / TT) (j < NB).  `run` takes the inputs of the first
-// stage in v[e] (thread t holds x[j + m N/R]), runs every stage, exchanging
-// through shared memory `sm` between stages, and hands the last stage's
-// outputs (v[e] holds y[j + m N/R_last]) to `fin(v, t)`.
-// Every thread of the block must call it (it contains barriers).
-// ---------------------------------------------------------------------------
-// Double buffering (DB): exchange number x of the block's sequence uses
-// buffer (BUF + x) mod 2 (sm and sm + bstride).  Consecutive exchanges then
-// use different buffers, so the write of an exchange only has to wait for
-// the readers of the exchange two before it -- which finished before the
-// previous exchange's barrier -- and one barrier per exchange suffices.
-template <int N, int DIR, int Ns, int SIdx, int TT, class S, bool DB = false, int BUF = 0> struct Chain;
-
-template <int N, int DIR, int Ns, int SIdx, int TT, int R, int... Rest, bool DB, int BUF>
-struct Chain<N, DIR, Ns, SIdx, TT, Seq<R, Rest...>, DB, BUF> {
-    static constexpr int NB = N / R;
-    static constexpr int E = (NB + TT - 1) / TT;
-    static constexpr int EXCHANGES = sizeof...(Rest);
-
-    template <class Fin>
-    __device__ __forceinline__ static void run(float2 (&v)[E][R], int t, float2* sm,
-                                               const TwChain& tw, Fin&& fin, int bstride = 0)
+template <int N_, int R0_, int R1_, int R2_>
+struct Geo {
+    static constexpr int N = N_, R0 = R0_, R1 = R1_, R2 = R2_, N1 = R1_ * R2_;
+    static_assert(R0 * R1 * R2 == N, "radices must multiply to N");
+    static constexpr int RM = R1 > R2 ? R1 : R2;
+    static_assert(RM <= 32, "a sub-transform's lanes are one warp at most");
+    static constexpr int G = RM <= 8 ? 8 : RM <= 16 ? 16 : 32;  // lanes of a sub-transform
+    static constexpr int GPW = 32 / G;                          // sub-transforms per warp and round
+    static constexpr int R1P = (R1 + 1) / 2 * 2;                // entries of w1 per m (16-byte rows)
+    static constexpr int W1 = R0 > 1 ? (R0 * R1P + 7) / 8 * 8 : 0;  // shared-memory entries of w1
+    // position in a spectrum column of frequency (m, k1, k2): the lanes of
+    // a sub-transform (k1) read VK consecutive k2 each, side by side
+    static constexpr int VK = R2 % 4 == 0 ? 4 : R2 % 2 == 0 ? 2 : 1;
+    static constexpr __host__ __device__ int kpos(int m, int k1, int k2)
     {
-#pragma unroll
-        for (int e = 0; e < E; ++e) {
-            const int j = t + e * TT;
-            if (j < NB) {
-                if constexpr (Ns > 1) {
-                    const float2* tab = tw.p[SIdx];
-                    // opaque to the optimiser: keeps the table loads inside
-                    // loops that repeat a chain instead of hoisting every
-                    // stage's twiddles into registers across iterations
-                    asm volatile("" : "+l"(tab));
-                    tab += j % Ns;
-#pragma unroll
-                    for (int m = 1; m < R; ++m) {
-                        float2 w = __ldg(tab + (m - 1) * Ns);
-                        if constexpr (DIR > 0) w.y = -w.y;
-                        v[e][m] = cmul(v[e][m], w);
-                    }
-                }
-                Dft<R, DIR, float2>::run(v[e]);
-            }
-        }
-        if constexpr (sizeof...(Rest) == 0) {
-            fin(v, t);
-        } else {
-            using Next = Chain<N, DIR, Ns * R, SIdx + 1, TT, Seq<Rest...>, DB, BUF>;
-            float2* xb = (DB && ((BUF + SIdx) & 1)) ? sm + bstride : sm;
-            constexpr int R2 = SeqInfo<Seq<Rest...>>::first;
-            constexpr int NB2 = N / R2;
-            constexpr int P = Ns * R;
-            constexpr int q = pad_q(Ns, R);
-            static_assert(NB2 % P == 0, "reader stride must be a multiple of the group size");
-            constexpr int rstride = NB2 + q * (NB2 / P);
-            if constexpr (!DB) __syncthreads();  // earlier readers of sm are done
-#pragma unroll
-            for (int e = 0; e < E; ++e) {
-                const int j = t + e * TT;
-                if (j < NB) {
-                    float2* w0 = xb + (j / Ns) * (P + q) + (j % Ns);
-#pragma unroll
-                    for (int m = 0; m < R; ++m) w0[m * Ns] = v[e][m];
-                }
-            }
-            __syncthreads();
-            float2 w[Next::E][R2];
-#pragma unroll
-            for (int e = 0; e < Next::E; ++e) {
-                const int j = t + e * TT;
-                if (j < NB2) {
-                    const float2* r0 = xb + j + q * (j / P);
-#pragma unroll
-                    for (int m = 0; m < R2; ++m) w[e][m] = r0[m * rstride];
-                }
-            }
-            Next::run(w, t, sm, tw, fin, bstride);
-        }
+        return ((m * (R2 / VK) + k2 / VK) * R1 + k1) * VK + k2 % VK;
     }
 };
+
+// Strides of the in-place layout.  Where R2 is even, stage 3 moves its R2
+// consecutive elements 16 bytes at a time: S1 is even with S1 / 2 odd, and S0
+// likewise (eight lanes of a 16-byte access on consecutive k1, or on
+// consecutive m in the row passes' sweep, then hit distinct banks); S1 = R2
+// wherever that is so already, which keeps stage 1's writes consecutive.
+// Where R2 is odd the accesses are 8 bytes, and S1 and S0 are odd.
+template <class Ge>
+struct Lay {
+    static constexpr bool VEC = Ge::R2 % 2 == 0;
+    static constexpr int S1 = !VEC ? Ge::R2 : (Ge::R2 / 2) % 2 ? Ge::R2 : Ge::R2 + 2;
+    static constexpr int S0_ = Ge::R1 * S1;
+    static constexpr int S0 = !VEC ? S0_ | 1 : (S0_ / 2) % 2 ? S0_ : S0_ + 2;
+    // elements of one transform, ELEMS mod 16 = 8: two transforms taken by
+    // alternating lanes do not share banks (and starts stay 16-byte aligned)
+    static constexpr int ELEMS = (Ge::R0 * S0 + 7) / 16 * 16 + 8;
+    static_assert(ELEMS >= Ge::R0 * S0, "layout extent");
+};
+
+template <class C> __device__ __forceinline__ C cmulc(C a, C w)  // a conj(w)
+{
+    return mk<C>(a.x * w.x + a.y * w.y, a.y * w.x - a.x * w.y);
+}
+
+// address of stage 1's butterfly j within a transform (its outputs m: + m S0)
+template <class Ge>
+__device__ __forceinline__ int stage1_addr(int j)
+{
+    return Lay<Ge>::S1 == Ge::R2 ? j : j + (j / Ge::R2) * (Lay<Ge>::S1 - Ge::R2);
+}
+
+// the block's copy of w1 (read after the barrier that follows stage 1)
+template <class Ge>
+__device__ __forceinline__ void load_w1(float2* w1, const float2* __restrict__ table, int t, int th)
+{
+    if constexpr (Ge::R0 > 1)
+        for (int i = t; i < Ge::R0 * Ge::R1P; i += th) w1[i] = __ldg(table + i);
+}
+
+// x[l] *= w1[m][l] (CONJ: its conjugate)
+template <class Ge, bool CONJ>
+__device__ __forceinline__ void twiddle_in(float2 (&x)[Ge::R1], const float2* w1m)
+{
+    if constexpr (Ge::R0 > 1) {
+#pragma unroll
+        for (int l = 0; l < Ge::R1; l += 2) {
+            const float4 w = *reinterpret_cast<const float4*>(w1m + l);
+            if (l > 0) x[l] = CONJ ? cmulc(x[l], make_float2(w.x, w.y)) : cmul(x[l], make_float2(w.x, w.y));
+            if (l + 1 < Ge::R1)
+                x[l + 1] = CONJ ? cmulc(x[l + 1], make_float2(w.z, w.w)) : cmul(x[l + 1], make_float2(w.z, w.w));
+        }
+    }
+}
+
+// stage 2 of lane i of sub-transform m at b (x loaded): twiddles and DFT over l, in place
+template <class Ge>
+__device__ __forceinline__ void stage2_fwd(float2 (&x)[Ge::R1], float2* b, int m, int i, const float2* w1,
+                                           const float2* __restrict__ w2)
+{
+    constexpr int K0 = Ge::R0 > 1 ? 0 : 1;  // (m = 0: output k1 = 0 has no twiddle)
+    twiddle_in<Ge, false>(x, w1 + m * Ge::R1P);
+    Dft<Ge::R1, -1, float2>::run(x);
+    const float2* w = w2 + m * Ge::N1 + i;
+    if constexpr (K0 == 1) b[i] = x[0];
+#pragma unroll
+    for (int k = K0; k < Ge::R1; ++k) b[i + k * Lay<Ge>::S1] = cmul(x[k], __ldg(w + k * Ge::R2));
+}
+template <class Ge>
+__device__ __forceinline__ void stage2_inv(float2 (&x)[Ge::R1], const float2* b, int m, int i, const float2* w1,
+                                           const float2* __restrict__ w2)
+{
+    constexpr int K0 = Ge::R0 > 1 ? 0 : 1;
+    const float2* w = w2 + m * Ge::N1 + i;
+    if constexpr (K0 == 1) x[0] = b[i];
+#pragma unroll
+    for (int k = K0; k < Ge::R1; ++k) x[k] = cmulc(b[i + k * Lay<Ge>::S1], __ldg(w + k * Ge::R2));
+    Dft<Ge::R1, 1, float2>::run(x);
+    twiddle_in<Ge, true>(x, w1 + m * Ge::R1P);
+}
+
+// the R2 consecutive elements of lane k1
+template <class Ge>
+__device__ __forceinline__ void load_run(float2 (&f)[Ge::R2], const float2* b, int k1)
+{
+    const float2* p = b + k1 * Lay<Ge>::S1;
+    if constexpr (Lay<Ge>::VEC) {
+#pragma unroll
+        for (int k = 0; k < Ge::R2; k += 2) {
+            const float4 q = *reinterpret_cast<const float4*>(p + k);
+            f[k] = make_float2(q.x, q.y);
+            f[k + 1] = make_float2(q.z, q.w);
+        }
+    } else {
+#pragma unroll
+        for (int k = 0; k < Ge::R2; ++k) f[k] = p[k];
+    }
+}
+template <class Ge>
+__device__ __forceinline__ void store_run(const float2 (&f)[Ge::R2], float2* b, int k1)
+{
+    float2* p = b + k1 * Lay<Ge>::S1;
+    if constexpr (Lay<Ge>::VEC) {
+#pragma unroll
+        for (int k = 0; k < Ge::R2; k += 2)
+            *reinterpret_cast<float4*>(p + k) = make_float4(f[k].x, f[k].y, f[k + 1].x, f[k + 1].y);
+    } else {
+#pragma unroll
+        for (int k = 0; k < Ge::R2; ++k) p[k] = f[k];
+    }
+}
 
 }  // namespace lpk

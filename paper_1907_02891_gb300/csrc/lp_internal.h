@@ -13,6 +13,15 @@ struct TwChain {
     const float2* p[6];
 };
 
+// Twiddle tables of one length's block transform N = R0 R1 R2 (N1 = R1 R2):
+// w1[m R1P + l] = exp(-i 2 pi l m / (R0 R1)), m < R0, l < R1 (R1P: R1 rounded
+// up to even), and w2[m N1 + k R2 + i] = exp(-i 2 pi i (m + R0 k) / N), k < R1,
+// i < R2.
+struct BlkTw {
+    const float2* w1;
+    const float2* w2;
+};
+
 struct P1Args;
 struct P2Args;
 struct P3Args;
@@ -22,15 +31,14 @@ struct P2TcArgs;
 // One supported FFT length with its compiled FP32 kernels.
 struct SizeKernels {
     int N;
+    int geo[3];          // R0, R1, R2 of the FP32 passes' block transforms
+    int vk;              // consecutive frequencies a spectrum run is read in (Geo::VK)
     int nstages;
-    int radices[6];      // forward order
-    int threads;         // threads per transform
-    int f1, f3;          // transforms per block in the row passes
-    int smem_bytes;      // dynamic shared memory of one transform
+    int radices[6];      // forward order of the tensor-core column pass's chain
     int batch;           // several spectra: one forward column transform, parked
+    int park_multi;      // the batched pass parks its column in global memory
+    int park_class;      // the Eq. (4) pass keeps its sums in global memory
     cudaError_t (*set_attrs)();
-    // launchers: pick the persistent prefetching kernel when its shared
-    // memory fits, the one-unit-per-block kernel otherwise
     cudaError_t (*p1)(const P1Args&, cudaStream_t);
     cudaError_t (*p2)(const P2Args&, bool kreal, cudaStream_t);
     cudaError_t (*p2m)(const P2MArgs&, bool kreal, cudaStream_t);
@@ -46,6 +54,13 @@ struct SizeKernels {
 extern const SizeKernels* const kAllSizes[];
 extern const int kNumSizes;
 
+// Order of the frequencies within a stored spectrum column: frequency
+// u = m + r0 (k1 + r1 k2) at ((m (r2 / vk) + k2 / vk) r1 + k1) vk + k2 mod vk
+// (r0 = 0: natural order).
+struct SpecOrder {
+    int r0, r1, r2, vk;
+};
+
 // FP64 spectrum pipeline (spectrum.cu)
 bool fft64_supported(int N);
 cudaError_t psf_fingerprint_launch(const double* K, long long n, unsigned long long* d_out,
@@ -54,7 +69,10 @@ cudaError_t psf_symmetry_launch(const double* K, int hk, int wk, int* d_asym, cu
 // *d_diff |= 1 where a[i] and b[i] differ in any bit (i < n)
 cudaError_t psf_compare_launch(const double* a, const double* b, long long n, int* d_diff, cudaStream_t st);
 cudaError_t psf_spectrum_build(const double* K, int hk, int wk, int Ny, int Nx, int real_only,
-                               void* dst, long long ldK, double2* W1, double2* W1b,
+                               void* dst, long long ldK, SpecOrder order, double2* W1, double2* W1b,
                                double2* W2a, double2* W2b, cudaStream_t st);
+// a stored spectrum's columns in natural order, packed (ny values each)
+cudaError_t spectrum_copy_natural(const void* data, long long ldK, int ny, int ncols, int is_real, SpecOrder order,
+                                  float* dst, cudaStream_t st);
 
 }  // namespace lpk

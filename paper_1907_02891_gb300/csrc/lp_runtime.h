@@ -31,7 +31,8 @@ struct PlanRec {
     const lpk::SizeKernels* k = nullptr;
     float2* tw = nullptr;  // device twiddle tables (forward chain, then reversed chain)
     size_t bytes = 0;
-    lpk::TwChain fwd{}, rev{};
+    lpk::BlkTw blk{};            // block transform (FP32 passes)
+    lpk::TwChain fwd{}, rev{};   // self-sorting chains (tensor-core column pass)
     // tables of the tensor-core column pass (split-BF16 DFT matrices, then
     // twiddle step factors; same block as tw; null where the length has no
     // such pass)
@@ -90,7 +91,6 @@ struct lp_spectrum {
 
 struct lp_ctx {
     int device = 0;
-    int sms = 0;  // multiprocessors of the device (0: not looked up yet)
     size_t budget = 0, used = 0;
     std::mutex mem_mu, plan_mu, spec_mu, ws_mu;
     std::map<int, std::unique_ptr<PlanRec>> plans;
@@ -134,7 +134,7 @@ lp_status lp_validate_map(lp_ctx* ctx, const float* L, int h, int w, int ldl,
 // bytes of one map's workspace: T, then U for up to kMaxSpectraPerLaunch
 // spectra (the spectra of one launch), + alignment slack
 size_t lp_workspace_bytes(const MapDims& d, int n);
-// parked forward column spectra of the batched column pass: Ny complex per column
+// parked column frequencies of the batched and Eq. (4) column passes: Ny complex per column
 size_t lp_park_bytes(const MapDims& d);
 lp_status lp_launch_map(lp_ctx* ctx, const float* L, int h, int w, int ldl,
                         const lp_spectrum* const* spectra, int n, float* const* out, int ldo,

@@ -150,9 +150,18 @@ __global__ void psf_scatter_cols(const double2* __restrict__ W1, int hk, int Nx,
     W2[(long long)yy * ncols + c] = W1[(long long)y * Nx + c];
 }
 
-// dst[c][u] = scale * W2[u][c], 32 x 32 tiles through shared memory
+// position of frequency u in a spectrum column (SpecOrder)
+__device__ __forceinline__ int spec_pos(SpecOrder o, int u)
+{
+    if (o.r0 == 0) return u;
+    const int m = u % o.r0, k = u / o.r0;
+    const int k1 = k % o.r1, k2 = k / o.r1;
+    return ((m * (o.r2 / o.vk) + k2 / o.vk) * o.r1 + k1) * o.vk + k2 % o.vk;
+}
+
+// dst[c][pos(u)] = scale * W2[u][c], 32 x 32 tiles through shared memory
 __global__ void psf_store_spectrum(const double2* __restrict__ W2, int Ny, int ncols, double scale,
-                                   int real_only, void* dst, long long ldK)
+                                   int real_only, void* dst, long long ldK, SpecOrder order)
 {
     __shared__ double2 tile[32][33];
     const int u0 = blockIdx.y * 32, c0 = blockIdx.x * 32;
@@ -165,10 +174,11 @@ __global__ void psf_store_spectrum(const double2* __restrict__ W2, int Ny, int n
         const int c = c0 + r, u = u0 + threadIdx.x;
         if (u < Ny && c < ncols) {
             const double2 z = tile[threadIdx.x][r];
+            const int p = spec_pos(order, u);
             if (real_only)
-                static_cast<float*>(dst)[(long long)c * ldK + u] = (float)(z.x * scale);
+                static_cast<float*>(dst)[(long long)c * ldK + p] = (float)(z.x * scale);
             else
-                static_cast<float2*>(dst)[(long long)c * ldK + u] =
+                static_cast<float2*>(dst)[(long long)c * ldK + p] =
                     make_float2((float)(z.x * scale), (float)(z.y * scale));
         }
     }
@@ -225,7 +235,7 @@ cudaError_t psf_symmetry_launch(const double* K, int hk, int wk, int* d_asym, cu
 
 // Full spectrum build.  W1 holds hk*Nx, W2a/W2b each Ny*ncols complex128.
 cudaError_t psf_spectrum_build(const double* K, int hk, int wk, int Ny, int Nx, int real_only,
-                               void* dst, long long ldK, double2* W1, double2* W1b,
+                               void* dst, long long ldK, SpecOrder order, double2* W1, double2* W1b,
                                double2* W2a, double2* W2b, cudaStream_t st)
 {
     const int ncols = Nx / 2 + 1;
@@ -249,7 +259,26 @@ cudaError_t psf_spectrum_build(const double* K, int hk, int wk, int Ny, int Nx, 
     if ((e = fft64_forward(W2a, W2b, Ny, ncols, 1, ncols, 1, st, &cols)) != cudaSuccess) return e;
     const double scale = 1.0 / (2.0 * (double)Ny * (double)Nx);
     dim3 grid((ncols + 31) / 32, (Ny + 31) / 32), block(32, 8);
-    psf_store_spectrum<<<grid, block, 0, st>>>(cols, Ny, ncols, scale, real_only, dst, ldK);
+    psf_store_spectrum<<<grid, block, 0, st>>>(cols, Ny, ncols, scale, real_only, dst, ldK, order);
+    return cudaGetLastError();
+}
+
+template <class V>
+__global__ void spectrum_natural(const V* __restrict__ src, long long ldK, int ny, SpecOrder order, V* __restrict__ dst)
+{
+    const int u = blockIdx.x * blockDim.x + threadIdx.x;
+    if (u < ny) dst[(long long)blockIdx.y * ny + u] = src[(long long)blockIdx.y * ldK + spec_pos(order, u)];
+}
+
+cudaError_t spectrum_copy_natural(const void* data, long long ldK, int ny, int ncols, int is_real, SpecOrder order,
+                                  float* dst, cudaStream_t st)
+{
+    const dim3 grid((ny + 255) / 256, ncols);  // ncols <= 8641: within the grid's y limit
+    if (is_real)
+        spectrum_natural<float><<<grid, 256, 0, st>>>(static_cast<const float*>(data), ldK, ny, order, dst);
+    else
+        spectrum_natural<float2><<<grid, 256, 0, st>>>(static_cast<const float2*>(data), ldK, ny, order,
+                                                       reinterpret_cast<float2*>(dst));
     return cudaGetLastError();
 }
 

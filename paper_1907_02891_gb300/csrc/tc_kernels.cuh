@@ -44,7 +44,8 @@ constexpr int ru16(int x) { return (x + 15) / 16 * 16; }
 // exp(-i 2 pi m k / (R_{s-1} R_s)) at [m R_{s-1} + k], m < R_s, k < R_{s-1}.
 // The inverse transform runs as conj(DFT(conj(x))) on the same matrices.
 struct P2TcArgs {
-    P2Args a;  // as the FP32 column pass, one spectrum (a.K[0])
+    P2Args a;  // as the FP32 column pass, one spectrum (a.K[0], natural order)
+    TwChain twf, twi;  // forward and reversed chains of the column plan
     const uint4* tables;
     int* err;  // device status word (bit 2: an MMA wait timed out)
     int no_mma;  // test hook: issue no MMA, so the first bounded wait runs out
@@ -484,17 +485,17 @@ __device__ __noinline__ void tc_column(const P2TcArgs& A, int c, TcState& st)
         for (int m = 0; m < R0; ++m) {
             const int row = t + m * NB0;
             const long long off = (NB0 % 2 == 0) ? t_row(t) + m * t_row_step<NB0>() : t_row(row);
-            tc_put<G0>(t, m, row < a.H ? __ldg(col + off) : make_float2(0.f, 0.f));
+            tc_put<G0>(t, m, row < a.H ? col[off] : make_float2(0.f, 0.f));
         }
     }
     {
         const void* kcol = static_cast<const char*>(a.K[0]) + (long long)c * a.ldK * (KREAL ? 4 : 8);
         TcProductSink<N, RL, KREAL, GI0> ps{kcol, t};
-        Fwd::run(st, a.twf, A.err, t, ps);
+        Fwd::run(st, A.twf, A.err, t, ps);
     }
     float2* Uc = u_column(a.U, a.ldU, c);
     TcStoreSink<N, R0> ss{Uc, a.r0, a.Hout, t};
-    Inv::run(st, a.twi, A.err, t, ss);
+    Inv::run(st, A.twi, A.err, t, ss);
     if (a.HoutPad != a.Hout && t == 0) Uc[u_row(a.Hout)] = make_float2(0.f, 0.f);
 }
 

@@ -1,22 +1,22 @@
-"""Autotuner of the FFT plans (radix order and launch shape) per length.
+"""Autotuner of the block transforms' geometry and launch shapes per length.
 
 For each length N it builds small variant libraries that contain only N,
-each with one candidate radix sequence and one setting of the launch knobs
-of the prefetching kernels (work units per block, minimum resident blocks per
-SM, spectrum-column staging), times the three passes of a map whose padded
-size is N x N on the GPU, and keeps, for the fastest radix sequence, the best
-knob setting of each pass, then refines it (double-buffered exchange; with
-several spectra per map, one single-spectrum column pass per spectrum
-against the batched kernel).  The result is written to ``tuned_plans.json``
-beside this file (or to the file $LP_TUNE_CACHE names); ``build.py`` uses
-it for every length it lists.
+each with one candidate factorisation N = R0 R1 R2 and one launch shape of
+the passes (transforms per block, threads, resident blocks per SM), times
+the three passes of a map whose padded size is N x N on the GPU, and keeps,
+for the factorisation whose best passes sum lowest, the best shape of each
+pass.  With several spectra per map it times the shapes of the batched column
+pass (and its groups per block) at that factorisation, against one
+single-spectrum pass per spectrum.  The result is written to
+``tuned_plans.json`` beside this file (or to the file $LP_TUNE_CACHE names)
+as the entry's "geo"; ``build.py`` uses it for every length it lists.
 
     python -m paper_1907_02891_gb300.tune --sizes 4704 [--quick] \
-        [--map-side 4096 --psf 541 --nspec 1] [--plan 21,16,14 ...]
+        [--map-side 4096 --psf 541 --nspec 1]
 
 The passes are timed one by one, with events between them, which stops the
-launch overlap between passes of a real map; check a stored plan on the
-whole map as well (a setting that speeds one pass up can slow the map down).
+launch overlap between passes of a real map; the last step times whole maps
+with the trigger of the next pass at block start and at block exit.
 
 Needs nvcc and one GPU.  Each variant is timed in a fresh subprocess (the
 variant libraries export the same symbols).
@@ -27,18 +27,18 @@ from __future__ import annotations
 import argparse
 import concurrent.futures as cf
 import hashlib
-import itertools
 import json
 import os
 import subprocess
 import sys
 import time
-from typing import Dict, List, Tuple
+from typing import Dict, List, Sequence, Tuple
 
 from . import build as B
 
 TUNE_DIR = os.path.join(B.OUT, "tune")
 COMMON_SRCS = ("api.cu", "spectrum.cu", "noalloc.cu", "serve.cpp")
+PASSES = ("p1_rows", "p2_cols", "p3_rows")
 
 
 def _prod(p) -> int:
@@ -48,59 +48,60 @@ def _prod(p) -> int:
     return r
 
 
-def candidate_plans(n: int, limit: int = 3) -> List[Tuple[int, ...]]:
-    """Radix sequences ordered like build.choose_plan, then the other orders
-    of the same multisets (first radix odd / large first)."""
-    scored = []
-    for f in B.factorizations(n):
-        if B.threads_for(n, f) > B.MAX_THREADS:
+def candidate_shapes(r: Sequence[int], limit: int, parked: bool = False) -> List[List[int]]:
+    """Launch shapes [transforms per block, threads, resident blocks] of a
+    factorisation, by the share of idle threads in their rounds and the
+    resident threads per SM; parked: with a parked column beside the working
+    set (the batched column pass)."""
+    r0, r1, r2 = r
+    n, g = _prod(r), B.lanes_for(r1, r2)
+    out = []
+    for nt in ((4, 8, 16) if n <= 256 else (1, 2, 4, 8) if n <= 1024 else (1, 2, 4) if n <= 2600 else
+               (1, 2) if n <= 6200 else (1,)):
+        smem = B.pass_smem(r, nt) + (8 * nt * n if parked else 0)
+        if smem > B.SMEM_LIMIT:
             continue
-        scored.append(((len(f), max(f), -min(f)), f))
-    scored.sort()
-    out: List[Tuple[int, ...]] = []
-    for _, f in scored:
-        for perm in (tuple(sorted(f, reverse=True)), tuple(sorted(f))):
-            if perm not in out:
-                out.append(perm)
-        if len(out) >= limit:
-            break
-    return out[:limit]
+        for w in range(1, 33):
+            t = 32 * w
+            if r0 == 1:
+                if t % g or nt % (t // g):
+                    continue
+                waste = 1.0
+            else:
+                if not 8 <= n * nt / t <= 48:
+                    continue
+                u1, ub, gr = r1 * r2 * nt, r0 * nt, w * (32 // g)
+                waste = (-(-u1 // t) * t / u1 + 2.0 * (-(-ub // gr) * gr / ub)) / 3
+            for regs in (2 * max(r) + 14, 2 * max(r) + 38):
+                regs = (regs + 7) // 8 * 8
+                mb = max(1, min((228 * 1024) // (smem + 1024), 65536 // (t * regs), 16))
+                out.append((waste * (1 + 300.0 / min(mb * t, 2048)), [nt, t, mb]))
+    out.sort(key=lambda x: x[0])
+    res: List[List[int]] = []
+    for _, s in out:
+        if s not in res:
+            res.append(s)
+    return res[:limit]
 
 
 def _compile_common(jobs: int) -> List[str]:
     os.makedirs(os.path.join(TUNE_DIR, "common"), exist_ok=True)
     deps = max(os.path.getmtime(h) for h in B._headers())
     srcs = [os.path.join(B.CSRC, f) for f in COMMON_SRCS]
-    objs = []
     with cf.ThreadPoolExecutor(jobs) as ex:
-        objs = list(ex.map(lambda s: B._compile(s, deps), srcs))
-    return objs
+        return list(ex.map(lambda s: B._compile(s, deps), srcs))
 
 
 def _variant_lib(n: int, plan: dict, common: List[str]) -> str:
-    key = json.dumps([n, plan], sort_keys=True)
-    vid = hashlib.sha1(key.encode()).hexdigest()[:12]
+    vid = hashlib.sha1(json.dumps([n, plan], sort_keys=True).encode()).hexdigest()[:12]
     d = os.path.join(TUNE_DIR, vid)
     lib = os.path.join(d, "liblp.so")
     if os.path.exists(lib):
         return lib
     os.makedirs(d, exist_ok=True)
-    r = list(plan["radices"])
-    text = B._SIZE_TU.format(n=n, seq=", ".join(map(str, r)), f1=plan["f1"], f3=plan["f3"], ns=len(r),
-                             tt=plan.get("tt", 0),
-                             upb1=plan["upb"][0], upb2=plan["upb"][1], upb3=plan["upb"][2],
-                             minb1=plan["minb"][0], minb2=plan["minb"][1], minb3=plan["minb"][2],
-                             kstage="true" if plan["kstage"] else "false",
-                             pf1=B._b(plan["pf"][0]), pf2=B._b(plan["pf"][1]), pf3=B._b(plan["pf"][2]),
-                             db1=B._b(plan["db"][0]), db2=B._b(plan["db"][1]), db3=B._b(plan["db"][2]),
-                             batch=B._b(plan.get("batch", True)),
-                             kst2=B._b(plan.get("kst2", False)), packed=int(bool(plan.get("packed", False))),
-                             late1=B._b(plan.get("late", B.DEFAULT_LATE)[0]), late2=B._b(plan.get("late", B.DEFAULT_LATE)[1]),
-                             rad6=", ".join(map(str, r + [0] * (6 - len(r)))))
-    src = os.path.join(d, f"size_{n}.cu")
+    src, reg = os.path.join(d, f"size_{n}.cu"), os.path.join(d, "registry.cu")
     with open(src, "w") as fh:
-        fh.write(text)
-    reg = os.path.join(d, "registry.cu")
+        fh.write(B.size_tu(n, plan))
     with open(reg, "w") as fh:
         fh.write(B._REGISTRY_TU.format(decls=f"extern const SizeKernels kSize_{n};",
                                        ptrs=f"&kSize_{n}", count=1))
@@ -182,177 +183,65 @@ def time_variant(lib: str, n: int, reps: int, side: int = 0, psf: int = 0, nspec
 
 
 def tune_size(n: int, quick: bool, jobs: int, common: List[str], log, side: int = 0, psf: int = 0,
-              nspec: int = 1, plans: List[Tuple[int, ...]] = (), packed: bool = False) -> dict:
-    base = dict(B.plan_table_entry(n), packed=packed)
-    plans = list(plans) or candidate_plans(n, 2 if quick else 3)
-    knobs = []
-    for upb, minb, kst in itertools.product((1, 2, 3), (1, 2, 3), (False, True)):
-        if quick and (minb == 3 and upb == 1):
-            continue
-        if upb == 3 and (quick or kst):
-            continue
-        knobs.append((upb, minb, kst, 1))
-    knobs.append((1, 1, False, 0))   # one-unit-per-block kernels (no prefetch)
-    knobs.append((1, 2, False, 0))
-    knobs.append((1, 3, False, 0))
-    variants = []
-    for r in plans:
-        # threads per transform: one butterfly per thread in every stage (0),
-        # or as many as the stage with the fewest butterflies (whole warps)
-        tts = [0]
-        few = (n // max(r) + 31) // 32 * 32
-        if few < B.threads_for(n, r):
-            tts.append(few)
-        for tt in tts:
-            for upb, minb, kst, pf in knobs:
-                if tt and (kst or not pf):   # staging / no-prefetch only at the default thread count
-                    continue
-                p = dict(base)
-                p.update(radices=list(r), threads=tt or B.threads_for(n, r), upb=[upb] * 3,
-                         minb=[minb] * 3, kstage=kst, tt=tt, pf=[pf] * 3, db=[0, 0, 0])
-                variants.append(p)
-    t0 = time.time()
+              nspec: int = 1) -> dict:
+    base = B.plan_table()[n]
+    reps = 100 if n <= 5200 else 20
 
-    def build_or_error(p):
-        try:
-            return _variant_lib(n, p, common)
-        except RuntimeError as e:  # a variant that does not compile is skipped
-            return e
-
-    with cf.ThreadPoolExecutor(jobs) as ex:
-        libs = list(ex.map(build_or_error, variants))
-    log(f"N={n}: built {sum(isinstance(l, str) for l in libs)} of {len(libs)} variants in {time.time() - t0:.0f} s")
-    results = []
-    for p, lib in zip(variants, libs):
-        if not isinstance(lib, str):
-            log(f"  skip {p['radices']} upb={p['upb'][0]} minb={p['minb'][0]}: build failed: "
-                f"{str(lib).strip().splitlines()[-1][:120]}")
-            continue
-        try:
-            t = time_variant(lib, n, 200 if n <= 5200 else 40, side, psf, nspec)
-        except Exception as e:  # a variant that does not launch (resources) is skipped
-            log(f"  skip {p['radices']} upb={p['upb'][0]} minb={p['minb'][0]} kstage={p['kstage']}: "
-                f"{str(e).splitlines()[-1][:120]}")
-            continue
-        results.append((p, t))
-        log(f"  {p['radices']} tt={p['tt']} pf={p['pf'][0]} upb={p['upb'][0]} minb={p['minb'][0]} kstage={int(p['kstage'])}: "
-            + " ".join(f"{k}={v * 1e3:.1f}us" for k, v in t.items()))
-    if not results:
-        raise RuntimeError(f"no variant of {n} ran")
-    # per (radix plan, threads per transform): best knob per pass; then the
-    # combination with the best total
-    best = None
-    for r, tt in sorted({(tuple(p["radices"]), p["tt"]) for p, _ in results}):
-        rs = [(p, t) for p, t in results if tuple(p["radices"]) == r and p["tt"] == tt]
-        if not rs:
-            continue
-        choice, total = {}, 0.0
-        for k, name in enumerate(("p1_rows", "p2_cols", "p3_rows")):
-            # fastest setting; among those within 1 % of it (a knob the
-            # timed workload does not exercise), the fewest resident blocks
-            # (highest register cap), fewest units per block, no staging
-            tbest = min(t[name] for _, t in rs)
-            near = [(p, t) for p, t in rs if t[name] <= tbest * 1.01]
-            p, t = min(near, key=lambda x: (x[0]["minb"][k], x[0]["upb"][k], x[0]["kstage"], x[1][name]))
-            choice[name] = p
-            total += t[name]
-        if best is None or total < best[0]:
-            best = (total, r, choice, tt)
-    total, r, choice, tt = best
-    out = dict(base)
-    out.update(radices=list(r), threads=tt or B.threads_for(n, r), tt=tt,
-               upb=[choice["p1_rows"]["upb"][0], choice["p2_cols"]["upb"][1], choice["p3_rows"]["upb"][2]],
-               minb=[choice["p1_rows"]["minb"][0], choice["p2_cols"]["minb"][1], choice["p3_rows"]["minb"][2]],
-               kstage=choice["p2_cols"]["kstage"], tuned_total_us=total * 1e3,
-               pf=[choice["p1_rows"]["pf"][0], choice["p2_cols"]["pf"][1], choice["p3_rows"]["pf"][2]])
-    log(f"N={n}: chose {out['radices']} tt={out['tt']} pf={out['pf']} upb={out['upb']} minb={out['minb']} kstage={out['kstage']} "
-        f"(sum of best passes {total * 1e3:.1f} us)")
-    # refinement: double-buffered exchange on top of the choice, with each
-    # resident-block setting; kept per pass where it is faster
-    best_pass = {name: min(t[name] for p, t in results if tuple(p["radices"]) == tuple(out["radices"])
-                           and p["tt"] == out["tt"] and p["upb"][i] == out["upb"][i] and p["pf"][i] == out["pf"][i]
-                           and p["minb"][i] == out["minb"][i] and (i != 1 or p["kstage"] == out["kstage"]))
-                 for i, name in enumerate(("p1_rows", "p2_cols", "p3_rows"))}
-    refine = []
-    for minb in (1, 2, 3):
-        p = dict(out)
-        p.update(db=[1, 1, 1], minb=[minb] * 3)
-        refine.append(p)
-    with cf.ThreadPoolExecutor(jobs) as ex:
-        rlibs = list(ex.map(build_or_error, refine))
-    db, minb = [0, 0, 0], list(out["minb"])
-    for p, lib in zip(refine, rlibs):
-        if not isinstance(lib, str):
-            continue
-        try:
-            t = time_variant(lib, n, 200 if n <= 5200 else 40, side, psf, nspec)
-        except Exception as e:
-            log(f"  skip db=1 minb={p['minb'][0]}: {str(e).splitlines()[-1][:120]}")
-            continue
-        log(f"  db=1 minb={p['minb'][0]}: " + " ".join(f"{k}={v * 1e3:.1f}us" for k, v in t.items()))
-        for i, name in enumerate(("p1_rows", "p2_cols", "p3_rows")):
-            if t[name] < best_pass[name] * 0.99:
-                best_pass[name] = t[name]
-                db[i], minb[i] = 1, p["minb"][0]
-    out.update(db=db, minb=minb, tuned_total_us=sum(best_pass.values()) * 1e3)
-    log(f"N={n}: refined db={db} minb={minb} (sum {out['tuned_total_us']:.1f} us)")
-    # packed FP32x2 DFT arithmetic: one switch for the whole length (its
-    # constants take registers, which can make a register-capped kernel
-    # spill); kept where all three passes together are faster
-    p = dict(out, packed=not out.get("packed", False))
-    lib = build_or_error(p)
-    if isinstance(lib, str):
-        try:
-            t = time_variant(lib, n, 200 if n <= 5200 else 40, side, psf, nspec)
-            log(f"  packed={int(p['packed'])}: " + " ".join(f"{k}={v * 1e3:.1f}us" for k, v in t.items()))
-            if sum(t.values()) < sum(best_pass.values()) * 0.99:
-                best_pass = dict(t)
-                out.update(packed=p["packed"], tuned_total_us=sum(best_pass.values()) * 1e3)
-        except Exception as e:
-            log(f"  skip packed={int(p['packed'])}: {str(e).splitlines()[-1][:120]}")
-    log(f"N={n}: packed={out.get('packed', False)}")
-    # whole-map refinement: the pass timings above stop the launch overlap
-    # between passes, which decides the trigger point and interacts with the
-    # forward row pass's resident blocks; time whole maps of the choice and
-    # of those neighbours, keep the fastest
-    reps = 200 if n <= 5200 else 40
-    late0 = list(out.get("late", B.DEFAULT_LATE))
-    cands = [dict(out, late=late0), dict(out, late=[0, 0, 0])]
-    m1 = out["minb"][0]
-    for mb in (m1 - 1, m1 + 1):
-        if 1 <= mb <= 3:
-            cands.append(dict(out, late=late0, minb=[mb] + list(out["minb"][1:])))
-    best_map = None
-    for p in cands:
-        lib = build_or_error(p)
-        if not isinstance(lib, str):
-            continue
-        try:
-            ms = min(time_variant(lib, n, reps, side, psf, nspec, whole=True)["map"] for _ in range(2))
-        except Exception as e:
-            log(f"  skip whole map late={p['late']} minb={p['minb']}: {str(e).splitlines()[-1][:120]}")
-            continue
-        log(f"  whole map late={p['late']} minb={p['minb']}: {ms * 1e3:.1f} us")
-        if best_map is None or ms < best_map[0] * 0.995:
-            best_map = (ms, p)
-    if best_map is not None:
-        out.update(late=best_map[1]["late"], minb=best_map[1]["minb"], tuned_map_us=best_map[0] * 1e3)
-    log(f"N={n}: late={out.get('late')} minb={out['minb']} (whole map {out.get('tuned_map_us', 0):.1f} us)")
-    if nspec > 1:
-        # several spectra: the batched column kernel against one single-
-        # spectrum pass per spectrum
-        p = dict(out, batch=False)
-        lib = build_or_error(p)
-        if isinstance(lib, str):
+    def run(plans, whole=False, ns=1):
+        """[(plan, timing)] of the plans that build and launch."""
+        def lib_or_error(p):
             try:
-                t = time_variant(lib, n, 200 if n <= 5200 else 40, side, psf, nspec)
-                log(f"  batch=0: " + " ".join(f"{k}={v * 1e3:.1f}us" for k, v in t.items()))
-                if t["p2_cols"] < best_pass["p2_cols"] * 0.99:
-                    best_pass["p2_cols"] = t["p2_cols"]
-                    out.update(batch=False, tuned_total_us=sum(best_pass.values()) * 1e3)
-            except Exception as e:
-                log(f"  skip batch=0: {str(e).splitlines()[-1][:120]}")
-        log(f"N={n}: batch={out.get('batch', True)} (sum {out['tuned_total_us']:.1f} us)")
+                return _variant_lib(n, p, common)
+            except RuntimeError as e:
+                return e
+        t0 = time.time()
+        with cf.ThreadPoolExecutor(jobs) as ex:
+            libs = list(ex.map(lib_or_error, plans))
+        log(f"N={n}: built {sum(isinstance(l, str) for l in libs)} of {len(libs)} variants in {time.time() - t0:.0f} s")
+        got = []
+        for p, lib in zip(plans, libs):
+            try:
+                if not isinstance(lib, str):
+                    raise lib
+                t = time_variant(lib, n, reps, side, psf, ns, whole)
+            except Exception as e:  # a variant that does not build or launch (resources) is skipped
+                log(f"  skip {p['geo']}: {str(e).strip().splitlines()[-1][:120]}")
+                continue
+            got.append((p, t))
+            log(f"  {p['geo']['r']} {p['geo']['p1']} pm={p['geo']['pm']}x{p['geo']['grp']} packed={int(p['packed'])} "
+                f"late={p.get('late')}: " + " ".join(f"{k}={v * 1e3:.1f}us" for k, v in t.items()))
+        return got
+
+    plans = []
+    for r in B.candidate_geos(n)[:2 if quick else 5]:
+        for s in candidate_shapes(r, 4 if quick else 8):
+            plans.append(dict(base, packed=True, geo=dict(B.geo_plan(r), p1=s, p2=s, p3=s)))
+    got = run(plans)
+    if not got:
+        raise RuntimeError(f"no variant of {n} ran")
+    best = None
+    for r in {tuple(p["geo"]["r"]) for p, _ in got}:
+        rs = [(p, t) for p, t in got if tuple(p["geo"]["r"]) == r]
+        pick = [min(rs, key=lambda x, k=k: x[1][k]) for k in PASSES]
+        total = sum(t[k] for k, (_, t) in zip(PASSES, pick))
+        if best is None or total < best[0]:
+            best = (total, r, [p["geo"][k] for k, (p, _) in zip(("p1", "p2", "p3"), pick)])
+    total, r, (s1, s2, s3) = best
+    out = dict(base, packed=True, geo=dict(B.geo_plan(r), p1=s1, p2=s2, p3=s3))
+    # packed FP32x2 arithmetic, and the trigger of the next pass: whole maps
+    late = list(base.get("late", B.DEFAULT_LATE))
+    whole = run([dict(out, packed=pk, late=l) for pk in (True, False) for l in (late, [0, 0, 0])], whole=True)
+    pick = min(whole, key=lambda x: x[1]["map"])
+    out = dict(pick[0], tuned_total_us=total * 1e3, tuned_map_us=pick[1]["map"] * 1e3)
+    if nspec > 1:
+        multi = [dict(out, batch=False)]
+        for s in candidate_shapes(r, 4 if quick else 8, parked=True):
+            for grp in (1, 2, 3):
+                if s[1] * grp <= 1024:
+                    multi.append(dict(out, batch=True, geo=dict(out["geo"], pm=s, grp=grp)))
+        out = min(run(multi, ns=nspec), key=lambda x: x[1]["p2_cols"])[0]
+    log(f"N={n}: chose {out['geo']} packed={out['packed']} late={out.get('late')} batch={out.get('batch')} "
+        f"(passes {out['tuned_total_us']:.1f} us, map {out['tuned_map_us']:.1f} us)")
     return out
 
 
@@ -364,15 +253,11 @@ def main() -> None:
     ap.add_argument("--out", default=B.tuned_json_path(),
                     help="plan file to update (default: $LP_TUNE_CACHE, else tuned_plans.json)")
     ap.add_argument("--log", default=None)
-    ap.add_argument("--plan", action="append", default=[],
-                    help="radix sequence to try, e.g. 7,7,8,12 (repeatable; default: the candidate list)")
     ap.add_argument("--psf", type=int, default=0, help="PSF side of the timed maps (default min(541, N/8))")
     ap.add_argument("--nspec", type=int, default=1, help="spectra per timed map (one forward transform)")
     ap.add_argument("--map-side", type=int, default=0,
                     help="time maps of this side instead of N - PSF + 1, to compare "
                          "padded lengths for one workload")
-    ap.add_argument("--packed", action="store_true",
-                    help="search the knobs with packed FP32x2 arithmetic (the last step still tries both)")
     args = ap.parse_args()
     jobs = args.jobs or (os.cpu_count() or 1)
     logf = open(args.log, "a") if args.log else None
@@ -386,18 +271,13 @@ def main() -> None:
     for n in args.sizes:
         if n not in B.SIZES:
             raise SystemExit(f"{n} is not in the supported size list")
-    plans = [tuple(int(x) for x in p.split(",")) for p in args.plan]
-    for p in plans:
-        if len(args.sizes) != 1 or _prod(p) != args.sizes[0] or max(p) > 32:
-            raise SystemExit(f"plan {p} is not a radix sequence of length {args.sizes}")
     common = _compile_common(jobs)
     table = {}
     if os.path.exists(args.out):
         with open(args.out) as fh:
             table = json.load(fh)
     for n in args.sizes:
-        table[str(n)] = tune_size(n, args.quick, jobs, common, log, args.map_side, args.psf, args.nspec, plans,
-                                  args.packed)
+        table[str(n)] = tune_size(n, args.quick, jobs, common, log, args.map_side, args.psf, args.nspec)
         table[str(n)]["tuned_on"] = {"map_side": args.map_side, "psf": args.psf, "nspec": args.nspec}
         with open(args.out, "w") as fh:
             json.dump(table, fh, indent=1, sort_keys=True)
