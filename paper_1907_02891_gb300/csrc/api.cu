@@ -81,8 +81,9 @@ extern "C" int lp_supported_size(int n)
 static SpecOrder spectrum_order(int ny, lp_precision prec)
 {
     const SizeKernels* k = find_size(ny);
-    if (!k || prec != LP_PREC_FP32) return SpecOrder{0, 0, 0, 0};
-    return SpecOrder{k->geo[0], k->geo[1], k->geo[2], k->vk};
+    if (!k || prec != LP_PREC_FP32) return SpecOrder{};
+    const auto inv = [](int r) { return (unsigned)((((1ull << 32) + r - 1) / r) & 0xffffffffull); };
+    return SpecOrder{k->geo[0], k->geo[1], k->geo[2], k->vk, inv(k->geo[0]), inv(k->geo[1])};
 }
 
 extern "C" int lp_split_supported(int n)
@@ -572,8 +573,7 @@ extern "C" lp_status lp_kernel_spectrum(lp_ctx* ctx, const double* K, int hk, in
     unsigned long long* d_fp = nullptr;
     CUDA_TRY(cudaMallocAsync((void**)&d_fp, 24, st));
     CUDA_TRY(cudaMemsetAsync(d_fp, 0, 24, st));
-    CUDA_TRY(psf_fingerprint_launch(K, (long long)hk * wk, d_fp, st));
-    CUDA_TRY(psf_symmetry_launch(K, hk, wk, reinterpret_cast<int*>(d_fp + 1), st));
+    CUDA_TRY(psf_inspect_launch(K, (long long)hk * wk, d_fp, reinterpret_cast<int*>(d_fp + 1), st));
     unsigned long long host_fp[2] = {0, 0};
     CUDA_TRY(cudaMemcpyAsync(host_fp, d_fp, 16, cudaMemcpyDeviceToHost, st));
     CUDA_TRY(cudaStreamSynchronize(st));
@@ -661,22 +661,19 @@ extern "C" lp_status lp_kernel_spectrum(lp_ctx* ctx, const double* K, int hk, in
         return lp_fail(sa, "%s", msg.c_str());
     }
     // FP64 scratch, stream-ordered, released right after the build
-    const size_t w1 = sizeof(double2) * (size_t)hk * Nx;
-    const size_t w2 = sizeof(double2) * (size_t)Ny * ncols;
-    char* scratch = nullptr;
-    cudaError_t e = cudaMallocAsync((void**)&scratch, 2 * w1 + 2 * w2, st);
+    const size_t scratch_bytes = psf_scratch_bytes(hk, wk, Ny, Nx, is_real);
+    void* scratch = nullptr;
+    cudaError_t e = cudaMallocAsync(&scratch, scratch_bytes, st);
     if (e != cudaSuccess) {
         cudaGetLastError();
         cudaFreeAsync(d_fp, st);
         discard(spec);
-        return lp_fail(LP_ERR_OOM, "spectrum scratch (%zu bytes): %s", 2 * w1 + 2 * w2, cudaGetErrorString(e));
+        return lp_fail(LP_ERR_OOM, "spectrum scratch (%zu bytes): %s", scratch_bytes, cudaGetErrorString(e));
     }
     e = cudaMemcpyAsync(spec->kcopy, K, spec->kbytes, cudaMemcpyDeviceToDevice, st);
-    if (e == cudaSuccess) e = cudaMemsetAsync(dptr, 0, bytes, st);
+    // (columns end in padding up to ldK, which nothing reads)
     if (e == cudaSuccess)
-        e = psf_spectrum_build(K, hk, wk, Ny, Nx, is_real, dptr, ldK, spectrum_order(Ny, prec), (double2*)scratch,
-                               (double2*)(scratch + w1), (double2*)(scratch + 2 * w1),
-                               (double2*)(scratch + 2 * w1 + w2), st);
+        e = psf_spectrum_build(K, hk, wk, Ny, Nx, is_real, dptr, ldK, spectrum_order(Ny, prec), scratch, st);
     cudaFreeAsync(scratch, st);
     for (int i = 0; e == cudaSuccess && i < lp_spectrum::kUseSlots; ++i)
         e = cudaEventCreateWithFlags(&spec->use_event[i], cudaEventDisableTiming);

@@ -59,18 +59,18 @@ extern const int kNumSizes;
 // (r0 = 0: natural order).
 struct SpecOrder {
     int r0, r1, r2, vk;
+    unsigned inv0, inv1;  // ceil(2^32 / r0), ceil(2^32 / r1) (r > 1): quotients by multiplication
 };
 
 // FP64 spectrum pipeline (spectrum.cu)
 bool fft64_supported(int N);
-cudaError_t psf_fingerprint_launch(const double* K, long long n, unsigned long long* d_out,
-                                   cudaStream_t st);
-cudaError_t psf_symmetry_launch(const double* K, int hk, int wk, int* d_asym, cudaStream_t st);
+// *d_out += the fingerprint of K's n values, *d_asym |= 1 where K is not point-symmetric
+cudaError_t psf_inspect_launch(const double* K, long long n, unsigned long long* d_out, int* d_asym, cudaStream_t st);
 // *d_diff |= 1 where a[i] and b[i] differ in any bit (i < n)
 cudaError_t psf_compare_launch(const double* a, const double* b, long long n, int* d_diff, cudaStream_t st);
-cudaError_t psf_spectrum_build(const double* K, int hk, int wk, int Ny, int Nx, int real_only,
-                               void* dst, long long ldK, SpecOrder order, double2* W1, double2* W1b,
-                               double2* W2a, double2* W2b, cudaStream_t st);
+size_t psf_scratch_bytes(int hk, int wk, int Ny, int Nx, int real_only);
+cudaError_t psf_spectrum_build(const double* K, int hk, int wk, int Ny, int Nx, int real_only, void* dst, long long ldK,
+                               SpecOrder order, void* scratch, cudaStream_t st);
 // a stored spectrum's columns in natural order, packed (ny values each)
 cudaError_t spectrum_copy_natural(const void* data, long long ldK, int ny, int ncols, int is_real, SpecOrder order,
                                   float* dst, cudaStream_t st);

@@ -7,179 +7,258 @@
 // the circular convolution of Sec. 2.5 needs no crop offset for the
 // same-size output, and the spectrum of a point-symmetric PSF is real.
 //
-// Pipeline (all on the caller's stream, FP64):
-//   scatter rows of K into hk x Nx (wrap in x)  ->  FFT along x
-//   scatter the first Nx/2+1 columns into Ny x (Nx/2+1) (wrap in y)  ->  FFT along y
-//   scale by 1/(2 Ny Nx) and store transposed as FP32: real part only when
-//   the PSF is point-symmetric (exact compare), complex otherwise.
-// The FFT is a global-memory Stockham pass per radix (2, 3, 4, 5, 7, 8)
-// with FP64 twiddles from sincospi; it is off the per-map hot path.
+// Pipeline (all on the caller's stream, FP64; the card's FP64 rate, two
+// multiply-adds per SM and clock, is what bounds it, so every step is there
+// to spend fewer of them):
+//   * two real rows of K share one complex row transform; of a
+//     point-symmetric K only the rows y >= 0 are transformed (row -y is the
+//     conjugate of row y);
+//   * the columns of a point-symmetric K have real transforms, so two of
+//     them share one complex transform;
+//   * a transform of length N = R M of k < N non-zero samples is, per residue
+//     m < R, the M-point transform of the samples times exp(-i 2 pi n m / N)
+//     folded modulo M: X[m + R k'] = sum_j w_M^{j k'} sum_{n = j mod M} x[n]
+//     w_N^{n m}.  R is chosen so that the folding and the M-point transform
+//     cost least (fft64_split); one block per (transform, m), in place in
+//     shared memory;
+//   * twiddles come from a table of N values made once per build; sincospi
+//     per element and stage had taken most of the build's time.
+// For the 541 x 541 PSF at 4704 x 4704 the transforms took 4.3 ms as one
+// global-memory pass per radix, and the fingerprint 0.19 ms with an atomic
+// per PSF value.
 #include "fft_core.cuh"
 #include "lp_internal.h"
 
 namespace lpk {
 
-template <int R, int DIR>
-__global__ void fft64_stage(const double2* __restrict__ in, double2* __restrict__ out, int N,
-                            int Ns, long long es, long long bs, int nb, int batch_fast)
-{
-    const long long NB = N / R;
-    const long long g = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (g >= NB * nb) return;
-    long long j, b;
-    if (batch_fast) {
-        b = g % nb;
-        j = g / nb;
-    } else {
-        j = g % NB;
-        b = g / NB;
-    }
-    double2 v[R];
-#pragma unroll
-    for (int m = 0; m < R; ++m) v[m] = in[b * bs + (j + m * NB) * es];
-    const long long k = j % Ns;
-    if (Ns > 1) {
-        const long long n = (long long)Ns * R;
-#pragma unroll
-        for (int m = 1; m < R; ++m) {
-            const long long tt = (k * m) % n;
-            double s, c;
-            sincospi(2.0 * (double)tt / (double)n, &s, &c);
-            v[m] = cmul(v[m], mk<double2>(c, DIR * s));
-        }
-    }
-    Dft<R, DIR, double2>::run(v);
-    const long long base = (j / Ns) * Ns * R + k;
-#pragma unroll
-    for (int m = 0; m < R; ++m) out[b * bs + (base + m * Ns) * es] = v[m];
-}
+constexpr int kMaxStages64 = 16;
+constexpr int kMaxM64 = 4608;  // points of one in-place transform: 72 KB, three blocks per SM
+
+// An M-point transform in shared memory: radices in stage order
+struct Fft64 {
+    int N, R, M, ns;
+    int radix[kMaxStages64];
+};
 
 static int pick_radix64(int rem)
 {
-    if (rem % 8 == 0) return 8;
-    if (rem % 4 == 0) return 4;
-    if (rem % 2 == 0) return 2;
-    if (rem % 3 == 0) return 3;
-    if (rem % 5 == 0) return 5;
-    if (rem % 7 == 0) return 7;
+    for (int r : {8, 4, 2, 3, 5, 7})
+        if (rem % r == 0) return r;
     return 0;
 }
 
-template <int DIR>
-static cudaError_t launch_stage64(int R, const double2* in, double2* out, int N, int Ns,
-                                  long long es, long long bs, int nb, int batch_fast,
-                                  cudaStream_t st)
+static int fft64_stages(int n, int* radix)
 {
-    const long long total = (long long)(N / R) * nb;
-    const int thr = 256;
-    const unsigned blocks = (unsigned)((total + thr - 1) / thr);
-    switch (R) {
-    case 2: fft64_stage<2, DIR><<<blocks, thr, 0, st>>>(in, out, N, Ns, es, bs, nb, batch_fast); break;
-    case 3: fft64_stage<3, DIR><<<blocks, thr, 0, st>>>(in, out, N, Ns, es, bs, nb, batch_fast); break;
-    case 4: fft64_stage<4, DIR><<<blocks, thr, 0, st>>>(in, out, N, Ns, es, bs, nb, batch_fast); break;
-    case 5: fft64_stage<5, DIR><<<blocks, thr, 0, st>>>(in, out, N, Ns, es, bs, nb, batch_fast); break;
-    case 7: fft64_stage<7, DIR><<<blocks, thr, 0, st>>>(in, out, N, Ns, es, bs, nb, batch_fast); break;
-    case 8: fft64_stage<8, DIR><<<blocks, thr, 0, st>>>(in, out, N, Ns, es, bs, nb, batch_fast); break;
-    default: return cudaErrorInvalidValue;
+    int ns = 0;
+    while (n > 1) {
+        const int r = pick_radix64(n);
+        if (r == 0 || ns == kMaxStages64) return -1;
+        if (radix) radix[ns] = r;
+        ++ns;
+        n /= r;
     }
-    return cudaGetLastError();
+    return ns;
 }
 
-// Forward FFT of nb transforms of length N; element stride es, batch stride
-// bs (elements).  Ping-pongs between a and tmp; *result gets the buffer that
-// holds the output.
-cudaError_t fft64_forward(double2* a, double2* tmp, int N, long long es, long long bs, int nb,
-                          int batch_fast, cudaStream_t st, double2** result)
+bool fft64_supported(int N) { return N >= 1 && fft64_stages(N, nullptr) >= 0; }
+
+// Split N = R M for k non-zero samples: the fewest FP64 instructions per
+// output (butterflies and twiddles by prime factor, four per folded sample),
+// with M points (16 bytes each) in at most 72 KB of shared memory, and enough
+// of them to fill a block.
+static Fft64 fft64_split(int N, int k)
 {
-    double2* src = a;
-    double2* dst = tmp;
-    int Ns = 1, rem = N;
-    while (rem > 1) {
-        const int R = pick_radix64(rem);
-        if (R == 0) return cudaErrorInvalidValue;
-        cudaError_t e = launch_stage64<-1>(R, src, dst, N, Ns, es, bs, nb, batch_fast, st);
-        if (e != cudaSuccess) return e;
-        Ns *= R;
-        rem /= R;
-        double2* x = src;
-        src = dst;
-        dst = x;
+    Fft64 best{};
+    double best_cost = 0.0;
+    for (int R = 1; R <= N; ++R) {
+        if (N % R != 0 || N / R > kMaxM64 || (N / R < 192 && R > 1)) continue;
+        Fft64 f{N, R, N / R, 0, {}};
+        f.ns = fft64_stages(f.M, f.radix);
+        if (f.ns < 0) continue;
+        double cost = 4.0 * (double)k / f.M;
+        for (int s = 0; s < f.ns; ++s) {
+            const int r = f.radix[s];
+            cost += 4.0 * (r - 1) / r + (r == 8 ? 6.5 : r == 4 ? 4.0 : r == 2 ? 2.0 : r == 3 ? 4.7 : r == 5 ? 7.2 : 9.4);
+        }
+        if (best.N == 0 || cost < best_cost) {
+            best = f;
+            best_cost = cost;
+        }
     }
-    *result = src;
-    return cudaSuccess;
+    return best;
 }
 
-bool fft64_supported(int N)
+// table[t] = exp(-i 2 pi t / N), t < N, and perm[p] = the frequency k' that
+// the in-place stages leave at position p of M
+__global__ void fft64_tables(Fft64 f, double2* table, unsigned short* perm)
 {
-    int rem = N;
-    while (rem > 1) {
-        const int R = pick_radix64(rem);
-        if (R == 0) return false;
-        rem /= R;
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t < f.N) {
+        double s, c;
+        sincospi(2.0 * (double)t / (double)f.N, &s, &c);
+        table[t] = mk<double2>(c, -s);
     }
-    return N >= 1;
+    if (t < f.M) {
+        int L = f.M, p = t, k = 0, w = 1;
+        for (int s = 0; s < f.ns; ++s) {
+            L /= f.radix[s];
+            const int d = p / L;
+            p -= d * L;
+            k += d * w;
+            w *= f.radix[s];
+        }
+        perm[t] = (unsigned short)k;
+    }
 }
 
-__global__ void psf_symmetry(const double* __restrict__ K, int hk, int wk, int* asym)
+// one decimation-in-frequency stage on blocks of length L: outputs m of
+// butterfly j to sub-block m, times w_L^{j m} = table[j m N / L]
+template <int R>
+__device__ __forceinline__ void stage64(double2* sm, int M, int L, int N, const double2* __restrict__ table)
 {
-    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= (long long)hk * wk) return;
-    const int y = (int)(i / wk), x = (int)(i % wk);
-    if (K[i] != K[(long long)(hk - 1 - y) * wk + (wk - 1 - x)]) atomicOr(asym, 1);
+    const int S = L / R, step = N / L;
+    for (int b = threadIdx.x; b < M / R; b += blockDim.x) {
+        const int g = b / S, j = b - g * S;
+        double2* x = sm + g * L + j;
+        double2 v[R];
+#pragma unroll
+        for (int q = 0; q < R; ++q) v[q] = x[q * S];
+        Dft<R, -1, double2>::run(v);
+        x[0] = v[0];
+#pragma unroll
+        for (int m = 1; m < R; ++m) x[m * S] = S > 1 ? cmul(v[m], __ldg(table + j * m * step)) : v[m];
+    }
+    __syncthreads();
 }
 
-__global__ void psf_scatter_rows(const double* __restrict__ K, int hk, int wk, int Nx, int cx,
-                                 double2* __restrict__ W1)
+__device__ __forceinline__ void fft64_inplace(double2* sm, const Fft64& f, const double2* __restrict__ table)
 {
-    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= (long long)hk * wk) return;
-    const int y = (int)(i / wk), x = (int)(i % wk);
-    int xx = x - cx;
-    if (xx < 0) xx += Nx;
-    W1[(long long)y * Nx + xx] = mk<double2>(K[i], 0.0);
+    int L = f.M;
+    for (int s = 0; s < f.ns; ++s) {
+        switch (f.radix[s]) {
+        case 2: stage64<2>(sm, f.M, L, f.N, table); break;
+        case 3: stage64<3>(sm, f.M, L, f.N, table); break;
+        case 4: stage64<4>(sm, f.M, L, f.N, table); break;
+        case 5: stage64<5>(sm, f.M, L, f.N, table); break;
+        case 7: stage64<7>(sm, f.M, L, f.N, table); break;
+        default: stage64<8>(sm, f.M, L, f.N, table); break;
+        }
+        L /= f.radix[s];
+    }
 }
 
-__global__ void psf_scatter_cols(const double2* __restrict__ W1, int hk, int Nx, int ncols,
-                                 int Ny, int cy, double2* __restrict__ W2)
+// bin j of the folded input: samples i of the window (position i - c) with
+// i - c = j mod M, times w_N^{(i - c) m}
+template <class Sample>
+__device__ __forceinline__ double2 fold64(const Fft64& f, const double2* __restrict__ table, int j, int m, int k, int c,
+                                          Sample&& sample)
 {
-    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= (long long)hk * ncols) return;
-    const int y = (int)(i / ncols), c = (int)(i % ncols);
-    int yy = y - cy;
-    if (yy < 0) yy += Ny;
-    W2[(long long)yy * ncols + c] = W1[(long long)y * Nx + c];
+    double2 acc = mk<double2>(0.0, 0.0);
+    for (int i = (j + c) % f.M; i < k; i += f.M) {
+        const double2 x = sample(i);
+        const int n = i - c < 0 ? i - c + f.N : i - c;
+        const double2 w = __ldg(table + (int)((long long)n * m % f.N));
+        acc.x = fma(x.x, w.x, fma(-x.y, w.y, acc.x));
+        acc.y = fma(x.x, w.y, fma(x.y, w.x, acc.y));
+    }
+    return acc;
+}
+
+extern __shared__ __align__(16) double2 sm64[];
+
+// Row pair p (rows y0 + 2p, y0 + 2p + 1 of K packed as a + i b), residue m
+// = blockIdx.x: frequencies m + R k' to W[p][.].
+__global__ void __launch_bounds__(256) psf_rows(const double* __restrict__ K, int hk, int wk, int y0, Fft64 f,
+                                                const double2* __restrict__ table, const unsigned short* __restrict__ perm,
+                                                double2* __restrict__ W)
+{
+    const int m = blockIdx.x, p = blockIdx.y;
+    const int ya = y0 + 2 * p;
+    const double* a = K + (long long)ya * wk;
+    const bool vb = ya + 1 < hk;
+    for (int j = threadIdx.x; j < f.M; j += blockDim.x)
+        sm64[j] = fold64(f, table, j, m, wk, (wk - 1) / 2, [&](int i) { return mk<double2>(a[i], vb ? a[wk + i] : 0.0); });
+    __syncthreads();
+    fft64_inplace(sm64, f, table);
+    double2* dst = W + (long long)p * f.N + m;
+    for (int t = threadIdx.x; t < f.M; t += blockDim.x) dst[(long long)f.R * perm[t]] = sm64[t];
+}
+
+// G_y[c] from the packed row transforms: rows a = 2p, b = 2p + 1 of pair p,
+// G_a = (Z[c] + conj Z[N-c]) / 2, G_b = -i (Z[c] - conj Z[N-c]) / 2
+__device__ __forceinline__ double2 row_spectrum(const double2* __restrict__ W, int Nx, int r, int c)
+{
+    const double2* row = W + (long long)(r >> 1) * Nx;
+    const double2 z = row[c], zm = row[c == 0 ? 0 : Nx - c];
+    return (r & 1) ? mk<double2>(0.5 * (z.y + zm.y), -0.5 * (z.x - zm.x)) : mk<double2>(0.5 * (z.x + zm.x), 0.5 * (z.y - zm.y));
 }
 
 // position of frequency u in a spectrum column (SpecOrder)
 __device__ __forceinline__ int spec_pos(SpecOrder o, int u)
 {
     if (o.r0 == 0) return u;
-    const int m = u % o.r0, k = u / o.r0;
-    const int k1 = k % o.r1, k2 = k / o.r1;
-    return ((m * (o.r2 / o.vk) + k2 / o.vk) * o.r1 + k1) * o.vk + k2 % o.vk;
+    // (u r < 2^32, so the high half of u ceil(2^32 / r) is u / r)
+    const int k = o.r0 > 1 ? (int)__umulhi((unsigned)u, o.inv0) : u, m = u - k * o.r0;
+    const int k2 = (int)__umulhi((unsigned)k, o.inv1), k1 = k - k2 * o.r1;
+    const int run = o.vk == 4 ? k2 >> 2 : o.vk == 2 ? k2 >> 1 : k2;
+    return ((m * (o.vk == 4 ? o.r2 >> 2 : o.vk == 2 ? o.r2 >> 1 : o.r2) + run) * o.r1 + k1) * o.vk + (k2 & (o.vk - 1));
 }
 
-// dst[c][pos(u)] = scale * W2[u][c], 32 x 32 tiles through shared memory
-__global__ void psf_store_spectrum(const double2* __restrict__ W2, int Ny, int ncols, double scale,
-                                   int real_only, void* dst, long long ldK, SpecOrder order)
+// Inputs of the column transforms, transposed: unit u's samples i < hk at
+// X[u hk + i].  SYM (point-symmetric K): the unit is columns c = 2u and c + 1
+// packed as G_c + i G_{c+1}, W holds the rows y >= 0, and G_{-y} = conj G_y.
+// Else the unit is column u, and W holds all rows.
+template <bool SYM>
+__global__ void __launch_bounds__(256) psf_pack(const double2* __restrict__ W, int hk, int Nx, int ncols, int units,
+                                                double2* __restrict__ X)
 {
     __shared__ double2 tile[32][33];
-    const int u0 = blockIdx.y * 32, c0 = blockIdx.x * 32;
-    for (int r = threadIdx.y; r < 32; r += blockDim.y) {
-        const int u = u0 + r, c = c0 + threadIdx.x;
-        if (u < Ny && c < ncols) tile[r][threadIdx.x] = W2[(long long)u * ncols + c];
+    const int u0 = blockIdx.x * 32, i0 = blockIdx.y * 32, cy = (hk - 1) / 2;
+    for (int q = threadIdx.y; q < 32; q += 8) {
+        const int i = i0 + q, u = u0 + threadIdx.x;
+        if (i >= hk || u >= units) continue;
+        if constexpr (SYM) {
+            const int r = i < cy ? cy - i : i - cy, c = 2 * u;
+            double2 g = row_spectrum(W, Nx, r, c);
+            double2 h = c + 1 < ncols ? row_spectrum(W, Nx, r, c + 1) : mk<double2>(0.0, 0.0);
+            if (i < cy) {
+                g.y = -g.y;
+                h.y = -h.y;
+            }
+            tile[q][threadIdx.x] = mk<double2>(g.x - h.y, g.y + h.x);
+        } else {
+            tile[q][threadIdx.x] = row_spectrum(W, Nx, i, u);
+        }
     }
     __syncthreads();
-    for (int r = threadIdx.y; r < 32; r += blockDim.y) {
-        const int c = c0 + r, u = u0 + threadIdx.x;
-        if (u < Ny && c < ncols) {
-            const double2 z = tile[threadIdx.x][r];
-            const int p = spec_pos(order, u);
-            if (real_only)
-                static_cast<float*>(dst)[(long long)c * ldK + p] = (float)(z.x * scale);
-            else
-                static_cast<float2*>(dst)[(long long)c * ldK + p] =
-                    make_float2((float)(z.x * scale), (float)(z.y * scale));
+    for (int q = threadIdx.y; q < 32; q += 8) {
+        const int u = u0 + q, i = i0 + threadIdx.x;
+        if (i < hk && u < units) X[(long long)u * hk + i] = tile[threadIdx.x][q];
+    }
+}
+
+// Column transforms of unit blockIdx.y, residue m = blockIdx.x.  SYM: the real
+// and imaginary parts of the result are the real spectra of columns 2u, 2u + 1.
+template <bool SYM>
+__global__ void __launch_bounds__(256) psf_cols(const double2* __restrict__ X, int hk, int ncols, Fft64 f,
+                                                const double2* __restrict__ table, const unsigned short* __restrict__ perm,
+                                                double scale, void* dst, long long ldK, SpecOrder order)
+{
+    const int m = blockIdx.x, u = blockIdx.y;
+    const double2* x = X + (long long)u * hk;
+    for (int j = threadIdx.x; j < f.M; j += blockDim.x)
+        sm64[j] = fold64(f, table, j, m, hk, (hk - 1) / 2, [&](int i) { return __ldg(x + i); });
+    __syncthreads();
+    fft64_inplace(sm64, f, table);
+    for (int t = threadIdx.x; t < f.M; t += blockDim.x) {
+        const double2 z = sm64[t];
+        const int p = spec_pos(order, m + f.R * perm[t]);
+        if constexpr (SYM) {
+            float* d = static_cast<float*>(dst) + (long long)(2 * u) * ldK + p;
+            d[0] = (float)(z.x * scale);
+            if (2 * u + 1 < ncols) d[ldK] = (float)(z.y * scale);
+        } else {
+            static_cast<float2*>(dst)[(long long)u * ldK + p] = make_float2((float)(z.x * scale), (float)(z.y * scale));
         }
     }
 }
@@ -196,19 +275,34 @@ __device__ __forceinline__ unsigned long long mix64(unsigned long long z)
     return z ^ (z >> 31);
 }
 
-__global__ void psf_fingerprint(const double* __restrict__ K, long long n, unsigned long long* out)
+// out[0] += the fingerprint, *asym |= 1 where K is not point-symmetric
+__global__ void __launch_bounds__(256) psf_inspect(const double* __restrict__ K, long long n, unsigned long long* out,
+                                                   int* asym)
 {
-    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const unsigned long long bits = (unsigned long long)__double_as_longlong(K[i]);
-    atomicAdd(out, mix64(bits ^ mix64((unsigned long long)i)));
+    unsigned long long sum = 0;
+    int differs = 0;
+    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
+        const double v = K[i];
+        sum += mix64((unsigned long long)__double_as_longlong(v) ^ mix64((unsigned long long)i));
+        if (v != K[n - 1 - i]) differs = 1;
+    }
+    differs = __syncthreads_or(differs);
+    __shared__ unsigned long long part[8];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+    if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = sum;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int w = 1; w < 8; ++w) sum += part[w];
+        atomicAdd(out, sum);
+        if (differs) atomicOr(asym, 1);
+    }
 }
 
-cudaError_t psf_fingerprint_launch(const double* K, long long n, unsigned long long* d_out,
-                                   cudaStream_t st)
+cudaError_t psf_inspect_launch(const double* K, long long n, unsigned long long* d_out, int* d_asym, cudaStream_t st)
 {
-    const unsigned blocks = (unsigned)((n + 255) / 256);
-    psf_fingerprint<<<blocks, 256, 0, st>>>(K, n, d_out);
+    const long long blocks = (n + 255) / 256;
+    psf_inspect<<<(unsigned)(blocks < 304 ? blocks : 304), 256, 0, st>>>(K, n, d_out, d_asym);
     return cudaGetLastError();
 }
 
@@ -226,60 +320,93 @@ cudaError_t psf_compare_launch(const double* a, const double* b, long long n, in
     return cudaGetLastError();
 }
 
-cudaError_t psf_symmetry_launch(const double* K, int hk, int wk, int* d_asym, cudaStream_t st)
+// scratch of a build: the packed row transforms, the column transforms'
+// inputs, then the tables
+size_t psf_scratch_bytes(int hk, int wk, int Ny, int Nx, int real_only)
 {
-    const long long n = (long long)hk * wk;
-    psf_symmetry<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(K, hk, wk, d_asym);
+    const size_t rows = real_only ? (hk + 1) / 2 : hk, ncols = Nx / 2 + 1, units = real_only ? (ncols + 1) / 2 : ncols;
+    (void)wk;
+    return 16ull * ((rows + 1) / 2 * (size_t)Nx + units * hk + (size_t)Nx + (size_t)Ny) + 2ull * ((size_t)Nx + (size_t)Ny) + 64;
+}
+
+// Full spectrum build in `scratch` (16-byte aligned).
+cudaError_t psf_spectrum_build(const double* K, int hk, int wk, int Ny, int Nx, int real_only, void* dst, long long ldK,
+                               SpecOrder order, void* scratch, cudaStream_t st)
+{
+    const int ncols = Nx / 2 + 1, units = real_only ? (ncols + 1) / 2 : ncols;
+    const Fft64 fx = fft64_split(Nx, wk), fy = fft64_split(Ny, hk);
+    if (fx.N == 0 || fy.N == 0) return cudaErrorInvalidValue;
+    const int rows = real_only ? (hk + 1) / 2 : hk, pairs = (rows + 1) / 2;
+    double2* W = static_cast<double2*>(scratch);
+    double2* X = W + (size_t)pairs * Nx;
+    double2* tx = X + (size_t)units * hk;
+    double2* ty = tx + Nx;
+    unsigned short* px = reinterpret_cast<unsigned short*>(ty + Ny);
+    unsigned short* py = px + Nx;
+    const int sx = 16 * fx.M, sy = 16 * fy.M;
+    if (sx > 48 * 1024 || sy > 48 * 1024) {  // (one value for all builds: they may run side by side)
+        constexpr auto attr = cudaFuncAttributeMaxDynamicSharedMemorySize;
+        cudaError_t e = cudaFuncSetAttribute(psf_rows, attr, 16 * kMaxM64);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(psf_cols<true>, attr, 16 * kMaxM64);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(psf_cols<false>, attr, 16 * kMaxM64);
+        if (e != cudaSuccess) return e;
+    }
+    fft64_tables<<<(Nx + 127) / 128, 128, 0, st>>>(fx, tx, px);
+    if (Ny == Nx && fy.R == fx.R) {
+        ty = tx;
+        py = px;
+    } else {
+        fft64_tables<<<(Ny + 127) / 128, 128, 0, st>>>(fy, ty, py);
+    }
+    // (threads: about one radix-8 butterfly each, whole warps)
+    const auto threads = [](int M) { return M >= 2048 ? 256 : M >= 512 ? 128 : 64; };
+    psf_rows<<<dim3(fx.R, pairs), threads(fx.M), sx, st>>>(K, hk, wk, real_only ? (hk - 1) / 2 : 0, fx, tx, px, W);
+    const dim3 gp((units + 31) / 32, (hk + 31) / 32), bp(32, 8), gc(fy.R, units);
+    const double scale = 1.0 / (2.0 * (double)Ny * (double)Nx);
+    if (real_only) {
+        psf_pack<true><<<gp, bp, 0, st>>>(W, hk, Nx, ncols, units, X);
+        psf_cols<true><<<gc, threads(fy.M), sy, st>>>(X, hk, ncols, fy, ty, py, scale, dst, ldK, order);
+    } else {
+        psf_pack<false><<<gp, bp, 0, st>>>(W, hk, Nx, ncols, units, X);
+        psf_cols<false><<<gc, threads(fy.M), sy, st>>>(X, hk, ncols, fy, ty, py, scale, dst, ldK, order);
+    }
     return cudaGetLastError();
 }
 
-// Full spectrum build.  W1 holds hk*Nx, W2a/W2b each Ny*ncols complex128.
-cudaError_t psf_spectrum_build(const double* K, int hk, int wk, int Ny, int Nx, int real_only,
-                               void* dst, long long ldK, SpecOrder order, double2* W1, double2* W1b,
-                               double2* W2a, double2* W2b, cudaStream_t st)
+// One stored column to natural order, by way of shared memory (reading the
+// gathered order straight from memory took 52 us at 4704 x 4704)
+template <class V>
+__global__ void __launch_bounds__(256) spectrum_natural(const V* __restrict__ src, long long ldK, int ny, SpecOrder order,
+                                                        V* __restrict__ dst)
 {
-    const int ncols = Nx / 2 + 1;
-    const int cy = (hk - 1) / 2, cx = (wk - 1) / 2;
-    cudaError_t e;
-    if ((e = cudaMemsetAsync(W1, 0, sizeof(double2) * (size_t)hk * Nx, st)) != cudaSuccess) return e;
-    {
-        const long long n = (long long)hk * wk;
-        psf_scatter_rows<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(K, hk, wk, Nx, cx, W1);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    }
-    double2* rows = nullptr;
-    if ((e = fft64_forward(W1, W1b, Nx, 1, Nx, hk, 0, st, &rows)) != cudaSuccess) return e;
-    if ((e = cudaMemsetAsync(W2a, 0, sizeof(double2) * (size_t)Ny * ncols, st)) != cudaSuccess) return e;
-    {
-        const long long n = (long long)hk * ncols;
-        psf_scatter_cols<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(rows, hk, Nx, ncols, Ny, cy, W2a);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    }
-    double2* cols = nullptr;
-    if ((e = fft64_forward(W2a, W2b, Ny, ncols, 1, ncols, 1, st, &cols)) != cudaSuccess) return e;
-    const double scale = 1.0 / (2.0 * (double)Ny * (double)Nx);
-    dim3 grid((ncols + 31) / 32, (Ny + 31) / 32), block(32, 8);
-    psf_store_spectrum<<<grid, block, 0, st>>>(cols, Ny, ncols, scale, real_only, dst, ldK, order);
-    return cudaGetLastError();
+    extern __shared__ __align__(16) unsigned char smn[];
+    V* col = reinterpret_cast<V*>(smn);
+    src += (long long)blockIdx.x * ldK;
+    dst += (long long)blockIdx.x * ny;
+    for (int p = threadIdx.x; p < ny; p += blockDim.x) col[p] = src[p];
+    __syncthreads();
+    for (int u = threadIdx.x; u < ny; u += blockDim.x) dst[u] = col[spec_pos(order, u)];
 }
 
 template <class V>
-__global__ void spectrum_natural(const V* __restrict__ src, long long ldK, int ny, SpecOrder order, V* __restrict__ dst)
+static cudaError_t natural_launch(const void* data, long long ldK, int ny, int ncols, SpecOrder order, float* dst,
+                                  cudaStream_t st)
 {
-    const int u = blockIdx.x * blockDim.x + threadIdx.x;
-    if (u < ny) dst[(long long)blockIdx.y * ny + u] = src[(long long)blockIdx.y * ldK + spec_pos(order, u)];
+    // (the attribute's value does not depend on the length: copies of
+    // different lengths may be launched side by side)
+    const cudaError_t e = cudaFuncSetAttribute(spectrum_natural<V>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                               (int)(sizeof(V) * 28 * 1024));
+    if (e != cudaSuccess) return e;
+    spectrum_natural<V><<<ncols, 256, sizeof(V) * (size_t)ny, st>>>(static_cast<const V*>(data), ldK, ny, order,
+                                                                    reinterpret_cast<V*>(dst));
+    return cudaGetLastError();
 }
 
 cudaError_t spectrum_copy_natural(const void* data, long long ldK, int ny, int ncols, int is_real, SpecOrder order,
                                   float* dst, cudaStream_t st)
 {
-    const dim3 grid((ny + 255) / 256, ncols);  // ncols <= 8641: within the grid's y limit
-    if (is_real)
-        spectrum_natural<float><<<grid, 256, 0, st>>>(static_cast<const float*>(data), ldK, ny, order, dst);
-    else
-        spectrum_natural<float2><<<grid, 256, 0, st>>>(static_cast<const float2*>(data), ldK, ny, order,
-                                                       reinterpret_cast<float2*>(dst));
-    return cudaGetLastError();
+    return is_real ? natural_launch<float>(data, ldK, ny, ncols, order, dst, st)
+                   : natural_launch<float2>(data, ldK, ny, ncols, order, dst, st);
 }
 
 }  // namespace lpk
