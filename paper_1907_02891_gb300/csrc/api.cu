@@ -169,6 +169,13 @@ static void free_spectrum(lp_ctx* ctx, lp_spectrum* s);
 // ---------------------------------------------------------------------------
 // context internals
 // ---------------------------------------------------------------------------
+// gives the pool's kept memory back; true when there is a pool
+static bool pool_trim(lp_ctx* ctx)
+{
+    std::lock_guard<std::mutex> g(ctx->pool_mu);
+    return ctx->pool && cudaMemPoolTrimTo(ctx->pool, 0) == cudaSuccess;
+}
+
 lp_status lp_ctx_alloc(lp_ctx* ctx, size_t bytes, void** p)
 {
     *p = nullptr;
@@ -181,6 +188,10 @@ lp_status lp_ctx_alloc(lp_ctx* ctx, size_t bytes, void** p)
         ctx->used += bytes;
     }
     cudaError_t e = cudaMalloc(p, bytes);
+    if (e == cudaErrorMemoryAllocation && pool_trim(ctx)) {
+        (void)cudaGetLastError();
+        e = cudaMalloc(p, bytes);
+    }
     if (e != cudaSuccess) {
         std::lock_guard<std::mutex> g(ctx->mem_mu);
         ctx->used -= bytes;
@@ -195,6 +206,72 @@ void lp_ctx_free(lp_ctx* ctx, void* p, size_t bytes)
 {
     if (!p) return;
     cudaFree(p);
+    std::lock_guard<std::mutex> g(ctx->mem_mu);
+    ctx->used -= bytes;
+}
+
+// bytes of the pool, in stream order (not counted as held by the context)
+static cudaError_t pool_alloc(lp_ctx* ctx, size_t bytes, void** p, cudaStream_t st)
+{
+    *p = nullptr;
+    {
+        std::lock_guard<std::mutex> g(ctx->pool_mu);
+        if (!ctx->pool) {
+            cudaMemPoolProps props = {};
+            props.allocType = cudaMemAllocationTypePinned;
+            props.location.type = cudaMemLocationTypeDevice;
+            props.location.id = ctx->device;
+            cudaMemPool_t pool = nullptr;
+            cudaStream_t ps = nullptr;
+            cudaError_t e = cudaStreamCreateWithFlags(&ps, cudaStreamNonBlocking);
+            if (e == cudaSuccess) e = cudaMemPoolCreate(&pool, &props);
+            unsigned long long keep = ctx->budget ? 0 : lp_ctx::kPoolKeep;
+            if (e == cudaSuccess) e = cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep);
+            if (e != cudaSuccess) {
+                if (pool) cudaMemPoolDestroy(pool);
+                if (ps) cudaStreamDestroy(ps);
+                return e;
+            }
+            ctx->pool = pool;
+            ctx->pool_stream = ps;
+        }
+    }
+    cudaError_t e = cudaMallocFromPoolAsync(p, bytes, ctx->pool, st);
+    if (e == cudaErrorMemoryAllocation && pool_trim(ctx)) {
+        (void)cudaGetLastError();
+        e = cudaMallocFromPoolAsync(p, bytes, ctx->pool, st);
+    }
+    return e;
+}
+
+// memory of a spectrum: from the pool, counted as held by the context
+static lp_status spectrum_alloc(lp_ctx* ctx, size_t bytes, void** p, cudaStream_t st)
+{
+    *p = nullptr;
+    {
+        std::lock_guard<std::mutex> g(ctx->mem_mu);
+        if (ctx->budget && ctx->used + bytes > ctx->budget)
+            return lp_fail(LP_ERR_OOM, "HBM budget: %zu bytes held + %zu requested > %zu", ctx->used, bytes,
+                           ctx->budget);
+        ctx->used += bytes;
+    }
+    const cudaError_t e = pool_alloc(ctx, bytes, p, st);
+    if (e != cudaSuccess) {
+        (void)cudaGetLastError();
+        std::lock_guard<std::mutex> g(ctx->mem_mu);
+        ctx->used -= bytes;
+        *p = nullptr;
+        return lp_fail(e == cudaErrorMemoryAllocation ? LP_ERR_OOM : LP_ERR_CUDA, "spectrum memory (%zu bytes): %s",
+                       bytes, cudaGetErrorString(e));
+    }
+    return LP_OK;
+}
+
+// (the device has completed every use of p)
+static void spectrum_free(lp_ctx* ctx, void* p, size_t bytes)
+{
+    if (!p) return;
+    cudaFreeAsync(p, ctx->pool_stream);
     std::lock_guard<std::mutex> g(ctx->mem_mu);
     ctx->used -= bytes;
 }
@@ -487,6 +564,11 @@ extern "C" void lp_destroy(lp_ctx* ctx)
     ctx->spectra.clear();
     for (lp_spectrum* sp : ctx->released) free_spectrum(ctx, sp);
     ctx->released.clear();
+    if (ctx->pool) {
+        cudaStreamSynchronize(ctx->pool_stream);
+        cudaStreamDestroy(ctx->pool_stream);
+        cudaMemPoolDestroy(ctx->pool);
+    }
     for (auto& w : ctx->ws) lp_ctx_free(ctx, w.ptr, w.bytes);
     ctx->ws.clear();
     for (auto& kv : ctx->plans) lp_ctx_free(ctx, kv.second->tw, kv.second->bytes);
@@ -571,13 +653,14 @@ extern "C" lp_status lp_kernel_spectrum(lp_ctx* ctx, const double* K, int hk, in
     // fingerprint + symmetry (one small device round trip); the third word
     // holds the flag of the value comparisons below
     unsigned long long* d_fp = nullptr;
-    CUDA_TRY(cudaMallocAsync((void**)&d_fp, 24, st));
+    CUDA_TRY(pool_alloc(ctx, 24, (void**)&d_fp, st));
     CUDA_TRY(cudaMemsetAsync(d_fp, 0, 24, st));
-    CUDA_TRY(psf_inspect_launch(K, (long long)hk * wk, d_fp, reinterpret_cast<int*>(d_fp + 1), st));
+    CUDA_TRY(psf_inspect_launch(K, hk, wk, d_fp, reinterpret_cast<int*>(d_fp + 1), st));
     unsigned long long host_fp[2] = {0, 0};
     CUDA_TRY(cudaMemcpyAsync(host_fp, d_fp, 16, cudaMemcpyDeviceToHost, st));
     CUDA_TRY(cudaStreamSynchronize(st));
-    const int is_real = (int)(host_fp[1] & 0xffffffffull) == 0;
+    const int asym = (int)(host_fp[1] & 0xffffffffull);
+    const int is_real = (asym & 1) == 0;
     if (ctx->test_hook & LP_TEST_FP_COLLIDE) host_fp[0] = 0;
     const SpecKey key0{host_fp[0], hk, wk, Ny, Nx, (int)prec, 0};
     int* d_diff = reinterpret_cast<int*>(d_fp + 2);
@@ -647,11 +730,11 @@ extern "C" lp_status lp_kernel_spectrum(lp_ctx* ctx, const double* K, int hk, in
         free_spectrum(ctx, sp);
     };
     void* dptr = nullptr;
-    lp_status sa = lp_ctx_alloc(ctx, bytes, &dptr);
+    lp_status sa = spectrum_alloc(ctx, bytes, &dptr, st);
     if (sa == LP_OK) {
         spec->data = dptr;
         void* kc = nullptr;
-        sa = lp_ctx_alloc(ctx, spec->kbytes, &kc);
+        sa = spectrum_alloc(ctx, spec->kbytes, &kc, st);
         spec->kcopy = static_cast<double*>(kc);
     }
     if (sa != LP_OK) {
@@ -663,7 +746,7 @@ extern "C" lp_status lp_kernel_spectrum(lp_ctx* ctx, const double* K, int hk, in
     // FP64 scratch, stream-ordered, released right after the build
     const size_t scratch_bytes = psf_scratch_bytes(hk, wk, Ny, Nx, is_real);
     void* scratch = nullptr;
-    cudaError_t e = cudaMallocAsync(&scratch, scratch_bytes, st);
+    cudaError_t e = pool_alloc(ctx, scratch_bytes, &scratch, st);
     if (e != cudaSuccess) {
         cudaGetLastError();
         cudaFreeAsync(d_fp, st);
@@ -673,10 +756,8 @@ extern "C" lp_status lp_kernel_spectrum(lp_ctx* ctx, const double* K, int hk, in
     e = cudaMemcpyAsync(spec->kcopy, K, spec->kbytes, cudaMemcpyDeviceToDevice, st);
     // (columns end in padding up to ldK, which nothing reads)
     if (e == cudaSuccess)
-        e = psf_spectrum_build(K, hk, wk, Ny, Nx, is_real, dptr, ldK, spectrum_order(Ny, prec), scratch, st);
+        e = psf_spectrum_build(K, hk, wk, Ny, Nx, is_real, (asym & 2) == 0, dptr, ldK, spectrum_order(Ny, prec), scratch, st);
     cudaFreeAsync(scratch, st);
-    for (int i = 0; e == cudaSuccess && i < lp_spectrum::kUseSlots; ++i)
-        e = cudaEventCreateWithFlags(&spec->use_event[i], cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&spec->ready, cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaEventRecord(spec->ready, st);
     if (e != cudaSuccess) {
@@ -741,8 +822,8 @@ extern "C" lp_status lp_spectrum_copy(const lp_spectrum* s, float* dst, size_t d
 
 static void free_spectrum(lp_ctx* ctx, lp_spectrum* s)
 {
-    lp_ctx_free(ctx, s->data, s->bytes);
-    lp_ctx_free(ctx, s->kcopy, s->kbytes);
+    spectrum_free(ctx, s->data, s->bytes);
+    spectrum_free(ctx, s->kcopy, s->kbytes);
     if (s->ready) cudaEventDestroy(s->ready);
     for (int i = 0; i < lp_spectrum::kUseSlots; ++i)
         if (s->use_event[i]) cudaEventDestroy(s->use_event[i]);
@@ -848,7 +929,9 @@ void lp_note_spectra_used(lp_ctx* ctx, const lp_spectrum* const* spectra, int n,
             slot = s->nuse++;
             s->use_stream[slot] = st;
         }
-        if (cudaEventRecord(s->use_event[slot], st) != cudaSuccess) {
+        if ((!s->use_event[slot] &&
+             cudaEventCreateWithFlags(&s->use_event[slot], cudaEventDisableTiming) != cudaSuccess) ||
+            cudaEventRecord(s->use_event[slot], st) != cudaSuccess) {
             cudaGetLastError();
             s->use_overflow = true;
         }

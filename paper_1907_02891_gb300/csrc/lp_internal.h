@@ -64,13 +64,14 @@ struct SpecOrder {
 
 // FP64 spectrum pipeline (spectrum.cu)
 bool fft64_supported(int N);
-// *d_out += the fingerprint of K's n values, *d_asym |= 1 where K is not point-symmetric
-cudaError_t psf_inspect_launch(const double* K, long long n, unsigned long long* d_out, int* d_asym, cudaStream_t st);
+// *d_out += the fingerprint of K's values; *d_asym |= 1 where K is not point-symmetric, |= 2 where its rows are not
+// mirror-symmetric
+cudaError_t psf_inspect_launch(const double* K, int hk, int wk, unsigned long long* d_out, int* d_asym, cudaStream_t st);
 // *d_diff |= 1 where a[i] and b[i] differ in any bit (i < n)
 cudaError_t psf_compare_launch(const double* a, const double* b, long long n, int* d_diff, cudaStream_t st);
 size_t psf_scratch_bytes(int hk, int wk, int Ny, int Nx, int real_only);
-cudaError_t psf_spectrum_build(const double* K, int hk, int wk, int Ny, int Nx, int real_only, void* dst, long long ldK,
-                               SpecOrder order, void* scratch, cudaStream_t st);
+cudaError_t psf_spectrum_build(const double* K, int hk, int wk, int Ny, int Nx, int real_only, int mirror, void* dst,
+                               long long ldK, SpecOrder order, void* scratch, cudaStream_t st);
 // a stored spectrum's columns in natural order, packed (ny values each)
 cudaError_t spectrum_copy_natural(const void* data, long long ldK, int ny, int ncols, int is_real, SpecOrder order,
                                   float* dst, cudaStream_t st);

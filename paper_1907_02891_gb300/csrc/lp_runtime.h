@@ -93,6 +93,15 @@ struct lp_ctx {
     int device = 0;
     size_t budget = 0, used = 0;
     std::mutex mem_mu, plan_mu, spec_mu, ws_mu;
+    // Stream-ordered memory of the spectrum builds (spectra and scratch): a
+    // pool of the context's own that keeps up to kPoolKeep bytes of freed
+    // memory for the next build (none under an HBM budget) and goes with the
+    // context.  Freed spectra go back through a stream of its own, once their
+    // uses are complete.
+    static constexpr unsigned long long kPoolKeep = 256ull << 20;
+    std::mutex pool_mu;
+    cudaMemPool_t pool = nullptr;
+    cudaStream_t pool_stream = nullptr;
     std::map<int, std::unique_ptr<PlanRec>> plans;
     std::map<SpecKey, lp_spectrum*> spectra;
     // released spectra whose last uses may still be running: freed once

@@ -15,6 +15,9 @@
 //     conjugate of row y);
 //   * the columns of a point-symmetric K have real transforms, so two of
 //     them share one complex transform;
+//   * of a K that is mirror-symmetric too (a radial PSF), every transform is
+//     even, so only the residues m <= R / 2 below are transformed and their
+//     mirror images stored with them;
 //   * a transform of length N = R M of k < N non-zero samples is, per residue
 //     m < R, the M-point transform of the samples times exp(-i 2 pi n m / N)
 //     folded modulo M: X[m + R k'] = sum_j w_M^{j k'} sum_{n = j mod M} x[n]
@@ -23,9 +26,10 @@
 //     shared memory;
 //   * twiddles come from a table of N values made once per build; sincospi
 //     per element and stage had taken most of the build's time.
-// For the 541 x 541 PSF at 4704 x 4704 the transforms took 4.3 ms as one
-// global-memory pass per radix, and the fingerprint 0.19 ms with an atomic
-// per PSF value.
+// For the 541 x 541 PSF at 4704 x 4704 (radial) the transforms took 4.3 ms as
+// one global-memory pass per radix with sincospi twiddles, and take 0.32 ms
+// (columns 254 us, 0.68 of the FP64 rate; rows 36, transposition 28 us); the
+// fingerprint took 190 us with an atomic per PSF value, and takes 6.
 #include "fft_core.cuh"
 #include "lp_internal.h"
 
@@ -167,8 +171,9 @@ __device__ __forceinline__ double2 fold64(const Fft64& f, const double2* __restr
 extern __shared__ __align__(16) double2 sm64[];
 
 // Row pair p (rows y0 + 2p, y0 + 2p + 1 of K packed as a + i b), residue m
-// = blockIdx.x: frequencies m + R k' to W[p][.].
-__global__ void __launch_bounds__(256) psf_rows(const double* __restrict__ K, int hk, int wk, int y0, Fft64 f,
+// = blockIdx.x: frequencies m + R k' to W[p][.]; mirror: the rows are even,
+// and so are their transforms (grid: residues 0 .. R / 2).
+__global__ void __launch_bounds__(256) psf_rows(const double* __restrict__ K, int hk, int wk, int y0, int mirror, Fft64 f,
                                                 const double2* __restrict__ table, const unsigned short* __restrict__ perm,
                                                 double2* __restrict__ W)
 {
@@ -180,8 +185,13 @@ __global__ void __launch_bounds__(256) psf_rows(const double* __restrict__ K, in
         sm64[j] = fold64(f, table, j, m, wk, (wk - 1) / 2, [&](int i) { return mk<double2>(a[i], vb ? a[wk + i] : 0.0); });
     __syncthreads();
     fft64_inplace(sm64, f, table);
-    double2* dst = W + (long long)p * f.N + m;
-    for (int t = threadIdx.x; t < f.M; t += blockDim.x) dst[(long long)f.R * perm[t]] = sm64[t];
+    double2* dst = W + (long long)p * f.N;
+    const bool both = mirror && m != 0 && 2 * m != f.R;
+    for (int t = threadIdx.x; t < f.M; t += blockDim.x) {
+        const int u = m + f.R * perm[t];
+        dst[u] = sm64[t];
+        if (both) dst[f.N - u] = sm64[t];
+    }
 }
 
 // G_y[c] from the packed row transforms: rows a = 2p, b = 2p + 1 of pair p,
@@ -238,9 +248,10 @@ __global__ void __launch_bounds__(256) psf_pack(const double2* __restrict__ W, i
 }
 
 // Column transforms of unit blockIdx.y, residue m = blockIdx.x.  SYM: the real
-// and imaginary parts of the result are the real spectra of columns 2u, 2u + 1.
+// and imaginary parts of the result are the real spectra of columns 2u, 2u + 1
+// (mirror: both are even; grid: residues 0 .. R / 2).
 template <bool SYM>
-__global__ void __launch_bounds__(256) psf_cols(const double2* __restrict__ X, int hk, int ncols, Fft64 f,
+__global__ void __launch_bounds__(256) psf_cols(const double2* __restrict__ X, int hk, int ncols, int mirror, Fft64 f,
                                                 const double2* __restrict__ table, const unsigned short* __restrict__ perm,
                                                 double scale, void* dst, long long ldK, SpecOrder order)
 {
@@ -250,15 +261,20 @@ __global__ void __launch_bounds__(256) psf_cols(const double2* __restrict__ X, i
         sm64[j] = fold64(f, table, j, m, hk, (hk - 1) / 2, [&](int i) { return __ldg(x + i); });
     __syncthreads();
     fft64_inplace(sm64, f, table);
+    const bool both = SYM && mirror && m != 0 && 2 * m != f.R;
     for (int t = threadIdx.x; t < f.M; t += blockDim.x) {
         const double2 z = sm64[t];
-        const int p = spec_pos(order, m + f.R * perm[t]);
+        const int v = m + f.R * perm[t];
         if constexpr (SYM) {
-            float* d = static_cast<float*>(dst) + (long long)(2 * u) * ldK + p;
-            d[0] = (float)(z.x * scale);
-            if (2 * u + 1 < ncols) d[ldK] = (float)(z.y * scale);
+            float* d = static_cast<float*>(dst) + (long long)(2 * u) * ldK;
+            for (int side = 0; side <= (both ? 1 : 0); ++side) {
+                const int p = spec_pos(order, side ? f.N - v : v);
+                d[p] = (float)(z.x * scale);
+                if (2 * u + 1 < ncols) d[ldK + p] = (float)(z.y * scale);
+            }
         } else {
-            static_cast<float2*>(dst)[(long long)u * ldK + p] = make_float2((float)(z.x * scale), (float)(z.y * scale));
+            static_cast<float2*>(dst)[(long long)u * ldK + spec_pos(order, v)] =
+                make_float2((float)(z.x * scale), (float)(z.y * scale));
         }
     }
 }
@@ -275,18 +291,23 @@ __device__ __forceinline__ unsigned long long mix64(unsigned long long z)
     return z ^ (z >> 31);
 }
 
-// out[0] += the fingerprint, *asym |= 1 where K is not point-symmetric
-__global__ void __launch_bounds__(256) psf_inspect(const double* __restrict__ K, long long n, unsigned long long* out,
+// out[0] += the fingerprint, *asym |= 1 where K is not point-symmetric, |= 2
+// where its rows are not mirror-symmetric
+__global__ void __launch_bounds__(256) psf_inspect(const double* __restrict__ K, int hk, int wk, unsigned long long* out,
                                                    int* asym)
 {
+    const long long n = (long long)hk * wk;
     unsigned long long sum = 0;
     int differs = 0;
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
         const double v = K[i];
         sum += mix64((unsigned long long)__double_as_longlong(v) ^ mix64((unsigned long long)i));
-        if (v != K[n - 1 - i]) differs = 1;
+        const long long y = i / wk;
+        if (v != K[n - 1 - i]) differs |= 1;
+        if (v != K[(hk - 1 - y) * wk + (i - y * wk)]) differs |= 2;
     }
-    differs = __syncthreads_or(differs);
+    differs = __syncthreads_or(differs & 1) ? 1 | (differs & 2) : differs & 2;
+    differs = __syncthreads_or(differs & 2) ? 2 | (differs & 1) : differs & 1;
     __shared__ unsigned long long part[8];
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
@@ -295,14 +316,14 @@ __global__ void __launch_bounds__(256) psf_inspect(const double* __restrict__ K,
     if (threadIdx.x == 0) {
         for (int w = 1; w < 8; ++w) sum += part[w];
         atomicAdd(out, sum);
-        if (differs) atomicOr(asym, 1);
+        if (differs) atomicOr(asym, differs);
     }
 }
 
-cudaError_t psf_inspect_launch(const double* K, long long n, unsigned long long* d_out, int* d_asym, cudaStream_t st)
+cudaError_t psf_inspect_launch(const double* K, int hk, int wk, unsigned long long* d_out, int* d_asym, cudaStream_t st)
 {
-    const long long blocks = (n + 255) / 256;
-    psf_inspect<<<(unsigned)(blocks < 304 ? blocks : 304), 256, 0, st>>>(K, n, d_out, d_asym);
+    const long long blocks = ((long long)hk * wk + 255) / 256;
+    psf_inspect<<<(unsigned)(blocks < 304 ? blocks : 304), 256, 0, st>>>(K, hk, wk, d_out, d_asym);
     return cudaGetLastError();
 }
 
@@ -330,8 +351,8 @@ size_t psf_scratch_bytes(int hk, int wk, int Ny, int Nx, int real_only)
 }
 
 // Full spectrum build in `scratch` (16-byte aligned).
-cudaError_t psf_spectrum_build(const double* K, int hk, int wk, int Ny, int Nx, int real_only, void* dst, long long ldK,
-                               SpecOrder order, void* scratch, cudaStream_t st)
+cudaError_t psf_spectrum_build(const double* K, int hk, int wk, int Ny, int Nx, int real_only, int mirror, void* dst,
+                               long long ldK, SpecOrder order, void* scratch, cudaStream_t st)
 {
     const int ncols = Nx / 2 + 1, units = real_only ? (ncols + 1) / 2 : ncols;
     const Fft64 fx = fft64_split(Nx, wk), fy = fft64_split(Ny, hk);
@@ -360,21 +381,24 @@ cudaError_t psf_spectrum_build(const double* K, int hk, int wk, int Ny, int Nx, 
     }
     // (threads: about one radix-8 butterfly each, whole warps)
     const auto threads = [](int M) { return M >= 2048 ? 256 : M >= 512 ? 128 : 64; };
-    psf_rows<<<dim3(fx.R, pairs), threads(fx.M), sx, st>>>(K, hk, wk, real_only ? (hk - 1) / 2 : 0, fx, tx, px, W);
-    const dim3 gp((units + 31) / 32, (hk + 31) / 32), bp(32, 8), gc(fy.R, units);
+    mirror = mirror && real_only;
+    const auto residues = [mirror](int R) { return mirror ? R / 2 + 1 : R; };
+    psf_rows<<<dim3(residues(fx.R), pairs), threads(fx.M), sx, st>>>(K, hk, wk, real_only ? (hk - 1) / 2 : 0, mirror, fx,
+                                                                    tx, px, W);
+    const dim3 gp((units + 31) / 32, (hk + 31) / 32), bp(32, 8), gc(residues(fy.R), units);
     const double scale = 1.0 / (2.0 * (double)Ny * (double)Nx);
     if (real_only) {
         psf_pack<true><<<gp, bp, 0, st>>>(W, hk, Nx, ncols, units, X);
-        psf_cols<true><<<gc, threads(fy.M), sy, st>>>(X, hk, ncols, fy, ty, py, scale, dst, ldK, order);
+        psf_cols<true><<<gc, threads(fy.M), sy, st>>>(X, hk, ncols, mirror, fy, ty, py, scale, dst, ldK, order);
     } else {
         psf_pack<false><<<gp, bp, 0, st>>>(W, hk, Nx, ncols, units, X);
-        psf_cols<false><<<gc, threads(fy.M), sy, st>>>(X, hk, ncols, fy, ty, py, scale, dst, ldK, order);
+        psf_cols<false><<<gc, threads(fy.M), sy, st>>>(X, hk, ncols, mirror, fy, ty, py, scale, dst, ldK, order);
     }
     return cudaGetLastError();
 }
 
 // One stored column to natural order, by way of shared memory (reading the
-// gathered order straight from memory took 52 us at 4704 x 4704)
+// gathered order straight from memory took 52 us at 4704 x 4704, this 28)
 template <class V>
 __global__ void __launch_bounds__(256) spectrum_natural(const V* __restrict__ src, long long ldK, int ny, SpecOrder order,
                                                         V* __restrict__ dst)
@@ -383,9 +407,14 @@ __global__ void __launch_bounds__(256) spectrum_natural(const V* __restrict__ sr
     V* col = reinterpret_cast<V*>(smn);
     src += (long long)blockIdx.x * ldK;
     dst += (long long)blockIdx.x * ny;
-    for (int p = threadIdx.x; p < ny; p += blockDim.x) col[p] = src[p];
+    // (one element of padding per 32: a step of one in m may be a multiple of
+    // 32 positions)
+    for (int p = threadIdx.x; p < ny; p += blockDim.x) col[p + (p >> 5)] = src[p];
     __syncthreads();
-    for (int u = threadIdx.x; u < ny; u += blockDim.x) dst[u] = col[spec_pos(order, u)];
+    for (int u = threadIdx.x; u < ny; u += blockDim.x) {
+        const int p = spec_pos(order, u);
+        dst[u] = col[p + (p >> 5)];
+    }
 }
 
 template <class V>
@@ -397,7 +426,7 @@ static cudaError_t natural_launch(const void* data, long long ldK, int ny, int n
     const cudaError_t e = cudaFuncSetAttribute(spectrum_natural<V>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                (int)(sizeof(V) * 28 * 1024));
     if (e != cudaSuccess) return e;
-    spectrum_natural<V><<<ncols, 256, sizeof(V) * (size_t)ny, st>>>(static_cast<const V*>(data), ldK, ny, order,
+    spectrum_natural<V><<<ncols, 256, sizeof(V) * (size_t)(ny + ny / 32 + 1), st>>>(static_cast<const V*>(data), ldK, ny, order,
                                                                     reinterpret_cast<V*>(dst));
     return cudaGetLastError();
 }

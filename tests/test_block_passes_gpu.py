@@ -68,3 +68,33 @@ def test_plans_name_block_geometries():
         assert r0 * r1 * r2 == n and 1 <= max(r1, r2) <= 32 and r0 <= B.R0_MAX
         for key in ("p1", "p2", "p3", "pm"):
             assert p["geo"][key][-2] % 32 == 0 and p["geo"][key][-2] <= B.MAX_THREADS
+
+
+@pytest.mark.parametrize("kind", ["radial", "point", "none"])
+@pytest.mark.parametrize("ny,nx,hk,wk", [(45, 64, 45, 63), (96, 45, 1, 1), (360, 1120, 101, 1119), (4704, 210, 541, 7),
+                                         (1536, 128, 1535, 3), (17280, 45, 801, 5), (64, 8820, 5, 601)])
+def test_spectrum_build_of_each_symmetry(ctx, kind, ny, nx, hk, wk):
+    """The folded FP64 build against numpy's FP64 transform, for PSFs that are
+    mirror-symmetric, point-symmetric only, and neither.  Tolerance: one
+    rounding to FP32 of the largest value, 2^-24 < 6e-8 of it, doubled."""
+    import torch
+    from paper_1907_02891_gb300 import lp
+    rng = np.random.default_rng(ny + 7 * nx)
+    K = rng.random((hk, wk)) + 0.01
+    if kind != "none":
+        K = (K + K[::-1, ::-1]) / 2
+    if kind == "radial":
+        K = (K + K[::-1]) / 2
+    spec = lp.lp_kernel_spectrum(ctx, torch.from_numpy(np.ascontiguousarray(K)).cuda(), pad_ny=ny, pad_nx=nx)
+    real = lp.lp_spectrum_info(spec)["is_real"]
+    assert real == bool((K == K[::-1, ::-1]).all())
+    got = torch.empty(nx // 2 + 1, ny, 1 if real else 2, device="cuda")
+    lp.lp_spectrum_copy(spec, got)
+    lp.lp_sync_status(ctx)
+    lp.lp_spectrum_release(ctx, spec)
+    P = np.zeros((ny, nx))
+    P[:hk, :wk] = K
+    S = np.fft.rfft2(np.roll(P, (-(hk // 2), -(wk // 2)), (0, 1))).T / (2.0 * ny * nx)
+    g = got.double().cpu().numpy()
+    diff = np.abs(g[..., 0] - S.real) if real else np.hypot(g[..., 0] - S.real, g[..., 1] - S.imag)
+    assert diff.max() <= 1.2e-7 * np.abs(S).max()
