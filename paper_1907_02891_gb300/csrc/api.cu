@@ -210,6 +210,15 @@ void lp_ctx_free(lp_ctx* ctx, void* p, size_t bytes)
     ctx->used -= bytes;
 }
 
+// The pool keeps kPoolKeep bytes beyond the live spectra (its release
+// threshold counts used memory as well).  Called with pool_mu held.
+static void pool_keep(lp_ctx* ctx, long long more)
+{
+    ctx->pool_used += more;
+    unsigned long long keep = ctx->budget ? 0 : ctx->pool_used + lp_ctx::kPoolKeep;
+    cudaMemPoolSetAttribute(ctx->pool, cudaMemPoolAttrReleaseThreshold, &keep);
+}
+
 // bytes of the pool, in stream order (not counted as held by the context)
 static cudaError_t pool_alloc(lp_ctx* ctx, size_t bytes, void** p, cudaStream_t st)
 {
@@ -225,8 +234,6 @@ static cudaError_t pool_alloc(lp_ctx* ctx, size_t bytes, void** p, cudaStream_t 
             cudaStream_t ps = nullptr;
             cudaError_t e = cudaStreamCreateWithFlags(&ps, cudaStreamNonBlocking);
             if (e == cudaSuccess) e = cudaMemPoolCreate(&pool, &props);
-            unsigned long long keep = ctx->budget ? 0 : lp_ctx::kPoolKeep;
-            if (e == cudaSuccess) e = cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep);
             if (e != cudaSuccess) {
                 if (pool) cudaMemPoolDestroy(pool);
                 if (ps) cudaStreamDestroy(ps);
@@ -234,6 +241,7 @@ static cudaError_t pool_alloc(lp_ctx* ctx, size_t bytes, void** p, cudaStream_t 
             }
             ctx->pool = pool;
             ctx->pool_stream = ps;
+            pool_keep(ctx, 0);
         }
     }
     cudaError_t e = cudaMallocFromPoolAsync(p, bytes, ctx->pool, st);
@@ -264,6 +272,8 @@ static lp_status spectrum_alloc(lp_ctx* ctx, size_t bytes, void** p, cudaStream_
         return lp_fail(e == cudaErrorMemoryAllocation ? LP_ERR_OOM : LP_ERR_CUDA, "spectrum memory (%zu bytes): %s",
                        bytes, cudaGetErrorString(e));
     }
+    std::lock_guard<std::mutex> g(ctx->pool_mu);
+    pool_keep(ctx, (long long)bytes);
     return LP_OK;
 }
 
@@ -271,7 +281,11 @@ static lp_status spectrum_alloc(lp_ctx* ctx, size_t bytes, void** p, cudaStream_
 static void spectrum_free(lp_ctx* ctx, void* p, size_t bytes)
 {
     if (!p) return;
-    cudaFreeAsync(p, ctx->pool_stream);
+    {
+        std::lock_guard<std::mutex> g(ctx->pool_mu);
+        cudaFreeAsync(p, ctx->pool_stream);
+        pool_keep(ctx, -(long long)bytes);
+    }
     std::lock_guard<std::mutex> g(ctx->mem_mu);
     ctx->used -= bytes;
 }

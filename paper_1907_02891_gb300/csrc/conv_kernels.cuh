@@ -622,6 +622,18 @@ __device__ __forceinline__ void load_spectrum(typename std::conditional<KREAL, f
     }
 }
 
+// Bulk prefetch of the spectrum columns c0 .. of one spectrum into L2 by NT
+// threads: a batched block's next spectrum, while it works on this one.
+template <class C, bool KREAL>
+__device__ __forceinline__ void prefetch_spectrum(const P2Args& a, const void* K, int c0, int t)
+{
+    if (t < C::NT && c0 + t < a.ncols) {
+        const float* p = static_cast<const float*>(K) + (long long)(c0 + t) * a.ldK * (KREAL ? 1 : 2);
+        asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;\n" ::"l"(p),
+                     "r"(16u * ((C::Ge::N * (KREAL ? 1 : 2) + 3) / 4)) : "memory");
+    }
+}
+
 template <bool KREAL, int R>
 __device__ __forceinline__ void spectrum_product(float2 (&f)[R],
                                                  const typename std::conditional<KREAL, float, float2>::type (&k)[R])
@@ -886,16 +898,18 @@ __global__ void __launch_bounds__(C::TH * GRP, C::MINB) p2_cols_multi(const __gr
     for (int cl = 0; cl < NT; ++cl)
         if (c0 + cl < a.ncols && !p2_column_ok(a, c0 + cl, Ge::N, KREAL ? 1 : 2)) return;
     float2* F = PARKG ? a.park + (size_t)c0 * Ge::N : lp_dsmem + Ge::W1 + GRP * C::WORK;
+    const int grp = GRP == 1 ? 0 : threadIdx.x / C::TH;
+    const int t = GRP == 1 ? threadIdx.x : threadIdx.x % C::TH;
+    if (grp < a.nspec) prefetch_spectrum<C, KREAL>(a, a.K[grp], c0, t);
     load_w1<Ge>(lp_dsmem, a.tw.w1, threadIdx.x, C::TH * GRP);
     columns_forward<C>(a.T, a.ldT, a.H, c0, a.ncols, a.tw, lp_dsmem + Ge::W1, threadIdx.x, C::TH * GRP,
                        [&](int cl, int m, int k1, float2(&f)[Ge::R2]) {
                            park_store<C>(F, (cl * Ge::R0 + m) * Ge::R1 + k1, f);
                        });
     __syncthreads();
-    const int grp = GRP == 1 ? 0 : threadIdx.x / C::TH;
-    const int t = GRP == 1 ? threadIdx.x : threadIdx.x % C::TH;
 #pragma unroll 1
     for (int s = grp; s < a.nspec; s += GRP) {
+        if (s + GRP < a.nspec) prefetch_spectrum<C, KREAL>(a, a.K[s + GRP], c0, t);
         p2_spectrum_pass<C, GRP, PARKG, KREAL>(a, c0, s, grp * C::WORK, t, grp);
         if constexpr (Ge::R0 > 1) group_sync<C::TH, GRP>(grp);  // the working set has been read
     }

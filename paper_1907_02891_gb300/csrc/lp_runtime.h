@@ -101,6 +101,7 @@ struct lp_ctx {
     static constexpr unsigned long long kPoolKeep = 256ull << 20;
     std::mutex pool_mu;
     cudaMemPool_t pool = nullptr;
+    size_t pool_used = 0;  // bytes of live spectra in it (the threshold counts them)
     cudaStream_t pool_stream = nullptr;
     std::map<int, std::unique_ptr<PlanRec>> plans;
     std::map<SpecKey, lp_spectrum*> spectra;
