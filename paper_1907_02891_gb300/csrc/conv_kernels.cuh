@@ -533,7 +533,7 @@ __device__ __forceinline__ void column_stage1(const float2* T, long long ldT, in
         for (int q = 0; q < R0; ++q) {
             const int row = j + q * N1;
             const long long off = (N1 % 2 == 0) ? t_row(j) + q * t_row_step<N1>() : t_row(row);
-            v[q] = (row < H && (NT == 1 || c < ncols)) ? col[off] : make_float2(0.f, 0.f);
+            v[q] = (row < H && (NT == 1 || c < ncols)) ? ld_once<Ge>(col + off) : make_float2(0.f, 0.f);
         }
         Dft<R0, -1, float2>::run(v);
         float2* w = sm + cl * La::ELEMS + stage1_addr<Ge>(j);
@@ -590,17 +590,17 @@ __device__ __forceinline__ void load_spectrum(typename std::conditional<KREAL, f
         for (int i = 0; i < R2; i += VK) {
             const float* q = p + i * Ge::R1;
             if constexpr (VK == 4) {
-                const float4 x = __ldg(reinterpret_cast<const float4*>(q));
+                const float4 x = ld_spectrum<Ge>(reinterpret_cast<const float4*>(q));
                 k[i] = x.x;
                 k[i + 1] = x.y;
                 k[i + 2] = x.z;
                 k[i + 3] = x.w;
             } else if constexpr (VK == 2) {
-                const float2 x = __ldg(reinterpret_cast<const float2*>(q));
+                const float2 x = ld_spectrum<Ge>(reinterpret_cast<const float2*>(q));
                 k[i] = x.x;
                 k[i + 1] = x.y;
             } else {
-                k[i] = __ldg(q);
+                k[i] = ld_spectrum<Ge>(q);
             }
         }
     } else {
@@ -611,12 +611,12 @@ __device__ __forceinline__ void load_spectrum(typename std::conditional<KREAL, f
             if constexpr (VK >= 2) {
 #pragma unroll
                 for (int h = 0; h < VK; h += 2) {
-                    const float4 x = __ldg(reinterpret_cast<const float4*>(q + h));
+                    const float4 x = ld_spectrum<Ge>(reinterpret_cast<const float4*>(q + h));
                     k[i + h] = make_float2(x.x, x.y);
                     k[i + h + 1] = make_float2(x.z, x.w);
                 }
             } else {
-                k[i] = __ldg(q);
+                k[i] = ld_spectrum<Ge>(q);
             }
         }
     }
@@ -655,7 +655,7 @@ __device__ __forceinline__ void column_direct(float2 (&x)[Ge::R1], const float2*
 #pragma unroll
     for (int l = 0; l < Ge::R1; ++l) {
         const int row = li + l * Ge::R2;
-        x[l] = row < H ? col[t_row(row)] : make_float2(0.f, 0.f);
+        x[l] = row < H ? ld_once<Ge>(col + t_row(row)) : make_float2(0.f, 0.f);
     }
 }
 template <class Ge>
@@ -1044,8 +1044,8 @@ __global__ void __launch_bounds__(C::TH, C::MINB) p3_rows(const __grid_constant_
                 const int c = u + k * UR;
                 q[k] = make_float4(0.f, 0.f, 0.f, 0.f);
                 if (load && (k < R2 / 2 || c < a.ncols)) {
-                    if constexpr (UR % kUCB == 0) q[k] = src[k * (UR / kUCB) * (ldq * kUCB)];
-                    else q[k] = Uq[u_index4(c, pair, ldq)];
+                    if constexpr (UR % kUCB == 0) q[k] = ld_once<Ge>(src + k * (UR / kUCB) * (ldq * kUCB));
+                    else q[k] = ld_once<Ge>(Uq + u_index4(c, pair, ldq));
                 }
                 if (!vb) q[k].z = q[k].w = 0.f;
             }
@@ -1091,8 +1091,8 @@ __global__ void __launch_bounds__(C::TH, C::MINB) p3_rows(const __grid_constant_
             for (int k = 0; k <= R2 / 2; ++k) {
                 const int c = u + k * UR;
                 if (k == R2 / 2 && c >= a.ncols) break;
-                if constexpr (UR % kUCB == 0) q[k] = src[k * (UR / kUCB) * (ldq * kUCB)];
-                else q[k] = Uq[u_index4(c, pair, ldq)];
+                if constexpr (UR % kUCB == 0) q[k] = ld_once<Ge>(src + k * (UR / kUCB) * (ldq * kUCB));
+                else q[k] = ld_once<Ge>(Uq + u_index4(c, pair, ldq));
                 if (!vb) q[k].z = q[k].w = 0.f;
             }
             if (La::VEC && u > 0) {

@@ -409,6 +409,7 @@ struct Geo {
     static constexpr int GPW = 32 / G;                          // sub-transforms per warp and round
     static constexpr int R1P = (R1 + 1) / 2 * 2;                // entries of w1 per m (16-byte rows)
     static constexpr int W1 = R0 > 1 ? (R0 * R1P + 7) / 8 * 8 : 0;  // shared-memory entries of w1
+    static constexpr bool STREAM = 4ll * N * N <= 129ll << 20;  // see ld_once
     // position in a spectrum column of frequency (m, k1, k2): the lanes of
     // a sub-transform (k1) read VK consecutive k2 each, side by side
     static constexpr int VK = R2 % 4 == 0 ? 4 : R2 % 2 == 0 ? 2 : 1;
@@ -446,6 +447,43 @@ template <class Ge>
 __device__ __forceinline__ int stage1_addr(int j)
 {
     return Lay<Ge>::S1 == Ge::R2 ? j : j + (j / Ge::R2) * (Lay<Ge>::S1 - Ge::R2);
+}
+
+// Loads that pass through once.  Where a square map's U (4 N^2 bytes) stays in
+// the 129 MB L2, T, U and the spectra are kept out of L1, which holds the
+// table w2: inverse row pass 41.3 -> 37.7 us at 4704, 51.5 -> 46.5 at 5376,
+// 73 -> 70 with eight spectra at 2250.  Beyond that the same loads cost more
+// (inverse row pass 709 -> 748, column pass 989 -> 1044 us at 17280: without
+// L1 allocation they fetch less of a line from memory at a time), and stay
+// plain.  The volatile forms are for what the previous grid
+// wrote: they stay behind the wait for it.
+template <class Ge, class V>
+__device__ __forceinline__ V ld_once(const V* p)
+{
+    V v;
+    if constexpr (!Ge::STREAM) {
+        v = *p;
+    } else if constexpr (sizeof(V) == 8) {
+        asm volatile("ld.global.L1::no_allocate.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "l"(p));
+    } else {
+        asm volatile("ld.global.L1::no_allocate.v4.f32 {%0, %1, %2, %3}, [%4];"
+                     : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p));
+    }
+    return v;
+}
+template <class Ge, class V>
+__device__ __forceinline__ V ld_spectrum(const V* p)
+{
+    V v;
+    if constexpr (!Ge::STREAM || sizeof(V) == 4) {
+        v = __ldg(p);
+    } else if constexpr (sizeof(V) == 8) {
+        asm("ld.global.nc.L1::no_allocate.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "l"(p));
+    } else {
+        asm("ld.global.nc.L1::no_allocate.v4.f32 {%0, %1, %2, %3}, [%4];"
+            : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p));
+    }
+    return v;
 }
 
 // the block's copy of w1 (read after the barrier that follows stage 1)
