@@ -823,14 +823,28 @@ extern "C" lp_status lp_spectrum_copy(const lp_spectrum* s, float* dst, size_t d
                        dst_floats, ncols * s->ny * per);
     DeviceGuard dg(s->ctx->device);
     const SpecOrder o = spectrum_order(s->ny, s->prec);
-    if (o.r0 > 0) {
-        CUDA_TRY(spectrum_copy_natural(s->data, s->ldK, s->ny, (int)ncols, s->is_real, o, dst,
-                                       static_cast<cudaStream_t>(stream)));
+    const cudaStream_t st = static_cast<cudaStream_t>(stream);
+    const size_t col = (size_t)s->ny * per * 4;
+    if (o.r0 == 0) {
+        CUDA_TRY(cudaMemcpy2DAsync(dst, col, s->data, (size_t)s->ldK * per * 4, col, ncols, cudaMemcpyDeviceToDevice, st));
         return LP_OK;
     }
-    CUDA_TRY(cudaMemcpy2DAsync(dst, (size_t)s->ny * per * 4, s->data, (size_t)s->ldK * per * 4,
-                               (size_t)s->ny * per * 4, ncols, cudaMemcpyDeviceToDevice,
-                               static_cast<cudaStream_t>(stream)));
+    // The reordering kernel writes whole values to this device's memory; any
+    // other destination that a copy takes gets one from a reordered buffer.
+    cudaPointerAttributes pa;
+    if (cudaPointerGetAttributes(&pa, dst) != cudaSuccess) {
+        (void)cudaGetLastError();
+        pa.type = cudaMemoryTypeUnregistered;
+    }
+    const bool direct = (uintptr_t)dst % (per * 4) == 0 && pa.type == cudaMemoryTypeDevice && pa.device == s->ctx->device;
+    float* out = dst;
+    if (!direct) CUDA_TRY(pool_alloc(s->ctx, col * ncols, (void**)&out, st));
+    cudaError_t e = spectrum_copy_natural(s->data, s->ldK, s->ny, (int)ncols, s->is_real, o, out, st);
+    if (!direct) {
+        if (e == cudaSuccess) e = cudaMemcpyAsync(dst, out, col * ncols, cudaMemcpyDeviceToDevice, st);
+        cudaFreeAsync(out, st);
+    }
+    CUDA_TRY(e);
     return LP_OK;
 }
 

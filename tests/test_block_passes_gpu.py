@@ -98,3 +98,22 @@ def test_spectrum_build_of_each_symmetry(ctx, kind, ny, nx, hk, wk):
     g = got.double().cpu().numpy()
     diff = np.abs(g[..., 0] - S.real) if real else np.hypot(g[..., 0] - S.real, g[..., 1] - S.imag)
     assert diff.max() <= 1.2e-7 * np.abs(S).max()
+
+
+@pytest.mark.parametrize("offset", [0, 1])
+def test_spectrum_copy_takes_any_float_address(ctx, offset):
+    """A complex spectrum to a destination of 4-byte alignment: the same values
+    as to an aligned one, nothing before or behind them."""
+    import torch
+    from paper_1907_02891_gb300 import lp
+    K = torch.rand(5, 7, dtype=torch.float64, device="cuda") + 0.01
+    spec = lp.lp_kernel_spectrum(ctx, K, pad_ny=96, pad_nx=64)
+    n = 33 * 96 * 2
+    aligned = torch.empty(n, device="cuda")
+    buf = torch.full((n + 4,), -7.0, device="cuda")
+    lp.lp_spectrum_copy(spec, aligned)
+    lp.lp_spectrum_copy(spec, buf[offset:offset + n])
+    lp.lp_sync_status(ctx)
+    lp.lp_spectrum_release(ctx, spec)
+    assert torch.equal(buf[offset:offset + n], aligned)
+    assert (buf[:offset] == -7).all() and (buf[offset + n:] == -7).all()
