@@ -41,11 +41,10 @@ NVCC_FLAGS = ["-O3", "-std=c++17", "--expt-relaxed-constexpr", "-lineinfo",
 # radices the in-register DFTs are instantiated for (7-smooth, <= 32)
 RADICES = (2, 3, 4, 5, 6, 7, 8, 9, 10, 12, 14, 15, 16, 18, 20, 21, 24, 25, 27, 28, 30, 32)
 MAX_THREADS = 1024
-PF_UNITS = 2          # work units per block of the prefetching kernels
 # trigger of the next pass at block exit for the forward row pass and the
-# one-spectrum column pass (the inverse row pass triggers at block start):
-# measured faster or equal on the whole map at 4608, 4704, 8820 (one and 16
-# spectra) and 17280
+# one-spectrum column pass; the inverse row pass triggers at block start.
+# Whole maps, against all three at block start: 15.3 / 18.3 us at 1260, 127.1 /
+# 130.9 at 4704, 555 / 558 at 8820, 2378 / 2387 at 17280; 480 equal
 DEFAULT_LATE = [1, 1, 0]
 SMEM_LIMIT = 227 * 1024
 
@@ -60,10 +59,6 @@ SIZES = (
     8192, 8400, 8640, 8820, 9000, 9216,
     10080, 10752, 12288, 13440, 15360, 16384, 17280,
 )
-
-
-def spad_size(n: int) -> int:
-    return n + (n >> 5) + 1
 
 
 def factorizations(n: int, max_stages: int = 4) -> List[Tuple[int, ...]]:
@@ -89,10 +84,9 @@ def threads_for(n: int, radices: Sequence[int]) -> int:
 
 
 def choose_plan(n: int) -> Tuple[int, ...]:
-    """Fewest stages; then the smallest largest radix (register pressure);
-    then the largest smallest radix (fewer threads).  Forward order is
-    descending, so the last forward radix -- whose outputs stay in registers
-    across the spectrum product -- is the smallest."""
+    """Radices of the tensor-core column pass: fewest stages; then the
+    smallest largest radix (register pressure); then the largest smallest
+    radix (fewer threads); descending."""
     best = None
     for f in factorizations(n):
         if threads_for(n, f) > MAX_THREADS:
@@ -222,32 +216,18 @@ def tuned_json_path() -> str:
 
 def plan_table_entry(n: int) -> dict:
     """Heuristic plan of one length (used when the autotuner has not
-    measured it)."""
+    measured it).  `radices` and `threads` are the tensor-core column pass's;
+    `geo` is the FP32 passes'.  upb, minb, pf and db are fields of the plan
+    files' form that no kernel reads."""
     r = choose_plan(n)
-    t = threads_for(n, r)
-    smem = 8 * (n + n // 16 + 16)   # upper bound of the padded extent
-    if smem > SMEM_LIMIT:
-        raise ValueError(f"length {n} needs {smem} bytes of shared memory")
-
-    def fits(f: int) -> bool:
-        return f * t <= MAX_THREADS and f * smem <= 100 * 1024
-
-    # transforms per block of the one-unit-per-block row kernels: two when
-    # they fit (32-byte column segments in T and U), one otherwise; more for
-    # tiny lengths
-    f = 1
-    for cand in (8, 4, 2):
-        if fits(cand) and (cand <= 2 or cand * t <= 256):
-            f = cand
-            break
-    return dict(radices=list(r), threads=t, f1=f, f3=f, smem=smem,
-                upb=[PF_UNITS] * 3, minb=[1, 1, 1], kstage=True, tt=0, pf=[1, 1, 1], db=[0, 0, 0],
+    return dict(radices=list(r), threads=threads_for(n, r), upb=[1] * 3, minb=[1] * 3, pf=[1] * 3, db=[0] * 3,
                 batch=True, geo=geo_plan(choose_geo(n)))
 
 
 def plan_table() -> Dict[int, dict]:
     """Plan of every supported length: the autotuner's measured choice from
-    tuned_plans.json where there is one, the heuristic otherwise."""
+    tuned_plans.json where there is one, the heuristic otherwise (a plan
+    without a geometry gets the heuristic one)."""
     tuned = {}
     path = tuned_json_path()
     if os.path.exists(path):
@@ -259,13 +239,9 @@ def plan_table() -> Dict[int, dict]:
         t = tuned.get(str(n))
         if t:
             e.update(radices=list(t["radices"]), threads=threads_for(n, t["radices"]),
-                     upb=list(t["upb"]), minb=list(t["minb"]), kstage=bool(t["kstage"]),
-                     tt=int(t.get("tt", 0)), pf=list(t.get("pf", [1, 1, 1])),
+                     upb=list(t["upb"]), minb=list(t["minb"]), pf=list(t.get("pf", [1, 1, 1])),
                      db=list(t.get("db", [0, 0, 0])), batch=bool(t.get("batch", True)),
-                     kst2=bool(t.get("kst2", False)), packed=bool(t.get("packed", False)),
-                     late=list(t.get("late", DEFAULT_LATE)))
-            if e["tt"]:
-                e["threads"] = e["tt"]
+                     packed=bool(t.get("packed", False)), late=list(t.get("late", DEFAULT_LATE)))
             if "geo" in t:
                 e["geo"] = dict(t["geo"])
         table[n] = e

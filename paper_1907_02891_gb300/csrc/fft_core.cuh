@@ -8,8 +8,7 @@
 // paper cites for FFTs (Sec. 2.3), one butterfly stage per factor of N: in
 // place, three factors at most, for the FP32 passes (block transforms
 // below), and in the self-sorting (Stockham) order, stage s of
-// N = R_0 R_1 ... R_{S-1}, for the tensor-core column pass and the FP64
-// spectrum build: with Ns = R_0 ... R_{s-1} and butterfly j in [0, N/R_s)
+// N = R_0 R_1 ... R_{S-1}, for the tensor-core column pass: with Ns = R_0 ... R_{s-1} and butterfly j in [0, N/R_s)
 //   inputs   x[j + m N/R_s],                      m = 0..R_s-1
 //   twiddle  x_m *= exp(DIR i 2 pi (j mod Ns) m / (Ns R_s))
 //   DFT of size R_s in registers
