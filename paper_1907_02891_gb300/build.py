@@ -308,7 +308,7 @@ cudaError_t set_attrs()
 
 cudaError_t p1(const P1Args& a, cudaStream_t s)
 {{
-    return launch_pdl(p1_rows<C1>, dim3((a.npairs - a.pair0 + C1::NT - 1) / C1::NT), dim3(C1::TH), C1::SMEM, s, a);
+    return launch_pdl(p1_rows<C1>, dim3((a.npairs - a.pair0 + C1::NT - 1) / C1::NT, a.nmaps), dim3(C1::TH), C1::SMEM, s, a);
 }}
 
 cudaError_t p2(const P2Args& a, bool kreal, cudaStream_t s)

@@ -1095,8 +1095,9 @@ static long long k_extent(const lp_spectrum* s) { return (long long)(s->bytes / 
 static lp_status launch_rows_forward(lp_ctx* ctx, const PlanRec* px, const float* L, int h, int w, int ldl,
                                      const MapDims& d, float2* T, int pair0, int pair1, cudaStream_t st)
 {
-    P1Args a1;
-    a1.L = L;
+    P1Args a1 = {};
+    a1.L[0] = L;
+    a1.nmaps = 1;
     a1.ldl = ldl;
     a1.H = h;
     a1.W = w;
@@ -1603,22 +1604,22 @@ extern "C" lp_status lp_map_multiclass(lp_ctx* ctx, const float* const* L, int T
     float2* accb = park_of(d, U, 1);
     const int npairs = (int)(d.ldT / 2);
     if ((st = lp_wait_spectra_built(spectra, T, s)) != LP_OK) return st;
-    for (int t = 0; t < T; ++t) {
-        P1Args a1;
-        a1.L = L[t];
-        a1.ldl = ldl;
-        a1.H = h;
-        a1.W = w;
-        a1.T = Tb + (size_t)t * d.ncolsT * d.ldT;
-        a1.ldT = d.ldT;
-        a1.pair0 = 0;
-        a1.npairs = npairs;
-        a1.ncols = d.ncols;
-        a1.tw = px->blk;
-        a1.err = ctx->d_err;
-        a1.t_elems = t_extent(ctx, d);
-        CUDA_TRY(px->k->p1(a1, s));
-    }
+    P1Args a1 = {};
+    for (int t = 0; t < T; ++t) a1.L[t] = L[t];
+    a1.nmaps = T;
+    a1.ldl = ldl;
+    a1.H = h;
+    a1.W = w;
+    a1.T = Tb;
+    a1.ldT = d.ldT;
+    a1.specT = (long long)d.ncolsT * d.ldT;
+    a1.pair0 = 0;
+    a1.npairs = npairs;
+    a1.ncols = d.ncols;
+    a1.tw = px->blk;
+    a1.err = ctx->d_err;
+    a1.t_elems = t_extent(ctx, d);
+    CUDA_TRY(px->k->p1(a1, s));
     // the real-spectrum kernel needs every class's spectrum real
     bool all_real = true;
     for (int t = 0; t < T; ++t) all_real = all_real && spectra[t]->is_real;

@@ -117,3 +117,29 @@ def test_spectrum_copy_takes_any_float_address(ctx, offset):
     lp.lp_spectrum_release(ctx, spec)
     assert torch.equal(buf[offset:offset + n], aligned)
     assert (buf[:offset] == -7).all() and (buf[offset + n:] == -7).all()
+
+
+@pytest.mark.parametrize("classes,h", [(1, 90), (2, 91), (32, 1)])
+def test_row_pass_of_several_classes(ctx, classes, h):
+    """One launch of the forward row pass for all classes' maps, the most that
+    the entry takes among them, against the sum of single maps.  Tolerance: a
+    class's two results differ by TOL of its maximum at most, and no class's
+    maximum is above the total's (all values are positive)."""
+    import torch
+    from paper_1907_02891_gb300 import lp
+    rng = np.random.default_rng(classes)
+    spectra, maps = [], []
+    total = torch.zeros(h, 88, dtype=torch.float64, device="cuda")
+    out = torch.empty(h, 88, device="cuda")
+    for i in range(classes):
+        K = torch.from_numpy(np.ascontiguousarray(_psf(rng, 7, 5, True))).cuda()
+        spectra.append(lp.lp_kernel_spectrum(ctx, K, pad_ny=120, pad_nx=96))
+        maps.append(torch.from_numpy(rng.random((h, 88), dtype=np.float32)).cuda())
+        lp.lp_map(ctx, maps[i], [spectra[i]], [out])
+        lp.lp_sync_status(ctx)
+        total += out.double()
+    lp.lp_map_multiclass(ctx, maps, spectra, out)
+    lp.lp_sync_status(ctx)
+    for s in spectra:
+        lp.lp_spectrum_release(ctx, s)
+    assert (out.double() - total).abs().max().item() <= classes * TOL * total.abs().max().item()
