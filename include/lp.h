@@ -150,14 +150,18 @@ lp_status lp_spectrum_info(const lp_spectrum* s, int* ny, int* nx, int* hk, int*
  * (nx/2+1) rows x ny, row c holding the column-frequency c of every
  * row-frequency u; FP32 real (is_real) or interleaved complex, scaled by
  * 1/(2 ny nx).  dst_floats must be >= (nx/2+1)*ny*(is_real ? 1 : 2).
+ * Asynchronous on `stream`.  Like a map, the copy waits in stream order for
+ * the spectrum's build (on whichever stream that runs), and the spectrum may
+ * be released as soon as the call has returned.
  */
 lp_status lp_spectrum_copy(const lp_spectrum* s, float* dst, size_t dst_floats, void* stream);
 
 /*
  * Drop one reference.  When the last one goes the handle becomes invalid at
  * once, but the device memory is freed in stream order: only after the
- * spectrum's build and every map call already enqueued with it (on any
- * stream) have completed.  The call never waits for the device; memory
+ * spectrum's build and every map call and copy already enqueued with it (on
+ * any stream) have completed.  (Calls captured into a CUDA graph are not
+ * seen: the spectrum must be kept while the graph may run.)  The call never waits for the device; memory
  * still held is freed by a later lp_kernel_spectrum, lp_spectrum_release,
  * lp_map or lp_sync_status call, or by lp_destroy.
  */

@@ -813,17 +813,12 @@ extern "C" lp_status lp_spectrum_info(const lp_spectrum* s, int* ny, int* nx, in
     return LP_OK;
 }
 
-extern "C" lp_status lp_spectrum_copy(const lp_spectrum* s, float* dst, size_t dst_floats, void* stream)
+// the copy itself, on stream st
+static lp_status enqueue_spectrum_copy(const lp_spectrum* s, float* dst, cudaStream_t st)
 {
-    if (!s || !dst) return lp_fail(LP_ERR_INVALID, "lp_spectrum_copy: NULL argument");
     const size_t per = s->is_real ? 1 : 2;
     const size_t ncols = (size_t)s->nx / 2 + 1;
-    if (dst_floats < ncols * s->ny * per)
-        return lp_fail(LP_ERR_INVALID, "lp_spectrum_copy: destination holds %zu floats, need %zu",
-                       dst_floats, ncols * s->ny * per);
-    DeviceGuard dg(s->ctx->device);
     const SpecOrder o = spectrum_order(s->ny, s->prec);
-    const cudaStream_t st = static_cast<cudaStream_t>(stream);
     const size_t col = (size_t)s->ny * per * 4;
     if (o.r0 == 0) {
         CUDA_TRY(cudaMemcpy2DAsync(dst, col, s->data, (size_t)s->ldK * per * 4, col, ncols, cudaMemcpyDeviceToDevice, st));
@@ -846,6 +841,25 @@ extern "C" lp_status lp_spectrum_copy(const lp_spectrum* s, float* dst, size_t d
     }
     CUDA_TRY(e);
     return LP_OK;
+}
+
+extern "C" lp_status lp_spectrum_copy(const lp_spectrum* s, float* dst, size_t dst_floats, void* stream)
+{
+    if (!s || !dst) return lp_fail(LP_ERR_INVALID, "lp_spectrum_copy: NULL argument");
+    const size_t need = ((size_t)s->nx / 2 + 1) * s->ny * (s->is_real ? 1 : 2);
+    if (dst_floats < need)
+        return lp_fail(LP_ERR_INVALID, "lp_spectrum_copy: destination holds %zu floats, need %zu", dst_floats, need);
+    DeviceGuard dg(s->ctx->device);
+    const cudaStream_t st = static_cast<cudaStream_t>(stream);
+    // A copy reads the spectrum as a map does: after its build, and before
+    // its memory goes back to the pool.  (Inside a stream capture neither, as
+    // for a map: the caller keeps the spectrum while the graph may run.)
+    if (lp_stream_capturing(st)) return enqueue_spectrum_copy(s, dst, st);
+    const lp_status ws = lp_wait_spectra_built(&s, 1, st);
+    if (ws != LP_OK) return ws;
+    const lp_status cs = enqueue_spectrum_copy(s, dst, st);
+    lp_note_spectra_used(s->ctx, &s, 1, st);
+    return cs;
 }
 
 static void free_spectrum(lp_ctx* ctx, lp_spectrum* s)

@@ -1,0 +1,108 @@
+"""What still reads a spectrum holds its memory: releases with work in
+flight, on other streams than the one that builds the next spectrum.  The
+results compared are the same kernels' on the same values, so they are equal
+bit for bit."""
+
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+from paper_1907_02891_gb300 import lp  # noqa: E402
+
+DEV = "cuda:0"
+SIDE = 2250                      # of the spectra under test: 20 MB complex
+
+
+@pytest.fixture()
+def ctx():
+    c = lp.lp_create(0)
+    yield c
+    lp.lp_destroy(c)
+
+
+def _psf(seed, side=31):
+    """Not point-symmetric: a complex spectrum."""
+    return torch.from_numpy(np.random.default_rng(seed).uniform(0.1, 1.0, (side, side))).to(DEV)
+
+
+def _copy_buffer():
+    return torch.full((SIDE // 2 + 1, SIDE, 2), float("nan"), device=DEV)
+
+
+class _Busy:
+    """Keeps a stream busy for tens of milliseconds: maps of a spectrum of its own."""
+
+    def __init__(self, ctx, stream):
+        self.ctx, self.stream = ctx, stream
+        self.spec = lp.lp_kernel_spectrum(ctx, _psf(100), pad_ny=8192, pad_nx=8192)
+        self.L = torch.ones(8000, 8000, device=DEV)
+        self.out = torch.empty_like(self.L)
+        lp.lp_sync_status(ctx)
+        lp.lp_map(ctx, self.L, [self.spec], [self.out], stream=stream)   # the stream's workspace
+        lp.lp_sync_status(ctx, stream=stream)
+
+    def start(self):
+        for _ in range(100):
+            lp.lp_map(self.ctx, self.L, [self.spec], [self.out], stream=self.stream)
+
+    def running(self):
+        return lp.lp_sync_status_code(self.ctx, stream=self.stream, timeout_ms=0) == lp.LP_ERR_TIMEOUT
+
+
+@pytest.mark.parametrize("symmetric,prec", [(False, lp.LP_PREC_FP32), (True, lp.LP_PREC_FP32),
+                                            (False, lp.LP_PREC_SPLIT_BF16)])
+def test_release_with_a_copy_in_flight(ctx, symmetric, prec):
+    """A copy queued behind other work, the spectrum released, and another
+    PSF's spectrum of the same size built on another stream: the memory is
+    still held, and the copy has the first spectrum's values."""
+    a, b = torch.cuda.Stream(), torch.cuda.Stream()
+    busy = _Busy(ctx, a)
+    side = next(n for n in lp.supported_sizes() if n >= SIDE and (prec == lp.LP_PREC_FP32 or lp.lp_split_supported(n)))
+
+    def build(seed, stream=None):
+        K = _psf(seed)
+        if symmetric:
+            K = K + K.flip(0, 1)
+        torch.cuda.synchronize()
+        return lp.lp_kernel_spectrum(ctx, K, pad_ny=side, pad_nx=side, prec=prec, stream=stream)
+
+    spec = build(1)
+    want, got = (torch.full((side // 2 + 1, side, 1 if symmetric else 2), float("nan"), device=DEV) for _ in range(2))
+    lp.lp_spectrum_copy(spec, want)
+    lp.lp_sync_status(ctx)
+    K2 = _psf(2)
+    if symmetric:
+        K2 = K2 + K2.flip(0, 1)
+    torch.cuda.synchronize()
+    held = lp.lp_bytes_in_use(ctx)
+    busy.start()
+    lp.lp_spectrum_copy(spec, got, stream=a)
+    lp.lp_spectrum_release(ctx, spec)
+    after_release = lp.lp_bytes_in_use(ctx)
+    other = lp.lp_kernel_spectrum(ctx, K2, pad_ny=side, pad_nx=side, prec=prec, stream=b)
+    after_build = lp.lp_bytes_in_use(ctx)
+    assert busy.running(), "the stream drained before the release could be told from a wait"
+    lp.lp_sync_status(ctx, stream=b)
+    lp.lp_sync_status(ctx, stream=a)
+    assert after_release == held
+    assert after_build > held
+    assert torch.equal(got, want)
+    lp.lp_sync_status(ctx)
+    assert lp.lp_bytes_in_use(ctx) == held       # the first went, the second of its size came
+    lp.lp_spectrum_release(ctx, other)
+
+
+def test_copy_waits_for_a_build_on_another_stream(ctx):
+    s_build, s_copy = torch.cuda.Stream(), torch.cuda.Stream()
+    got, want = (torch.full((8820 // 2 + 1, 8820, 2), float("nan"), device=DEV) for _ in range(2))
+    K = _psf(3, 601)
+    torch.cuda.synchronize()
+    spec = lp.lp_kernel_spectrum(ctx, K, pad_ny=8820, pad_nx=8820, stream=s_build)
+    lp.lp_spectrum_copy(spec, got, stream=s_copy)
+    torch.cuda.synchronize()
+    lp.lp_spectrum_copy(spec, want)
+    lp.lp_sync_status(ctx)
+    assert torch.equal(got, want)
+    lp.lp_spectrum_release(ctx, spec)
