@@ -957,19 +957,28 @@ lp_status lp_wait_spectra_built(const lp_spectrum* const* spectra, int n, cudaSt
 
 void lp_note_spectra_used(lp_ctx* ctx, const lp_spectrum* const* spectra, int n, cudaStream_t st)
 {
+    unsigned long long id = 0;
+    const bool known = cudaStreamGetId(st, &id) == cudaSuccess;
+    if (!known) cudaGetLastError();
     std::lock_guard<std::mutex> g(ctx->spec_mu);
     for (int k = 0; k < n; ++k) {
         lp_spectrum* s = const_cast<lp_spectrum*>(spectra[k]);
         int slot = -1;
         for (int i = 0; i < s->nuse; ++i)
-            if (s->use_stream[i] == st) slot = i;
-        if (slot < 0) {
-            if (s->nuse == lp_spectrum::kUseSlots) {
-                s->use_overflow = true;
-                continue;
+            if (s->use_stream[i] == id) slot = i;
+        // (all taken: one whose use is complete)
+        for (int i = 0; slot < 0 && s->nuse == lp_spectrum::kUseSlots && i < s->nuse; ++i)
+            if (s->use_event[i] && cudaEventQuery(s->use_event[i]) == cudaSuccess) {
+                slot = i;
+                s->use_stream[i] = id;
             }
+        if (!known || (slot < 0 && s->nuse == lp_spectrum::kUseSlots)) {
+            s->use_overflow = true;
+            continue;
+        }
+        if (slot < 0) {
             slot = s->nuse++;
-            s->use_stream[slot] = st;
+            s->use_stream[slot] = id;
         }
         if ((!s->use_event[slot] &&
              cudaEventCreateWithFlags(&s->use_event[slot], cudaEventDisableTiming) != cudaSuccess) ||

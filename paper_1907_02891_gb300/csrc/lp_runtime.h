@@ -79,11 +79,15 @@ struct lp_spectrum {
     // the requested PSF with it value by value
     double* kcopy = nullptr;
     size_t kbytes = 0;
-    // Last use per stream, for stream-ordered release: every map call
-    // re-records the event of its stream's slot at its end.  Streams beyond
-    // the slots set `use_overflow`, and the release then waits for the device.
+    // Last use per stream, for stream-ordered release: every map call and
+    // copy re-records the event of its stream's slot at its end.  Slots go by
+    // the stream's id, not its handle: a handle is given to another stream
+    // once its own is destroyed (whose work may still be running), and
+    // cudaStreamPerThread is one handle for every thread's stream.  With
+    // more streams in flight than slots `use_overflow` is set, and only a wait
+    // for the device frees the spectrum.
     static constexpr int kUseSlots = 8;
-    cudaStream_t use_stream[kUseSlots] = {};
+    unsigned long long use_stream[kUseSlots] = {};
     cudaEvent_t use_event[kUseSlots] = {};
     int nuse = 0;
     bool use_overflow = false;

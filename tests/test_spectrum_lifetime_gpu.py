@@ -3,6 +3,8 @@ flight, on other streams than the one that builds the next spectrum.  The
 results compared are the same kernels' on the same values, so they are equal
 bit for bit."""
 
+from concurrent.futures import ThreadPoolExecutor
+
 import numpy as np
 import pytest
 
@@ -106,3 +108,45 @@ def test_copy_waits_for_a_build_on_another_stream(ctx):
     lp.lp_sync_status(ctx)
     assert torch.equal(got, want)
     lp.lp_spectrum_release(ctx, spec)
+
+
+def test_uses_go_by_stream_not_by_handle(ctx):
+    """cudaStreamPerThread (handle 2) is another stream in every thread: a
+    finished use in one thread says nothing about another's."""
+    worker = ThreadPoolExecutor(1)              # one thread, its per-thread stream
+
+    def there(f, *a, **k):
+        return worker.submit(f, *a, **k).result()
+
+    busy = there(_Busy, ctx, 2)
+    spec = lp.lp_kernel_spectrum(ctx, _psf(4), pad_ny=SIDE, pad_nx=SIDE)
+    want, got, here = (_copy_buffer() for _ in range(3))
+    lp.lp_spectrum_copy(spec, want)
+    lp.lp_sync_status(ctx)
+    held = lp.lp_bytes_in_use(ctx)
+    there(busy.start)
+    there(lp.lp_spectrum_copy, spec, got, stream=2)
+    lp.lp_spectrum_copy(spec, here, stream=2)
+    torch.cuda.ExternalStream(2).synchronize()  # this thread's
+    lp.lp_spectrum_release(ctx, spec)
+    after_release = lp.lp_bytes_in_use(ctx)
+    assert there(busy.running)
+    there(lp.lp_sync_status, ctx, stream=2)
+    assert after_release == held
+    assert lp.lp_bytes_in_use(ctx) < held
+    assert torch.equal(got, want) and torch.equal(here, want)
+    worker.shutdown()
+
+
+def test_release_after_uses_on_many_streams(ctx):
+    """More streams than a spectrum keeps use events for, one after the other."""
+    spec = lp.lp_kernel_spectrum(ctx, _psf(5), pad_ny=SIDE, pad_nx=SIDE)
+    dst = _copy_buffer()
+    torch.cuda.synchronize()
+    held = lp.lp_bytes_in_use(ctx)
+    for _ in range(12):
+        s = torch.cuda.Stream()
+        lp.lp_spectrum_copy(spec, dst, stream=s)
+        s.synchronize()
+    lp.lp_spectrum_release(ctx, spec)
+    assert lp.lp_bytes_in_use(ctx) < held
