@@ -1699,7 +1699,9 @@ extern "C" lp_status lp_map_multiclass(lp_ctx* ctx, const float* const* L, int T
     a3.err = ctx->d_err;
     a3.u_elems = (long long)d.ncolsU * d.ldU;
     CUDA_TRY(px->k->p3(a3, 1, s));
-    lp_note_spectra_used(ctx, spectra, T, s);
+    // (not inside a stream capture, where recording would take the event of
+    // this stream's earlier work with these spectra into the capture)
+    if (!lp_stream_capturing(s)) lp_note_spectra_used(ctx, spectra, T, s);
     return LP_OK;
 }
 

@@ -3,6 +3,7 @@ flight, on other streams than the one that builds the next spectrum.  The
 results compared are the same kernels' on the same values, so they are equal
 bit for bit."""
 
+import ctypes
 from concurrent.futures import ThreadPoolExecutor
 
 import numpy as np
@@ -108,6 +109,69 @@ def test_copy_waits_for_a_build_on_another_stream(ctx):
     lp.lp_sync_status(ctx)
     assert torch.equal(got, want)
     lp.lp_spectrum_release(ctx, spec)
+
+
+class _Capture:
+    """Capture of a stream into a graph of its own, by the driver's calls
+    (torch's synchronises the device first)."""
+
+    def __init__(self, stream):
+        self.cuda, self.stream = ctypes.CDLL("libcuda.so.1"), ctypes.c_void_p(stream.cuda_stream)
+
+    def __enter__(self):
+        assert self.cuda.cuStreamBeginCapture_v2(self.stream, 2) == 0       # relaxed
+        return self
+
+    def __exit__(self, *exc):
+        self.graph = ctypes.c_void_p()
+        assert self.cuda.cuStreamEndCapture(self.stream, ctypes.byref(self.graph)) == 0
+
+    def node_types(self):
+        n = ctypes.c_size_t()
+        assert self.cuda.cuGraphGetNodes(self.graph, None, ctypes.byref(n)) == 0
+        nodes, kind, kinds = (ctypes.c_void_p * n.value)(), ctypes.c_int(), []
+        assert self.cuda.cuGraphGetNodes(self.graph, nodes, ctypes.byref(n)) == 0
+        for node in nodes:
+            assert self.cuda.cuGraphNodeGetType(ctypes.c_void_p(node), ctypes.byref(kind)) == 0
+            kinds.append(kind.value)
+        return kinds
+
+    def destroy(self):
+        assert self.cuda.cuGraphDestroy(self.graph) == 0
+
+
+@pytest.mark.parametrize("entry", ["map", "multiclass", "copy"])
+def test_capture_leaves_earlier_uses_alone(ctx, entry):
+    """A call captured on a stream does not hide the stream's queued work with
+    the same spectrum from the release."""
+    a = torch.cuda.Stream()
+    busy = _Busy(ctx, a)
+    spec = lp.lp_kernel_spectrum(ctx, _psf(6), pad_ny=SIDE, pad_nx=SIDE)
+    L = torch.ones(2200, 2200, device=DEV)
+    out = torch.empty_like(L)
+    want, got = _copy_buffer(), _copy_buffer()
+    lp.lp_spectrum_copy(spec, want)
+    lp.lp_map_multiclass(ctx, [L], [spec], out, stream=a)       # workspace
+    torch.cuda.synchronize()
+    held = lp.lp_bytes_in_use(ctx)
+    busy.start()
+    lp.lp_spectrum_copy(spec, got, stream=a)
+    with _Capture(a) as c:
+        if entry == "map":
+            lp.lp_map(ctx, L, [spec], [out], stream=a)
+        elif entry == "multiclass":
+            lp.lp_map_multiclass(ctx, [L], [spec], out, stream=a)
+        else:
+            lp.lp_spectrum_copy(spec, got, stream=a)
+    assert 0 in c.node_types()                                  # kernels
+    c.destroy()
+    lp.lp_spectrum_release(ctx, spec)
+    after_release = lp.lp_bytes_in_use(ctx)
+    assert busy.running()
+    lp.lp_sync_status(ctx, stream=a)
+    assert after_release == held
+    assert lp.lp_bytes_in_use(ctx) < held
+    assert torch.equal(got, want)
 
 
 def test_uses_go_by_stream_not_by_handle(ctx):
