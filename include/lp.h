@@ -303,6 +303,10 @@ lp_status lp_sync_status(lp_ctx* ctx, void* stream, int timeout_ms);
  * LP_ERR_DEVICE; no access leaves the real buffer.  The release build
  * compiles the checks away and ignores the hook. */
 #define LP_TEST_BOUNDS 8
+/* LP_TEST_ROWS_FAIL: the next inverse row pass (the last pass of a map)
+ * fails as if its launch had (LP_ERR_CUDA, from the host), then the bit is
+ * cleared; the passes before it have been enqueued. */
+#define LP_TEST_ROWS_FAIL 16
 lp_status lp_set_test_hook(lp_ctx* ctx, int hook);
 
 /*

@@ -813,6 +813,22 @@ extern "C" lp_status lp_spectrum_info(const lp_spectrum* s, int* ny, int* nx, in
     return LP_OK;
 }
 
+// Records the use of a call's spectra when the call returns, after the last
+// thing it has enqueued (an event between the passes would stop the next
+// pass's launch from overlapping the previous one's tail), and also when it
+// returns early with an error: what it had enqueued by then still reads them.
+struct SpectraUse {
+    lp_ctx* ctx;
+    const lp_spectrum* const* spectra;
+    int n;
+    cudaStream_t st;
+    bool record;  // not inside a stream capture
+    ~SpectraUse()
+    {
+        if (record) lp_note_spectra_used(ctx, spectra, n, st);
+    }
+};
+
 // the copy itself, on stream st
 static lp_status enqueue_spectrum_copy(const lp_spectrum* s, float* dst, cudaStream_t st)
 {
@@ -857,9 +873,8 @@ extern "C" lp_status lp_spectrum_copy(const lp_spectrum* s, float* dst, size_t d
     if (lp_stream_capturing(st)) return enqueue_spectrum_copy(s, dst, st);
     const lp_status ws = lp_wait_spectra_built(&s, 1, st);
     if (ws != LP_OK) return ws;
-    const lp_status cs = enqueue_spectrum_copy(s, dst, st);
-    lp_note_spectra_used(s->ctx, &s, 1, st);
-    return cs;
+    const SpectraUse use{s->ctx, &s, 1, st, true};
+    return enqueue_spectrum_copy(s, dst, st);
 }
 
 static void free_spectrum(lp_ctx* ctx, lp_spectrum* s)
@@ -987,6 +1002,14 @@ void lp_note_spectra_used(lp_ctx* ctx, const lp_spectrum* const* spectra, int n,
             s->use_overflow = true;
         }
     }
+}
+
+// test hook: the next inverse row pass fails as its launch would
+static lp_status injected_row_failure(lp_ctx* ctx)
+{
+    if ((ctx->test_hook.load() & LP_TEST_ROWS_FAIL) && (ctx->test_hook.fetch_and(~LP_TEST_ROWS_FAIL) & LP_TEST_ROWS_FAIL))
+        return lp_fail(LP_ERR_CUDA, "injected launch failure (LP_TEST_ROWS_FAIL)");
+    return LP_OK;
 }
 
 // ---------------------------------------------------------------------------
@@ -1237,6 +1260,8 @@ static lp_status launch_rows_inverse(lp_ctx* ctx, const PlanRec* px, const MapDi
     a3.tw = px->blk;
     a3.err = ctx->d_err;
     a3.u_elems = (long long)cnt * d.ncolsU * d.ldU;
+    const lp_status is = injected_row_failure(ctx);
+    if (is != LP_OK) return is;
     const int tok = lp_pass_begin(ctx, 2, st);
     CUDA_TRY(px->k->p3(a3, cnt, st));
     lp_pass_end(ctx, tok, st);
@@ -1280,6 +1305,7 @@ lp_status lp_launch_map(lp_ctx* ctx, const float* L, int h, int w, int ldl,
     } else if ((ps = lp_wait_spectra_built(spectra, n, st)) != LP_OK) {
         return ps;
     }
+    const SpectraUse use{ctx, spectra, n, st, !capturing};
     if ((ps = launch_rows_forward(ctx, px, L, h, w, ldl, d, T, 0, (int)(d.ldT / 2), st)) != LP_OK) return ps;
     for (int base = 0; base < n; base += kMaxSpectraPerLaunch) {
         const int cnt = (n - base) < kMaxSpectraPerLaunch ? (n - base) : kMaxSpectraPerLaunch;
@@ -1287,9 +1313,6 @@ lp_status lp_launch_map(lp_ctx* ctx, const float* L, int h, int w, int ldl,
         if ((ps = launch_rows_inverse(ctx, px, d, U, cnt, out + base, ldo, 0, (int)(d.ldU / 2), st)) != LP_OK)
             return ps;
     }
-    // recorded after the last pass (an event between the passes would stop
-    // the next pass's launch from overlapping the previous one's tail)
-    if (!capturing) lp_note_spectra_used(ctx, spectra, n, st);
     return LP_OK;
 }
 
@@ -1509,6 +1532,7 @@ extern "C" lp_status lp_map_host(lp_ctx* ctx, const float* L_host, int h, int w,
     else CUDA_TRY(cudaStreamWaitEvent(ctx->hs_in, ev_start, 0));
     CUDA_TRY(cudaStreamWaitEvent(ctx->hs_out, ev_start, 0));
     for (int k = 0; k < n; ++k) CUDA_TRY(cudaStreamWaitEvent(c, spectra[k]->ready, 0));
+    const SpectraUse use{ctx, spectra, n, c, true};
 
     const int npairs = (int)(d.ldT / 2);
     const int nb_in = host_bands(lbytes, npairs);
@@ -1545,7 +1569,6 @@ extern "C" lp_status lp_map_host(lp_ctx* ctx, const float* L_host, int h, int w,
                                            ctx->hs_out));
         }
     }
-    lp_note_spectra_used(ctx, spectra, n, c);
     CUDA_TRY(cudaEventRecord(ctx->hs_ofree[obuf], ctx->hs_out));
     ctx->hs_ofree_valid[obuf] = true;
     ctx->hs_obuf = obuf ^ 1;
@@ -1557,7 +1580,7 @@ extern "C" lp_status lp_map_host(lp_ctx* ctx, const float* L_host, int h, int w,
 extern "C" lp_status lp_set_test_hook(lp_ctx* ctx, int hook)
 {
     if (!ctx) return lp_fail(LP_ERR_INVALID, "lp_set_test_hook: NULL context");
-    if (hook & ~(LP_TEST_TC_NO_MMA | LP_TEST_FP_COLLIDE | LP_TEST_SERVE_FAIL | LP_TEST_BOUNDS))
+    if (hook & ~(LP_TEST_TC_NO_MMA | LP_TEST_FP_COLLIDE | LP_TEST_SERVE_FAIL | LP_TEST_BOUNDS | LP_TEST_ROWS_FAIL))
         return lp_fail(LP_ERR_INVALID, "lp_set_test_hook: unknown hook 0x%x", hook);
     ctx->test_hook = hook;
     return LP_OK;
@@ -1627,6 +1650,9 @@ extern "C" lp_status lp_map_multiclass(lp_ctx* ctx, const float* const* L, int T
     float2* accb = park_of(d, U, 1);
     const int npairs = (int)(d.ldT / 2);
     if ((st = lp_wait_spectra_built(spectra, T, s)) != LP_OK) return st;
+    // (inside a stream capture recording would take the event of this
+    // stream's earlier work with these spectra into the capture)
+    const SpectraUse use{ctx, spectra, T, s, !lp_stream_capturing(s)};
     P1Args a1 = {};
     for (int t = 0; t < T; ++t) a1.L[t] = L[t];
     a1.nmaps = T;
@@ -1698,10 +1724,8 @@ extern "C" lp_status lp_map_multiclass(lp_ctx* ctx, const float* const* L, int T
     a3.tw = px->blk;
     a3.err = ctx->d_err;
     a3.u_elems = (long long)d.ncolsU * d.ldU;
+    if ((st = injected_row_failure(ctx)) != LP_OK) return st;
     CUDA_TRY(px->k->p3(a3, 1, s));
-    // (not inside a stream capture, where recording would take the event of
-    // this stream's earlier work with these spectra into the capture)
-    if (!lp_stream_capturing(s)) lp_note_spectra_used(ctx, spectra, T, s);
     return LP_OK;
 }
 

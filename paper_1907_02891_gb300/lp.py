@@ -299,6 +299,7 @@ LP_TEST_TC_NO_MMA = 1
 LP_TEST_FP_COLLIDE = 2
 LP_TEST_SERVE_FAIL = 4
 LP_TEST_BOUNDS = 8
+LP_TEST_ROWS_FAIL = 16
 
 
 def lp_set_test_hook(ctx: int, hook: int) -> None:

@@ -214,3 +214,50 @@ def test_release_after_uses_on_many_streams(ctx):
         s.synchronize()
     lp.lp_spectrum_release(ctx, spec)
     assert lp.lp_bytes_in_use(ctx) < held
+
+
+@pytest.mark.parametrize("entry", ["map", "tiled", "multiclass", "host", "serve"])
+def test_a_call_that_fails_half_way_holds_its_spectra(ctx, entry):
+    """The column pass is enqueued (behind other work, where the call runs on
+    the caller's stream) when the call fails: its spectrum stays until that
+    pass is done, and not longer."""
+    a = torch.cuda.Stream()
+    busy = _Busy(ctx, a)
+    spec = lp.lp_kernel_spectrum(ctx, _psf(7), pad_ny=SIDE, pad_nx=SIDE)
+    L = torch.ones(2200, 2200, device=DEV)
+    out = torch.empty_like(L)
+    hL, hout = (torch.ones(2200, 2200).pin_memory() for _ in range(2))
+    if entry == "serve":
+        lp.lp_serve_start(ctx, 1)
+
+    def call():
+        if entry == "map":
+            lp.lp_map(ctx, L, [spec], [out], stream=a)
+        elif entry == "tiled":
+            lp.lp_map_tiled(ctx, L, [spec], [out], stream=a)
+        elif entry == "multiclass":
+            lp.lp_map_multiclass(ctx, [L], [spec], out, stream=a)
+        elif entry == "host":
+            lp.lp_map_host(ctx, hL, [spec], [hout], stream=a)
+        else:
+            lp.lp_serve_poll(ctx, lp.lp_serve_submit(ctx, L, [spec], [out]), timeout_ms=60000)
+
+    call()                                                      # workspaces
+    torch.cuda.synchronize()
+    held = lp.lp_bytes_in_use(ctx)
+    if entry in ("map", "tiled", "multiclass"):                 # (the others run on streams of their own)
+        busy.start()
+    lp.lp_set_test_hook(ctx, lp.LP_TEST_ROWS_FAIL)
+    with pytest.raises(lp.LpError) as e:
+        call()
+    assert e.value.status == lp.LP_ERR_CUDA
+    lp.lp_spectrum_release(ctx, spec)
+    if entry in ("map", "tiled", "multiclass"):
+        after_release = lp.lp_bytes_in_use(ctx)
+        assert busy.running()
+        assert after_release == held
+    torch.cuda.synchronize()
+    lp.lp_sync_status(ctx)
+    assert lp.lp_bytes_in_use(ctx) < held
+    if entry == "serve":
+        lp.lp_serve_stop(ctx)
