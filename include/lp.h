@@ -307,6 +307,10 @@ lp_status lp_sync_status(lp_ctx* ctx, void* stream, int timeout_ms);
  * fails as if its launch had (LP_ERR_CUDA, from the host), then the bit is
  * cleared; the passes before it have been enqueued. */
 #define LP_TEST_ROWS_FAIL 16
+/* LP_TEST_OOM: the context's next device allocation is reported as out of
+ * memory the first time it is tried (then the bit is cleared), and takes the
+ * way of a real one: kept memory is given back and the allocation retried. */
+#define LP_TEST_OOM 32
 lp_status lp_set_test_hook(lp_ctx* ctx, int hook);
 
 /*

@@ -169,11 +169,22 @@ static void free_spectrum(lp_ctx* ctx, lp_spectrum* s);
 // ---------------------------------------------------------------------------
 // context internals
 // ---------------------------------------------------------------------------
-// gives the pool's kept memory back; true when there is a pool
+// After an allocation has failed: gives the pool's free memory back; true
+// when there is a pool.  A stream-ordered free counts only once the host has
+// seen it complete, so the device is waited for first: the spectra released
+// last and the scratch of the last build go back too.
 static bool pool_trim(lp_ctx* ctx)
 {
     std::lock_guard<std::mutex> g(ctx->pool_mu);
-    return ctx->pool && cudaMemPoolTrimTo(ctx->pool, 0) == cudaSuccess;
+    if (!ctx->pool) return false;
+    if (cudaDeviceSynchronize() != cudaSuccess) (void)cudaGetLastError();
+    return cudaMemPoolTrimTo(ctx->pool, 0) == cudaSuccess;
+}
+
+// test hook: the next device allocation is reported as out of memory at first
+static bool injected_oom(lp_ctx* ctx)
+{
+    return (ctx->test_hook.load() & LP_TEST_OOM) && (ctx->test_hook.fetch_and(~LP_TEST_OOM) & LP_TEST_OOM);
 }
 
 lp_status lp_ctx_alloc(lp_ctx* ctx, size_t bytes, void** p)
@@ -187,7 +198,7 @@ lp_status lp_ctx_alloc(lp_ctx* ctx, size_t bytes, void** p)
                            bytes, ctx->budget);
         ctx->used += bytes;
     }
-    cudaError_t e = cudaMalloc(p, bytes);
+    cudaError_t e = injected_oom(ctx) ? cudaErrorMemoryAllocation : cudaMalloc(p, bytes);
     if (e == cudaErrorMemoryAllocation && pool_trim(ctx)) {
         (void)cudaGetLastError();
         e = cudaMalloc(p, bytes);
@@ -244,8 +255,8 @@ static cudaError_t pool_alloc(lp_ctx* ctx, size_t bytes, void** p, cudaStream_t 
             pool_keep(ctx, 0);
         }
     }
-    cudaError_t e = cudaMallocFromPoolAsync(p, bytes, ctx->pool, st);
-    if (e == cudaErrorMemoryAllocation && pool_trim(ctx)) {
+    cudaError_t e = injected_oom(ctx) ? cudaErrorMemoryAllocation : cudaMallocFromPoolAsync(p, bytes, ctx->pool, st);
+    if (e == cudaErrorMemoryAllocation && !lp_stream_capturing(st) && pool_trim(ctx)) {
         (void)cudaGetLastError();
         e = cudaMallocFromPoolAsync(p, bytes, ctx->pool, st);
     }
@@ -1580,7 +1591,8 @@ extern "C" lp_status lp_map_host(lp_ctx* ctx, const float* L_host, int h, int w,
 extern "C" lp_status lp_set_test_hook(lp_ctx* ctx, int hook)
 {
     if (!ctx) return lp_fail(LP_ERR_INVALID, "lp_set_test_hook: NULL context");
-    if (hook & ~(LP_TEST_TC_NO_MMA | LP_TEST_FP_COLLIDE | LP_TEST_SERVE_FAIL | LP_TEST_BOUNDS | LP_TEST_ROWS_FAIL))
+    if (hook & ~(LP_TEST_TC_NO_MMA | LP_TEST_FP_COLLIDE | LP_TEST_SERVE_FAIL | LP_TEST_BOUNDS | LP_TEST_ROWS_FAIL |
+                 LP_TEST_OOM))
         return lp_fail(LP_ERR_INVALID, "lp_set_test_hook: unknown hook 0x%x", hook);
     ctx->test_hook = hook;
     return LP_OK;

@@ -300,6 +300,7 @@ LP_TEST_FP_COLLIDE = 2
 LP_TEST_SERVE_FAIL = 4
 LP_TEST_BOUNDS = 8
 LP_TEST_ROWS_FAIL = 16
+LP_TEST_OOM = 32
 
 
 def lp_set_test_hook(ctx: int, hook: int) -> None:

@@ -261,3 +261,29 @@ def test_a_call_that_fails_half_way_holds_its_spectra(ctx, entry):
     assert lp.lp_bytes_in_use(ctx) < held
     if entry == "serve":
         lp.lp_serve_stop(ctx)
+
+
+@pytest.mark.parametrize("by", ["workspace", "build"])
+def test_failed_allocation_gives_kept_memory_back(ctx, by):
+    """An allocation that fails (on the host, by LP_TEST_OOM) right after a
+    spectrum has been released gets its memory: most of the 155 MB that the
+    context would have kept for the next build are the device's again (all but
+    the pool's blocks that hold a live spectrum beside it)."""
+    small = lp.lp_kernel_spectrum(ctx, _psf(8), pad_ny=128, pad_nx=128)
+    K = _psf(9)
+    K = K + K.flip(0, 1)
+    L, out = torch.ones(90, 90, device=DEV), torch.empty(90, 90, device=DEV)
+    big = lp.lp_kernel_spectrum(ctx, K, pad_ny=8820, pad_nx=8820)
+    torch.cuda.synchronize()
+    size = 4 * 4411 * 8820
+    free = torch.cuda.mem_get_info()[0]
+    lp.lp_spectrum_release(ctx, big)
+    lp.lp_set_test_hook(ctx, lp.LP_TEST_OOM)
+    if by == "workspace":
+        lp.lp_map(ctx, L, [small], [out])
+    else:
+        K2 = _psf(10)
+        lp.lp_kernel_spectrum(ctx, K2, pad_ny=128, pad_nx=128)
+    assert torch.cuda.mem_get_info()[0] >= free + size // 2
+    torch.cuda.synchronize()
+    lp.lp_sync_status(ctx)
