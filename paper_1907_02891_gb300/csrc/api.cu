@@ -840,6 +840,27 @@ struct SpectraUse {
     }
 };
 
+// The address at which kernels of the context's device see `bytes` bytes at p
+// (its own memory, managed memory, pinned host memory), or null where they do
+// not or where p is not a float's address.  Looked at at both ends.
+static float* device_view(const lp_ctx* ctx, float* p, size_t bytes)
+{
+    if ((uintptr_t)p % 4 != 0) return nullptr;
+    char* view[2];
+    for (int end = 0; end < 2; ++end) {
+        cudaPointerAttributes pa;
+        if (cudaPointerGetAttributes(&pa, reinterpret_cast<char*>(p) + (end ? bytes - 4 : 0)) != cudaSuccess) {
+            (void)cudaGetLastError();
+            return nullptr;
+        }
+        const bool seen = pa.type == cudaMemoryTypeManaged || pa.type == cudaMemoryTypeHost ||
+                          (pa.type == cudaMemoryTypeDevice && pa.device == ctx->device);
+        view[end] = seen ? static_cast<char*>(pa.devicePointer) : nullptr;
+        if (!view[end]) return nullptr;
+    }
+    return view[1] == view[0] + (bytes - 4) ? reinterpret_cast<float*>(view[0]) : nullptr;
+}
+
 // the copy itself, on stream st
 static lp_status enqueue_spectrum_copy(const lp_spectrum* s, float* dst, cudaStream_t st)
 {
@@ -851,21 +872,18 @@ static lp_status enqueue_spectrum_copy(const lp_spectrum* s, float* dst, cudaStr
         CUDA_TRY(cudaMemcpy2DAsync(dst, col, s->data, (size_t)s->ldK * per * 4, col, ncols, cudaMemcpyDeviceToDevice, st));
         return LP_OK;
     }
-    // The reordering kernel writes whole values to this device's memory; any
-    // other destination that a copy takes gets one from a reordered buffer.
-    cudaPointerAttributes pa;
-    if (cudaPointerGetAttributes(&pa, dst) != cudaSuccess) {
-        (void)cudaGetLastError();
-        pa.type = cudaMemoryTypeUnregistered;
+    // The reordering kernel writes to every destination that this device can
+    // address; any other that a copy takes (another device's memory, pageable
+    // host memory) gets one from a reordered buffer.
+    float* out = device_view(s->ctx, dst, col * ncols);
+    if (out) {
+        CUDA_TRY(spectrum_copy_natural(s->data, s->ldK, s->ny, (int)ncols, s->is_real, o, out, st));
+        return LP_OK;
     }
-    const bool direct = (uintptr_t)dst % (per * 4) == 0 && pa.type == cudaMemoryTypeDevice && pa.device == s->ctx->device;
-    float* out = dst;
-    if (!direct) CUDA_TRY(pool_alloc(s->ctx, col * ncols, (void**)&out, st));
+    CUDA_TRY(pool_alloc(s->ctx, col * ncols, (void**)&out, st));
     cudaError_t e = spectrum_copy_natural(s->data, s->ldK, s->ny, (int)ncols, s->is_real, o, out, st);
-    if (!direct) {
-        if (e == cudaSuccess) e = cudaMemcpyAsync(dst, out, col * ncols, cudaMemcpyDeviceToDevice, st);
-        cudaFreeAsync(out, st);
-    }
+    if (e == cudaSuccess) e = cudaMemcpyAsync(dst, out, col * ncols, cudaMemcpyDeviceToDevice, st);
+    cudaFreeAsync(out, st);
     CUDA_TRY(e);
     return LP_OK;
 }

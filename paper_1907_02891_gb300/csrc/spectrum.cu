@@ -398,44 +398,50 @@ cudaError_t psf_spectrum_build(const double* K, int hk, int wk, int Ny, int Nx, 
 }
 
 // One stored column to natural order, by way of shared memory (reading the
-// gathered order straight from memory took 52 us at 4704 x 4704, this 28)
-template <class V>
+// gathered order straight from memory took 52 us at 4704 x 4704, this 28).
+// The destination is written as D: whole values, or the floats of complex ones
+// where it is not aligned for them.
+template <class V, class D>
 __global__ void __launch_bounds__(256) spectrum_natural(const V* __restrict__ src, long long ldK, int ny, SpecOrder order,
-                                                        V* __restrict__ dst)
+                                                        D* __restrict__ dst)
 {
     extern __shared__ __align__(16) unsigned char smn[];
+    constexpr int PER = sizeof(V) / sizeof(D);
     V* col = reinterpret_cast<V*>(smn);
     src += (long long)blockIdx.x * ldK;
-    dst += (long long)blockIdx.x * ny;
+    dst += (long long)blockIdx.x * ny * PER;
     // (one element of padding per 32: a step of one in m may be a multiple of
     // 32 positions)
     for (int p = threadIdx.x; p < ny; p += blockDim.x) col[p + (p >> 5)] = src[p];
     __syncthreads();
-    for (int u = threadIdx.x; u < ny; u += blockDim.x) {
-        const int p = spec_pos(order, u);
-        dst[u] = col[p + (p >> 5)];
+    const D* val = reinterpret_cast<const D*>(smn);
+    for (int i = threadIdx.x; i < ny * PER; i += blockDim.x) {
+        const int p = spec_pos(order, i / PER);
+        dst[i] = val[(p + (p >> 5)) * PER + i % PER];
     }
 }
 
-template <class V>
+template <class V, class D>
 static cudaError_t natural_launch(const void* data, long long ldK, int ny, int ncols, SpecOrder order, float* dst,
                                   cudaStream_t st)
 {
     // (the attribute's value does not depend on the length: copies of
     // different lengths may be launched side by side)
-    const cudaError_t e = cudaFuncSetAttribute(spectrum_natural<V>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    const cudaError_t e = cudaFuncSetAttribute(spectrum_natural<V, D>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                (int)(sizeof(V) * 28 * 1024));
     if (e != cudaSuccess) return e;
-    spectrum_natural<V><<<ncols, 256, sizeof(V) * (size_t)(ny + ny / 32 + 1), st>>>(static_cast<const V*>(data), ldK, ny, order,
-                                                                    reinterpret_cast<V*>(dst));
+    spectrum_natural<V, D><<<ncols, 256, sizeof(V) * (size_t)(ny + ny / 32 + 1), st>>>(static_cast<const V*>(data), ldK, ny, order,
+                                                                       reinterpret_cast<D*>(dst));
     return cudaGetLastError();
 }
 
 cudaError_t spectrum_copy_natural(const void* data, long long ldK, int ny, int ncols, int is_real, SpecOrder order,
                                   float* dst, cudaStream_t st)
 {
-    return is_real ? natural_launch<float>(data, ldK, ny, ncols, order, dst, st)
-                   : natural_launch<float2>(data, ldK, ny, ncols, order, dst, st);
+    if (is_real) return natural_launch<float, float>(data, ldK, ny, ncols, order, dst, st);
+    return reinterpret_cast<uintptr_t>(dst) % sizeof(float2) == 0
+               ? natural_launch<float2, float2>(data, ldK, ny, ncols, order, dst, st)
+               : natural_launch<float2, float>(data, ldK, ny, ncols, order, dst, st);
 }
 
 }  // namespace lpk

@@ -287,3 +287,34 @@ def test_failed_allocation_gives_kept_memory_back(ctx, by):
     assert torch.cuda.mem_get_info()[0] >= free + size // 2
     torch.cuda.synchronize()
     lp.lp_sync_status(ctx)
+
+
+@pytest.mark.parametrize("symmetric", [True, False])
+@pytest.mark.parametrize("where", ["pinned", "pinned+4", "device+4"])
+def test_copy_writes_any_addressable_destination_itself(ctx, symmetric, where):
+    """Pinned host memory and 4-byte aligned addresses: the same values as an
+    aligned device destination, nothing beside them, and a captured copy is
+    kernels alone (a buffer in between would be an allocation in the graph)."""
+    K = _psf(11)
+    if symmetric:
+        K = K + K.flip(0, 1)
+    spec = lp.lp_kernel_spectrum(ctx, K, pad_ny=210, pad_nx=96)
+    n = 49 * 210 * (1 if symmetric else 2)
+    want = torch.empty(n, device=DEV)
+    lp.lp_spectrum_copy(spec, want)
+    lp.lp_sync_status(ctx)
+    buf = torch.full((n + 4,), -7.0)
+    buf = buf.pin_memory() if where.startswith("pinned") else buf.to(DEV)
+    off = 1 if where.endswith("+4") else 0
+    torch.cuda.synchronize()
+    a = torch.cuda.Stream()
+    with _Capture(a) as c:
+        lp.lp_spectrum_copy(spec, buf[off:off + n], stream=a)
+    kinds = c.node_types()
+    c.destroy()
+    assert kinds and set(kinds) == {0}
+    assert (buf == -7).all()
+    lp.lp_spectrum_copy(spec, buf[off:off + n], stream=a)
+    lp.lp_sync_status(ctx, stream=a)
+    assert torch.equal(buf[off:off + n].to(DEV), want)
+    assert (buf[:off] == -7).all() and (buf[off + n:] == -7).all()
