@@ -388,7 +388,7 @@ cudaError_t p3(const P3Args& a, int nspec, cudaStream_t s)
 }}
 }}  // namespace
 
-extern const SizeKernels kSize_{n} = {{kN, {{{geo}}}, Ge::VK, {ns}, {{{rad6}}}, kBatch ? 1 : 0, kParkG ? 1 : 0, kParkG ? 1 : 0,
+extern const SizeKernels kSize_{n} = {{kN, {{{geo}}}, Ge::VK, {ns}, {{{rad6}}}, kBatch ? 1 : 0, kParkG ? 1 : 0, kParkG ? 1 : 0, CM::NT,
                                        set_attrs, p1, p2, p2m, p3,
                                        kTC ? TP::THREADS : 0, kTcSmem, p2tc}};
 }}  // namespace lpk

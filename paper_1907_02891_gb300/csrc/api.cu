@@ -1074,8 +1074,13 @@ static void map_dims(int h, int w, int ny, int nx, int hk, int wk, lp_outmode mo
     d->batch = (k && k->batch) ? 1 : 0;
 }
 
-// (whole blocks of columns: the passes park up to kUCB columns side by side)
-size_t lp_park_bytes(const MapDims& d) { return 8ull * (size_t)d.ncolsU * (size_t)d.ny; }
+// (whole blocks of the columns that a plan parks side by side)
+size_t lp_park_bytes(const MapDims& d)
+{
+    const SizeKernels* k = find_size(d.ny);
+    const long long nt = k ? k->park_cols : 1;
+    return 8ull * (size_t)std::max(d.ncolsU, (d.ncols + nt - 1) / nt * nt) * (size_t)d.ny;
+}
 
 // the batched column pass parks its forward column spectra in the workspace
 // where they do not fit shared memory next to the exchange buffer

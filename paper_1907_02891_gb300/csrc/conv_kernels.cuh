@@ -174,8 +174,9 @@ __device__ __forceinline__ bool p1_unit_ok(const P1Args& a, int pair)
 }
 
 // P2 unit: column c of T (all ldT rows), of each spectrum, of each of the
-// launch's U blocks (HoutPad rows) and of the park area
-__device__ __forceinline__ bool p2_column_ok(const P2Args& a, int c, int n, int kw)
+// launch's U blocks (HoutPad rows), and the park area up to column park_end
+// (a block's columns are parked interleaved, those past the last one too)
+__device__ __forceinline__ bool p2_column_ok(const P2Args& a, int c, int n, int kw, int park_end)
 {
 #if LP_DEBUG
     const bool t_ok = 2 * t_index4(c, 0, a.ldT / 2) + t_row((int)a.ldT - 1) < a.t_elems && a.H <= a.ldT;
@@ -183,7 +184,7 @@ __device__ __forceinline__ bool p2_column_ok(const P2Args& a, int c, int n, int 
     const bool u_ok = a.HoutPad <= a.ldU &&
                       (long long)(a.nspec - 1) * a.specU + 2 * u_index4(c, 0, a.ldU / 2) + u_row(a.HoutPad - 1) <
                           a.u_elems;
-    const bool p_ok = a.park == nullptr || (long long)(c + 1) * n <= a.park_elems;
+    const bool p_ok = a.park == nullptr || (long long)park_end * n <= a.park_elems;
     (void)kw;
     return lp_checked(a.err, c >= 0 && c < a.ncols && t_ok && k_ok && u_ok && p_ok);
 #else
@@ -191,6 +192,7 @@ __device__ __forceinline__ bool p2_column_ok(const P2Args& a, int c, int n, int 
     (void)c;
     (void)n;
     (void)kw;
+    (void)park_end;
     return true;
 #endif
 }
@@ -687,7 +689,7 @@ __global__ void __launch_bounds__(C::TH, C::MINB) p2_cols(const __grid_constant_
     const int t = threadIdx.x;
     float2* work = lp_dsmem + Ge::W1;
     for (int cl = 0; cl < NT; ++cl)
-        if (c0 + cl < a.ncols && !p2_column_ok(a, c0 + cl, Ge::N, KREAL ? 1 : 2)) return;
+        if (c0 + cl < a.ncols && !p2_column_ok(a, c0 + cl, Ge::N, KREAL ? 1 : 2, c0 + cl + 1)) return;
     if constexpr (R0 > 1) {
         load_w1<Ge>(lp_dsmem, a.tw.w1, t, C::TH);
         column_stage1<C>(a.T, a.ldT, a.H, c0, a.ncols, work, t, C::TH);
@@ -901,7 +903,7 @@ __global__ void __launch_bounds__(C::TH * GRP, C::MINB) p2_cols_multi(const __gr
     constexpr int NT = C::NT;
     const int c0 = blockIdx.x * NT;
     for (int cl = 0; cl < NT; ++cl)
-        if (c0 + cl < a.ncols && !p2_column_ok(a, c0 + cl, Ge::N, KREAL ? 1 : 2)) return;
+        if (c0 + cl < a.ncols && !p2_column_ok(a, c0 + cl, Ge::N, KREAL ? 1 : 2, c0 + NT)) return;
     float2* F = PARKG ? a.park + (size_t)c0 * Ge::N : lp_dsmem + Ge::W1 + GRP * C::WORK;
     const int grp = GRP == 1 ? 0 : threadIdx.x / C::TH;
     const int t = GRP == 1 ? threadIdx.x : threadIdx.x % C::TH;
@@ -933,9 +935,9 @@ struct P2MArgs {
 };
 
 // multiclass unit: column c of every class's T, of every spectrum, of U and of the sums
-__device__ __forceinline__ bool p2m_column_ok(const P2MArgs& m, int c, int n, int kw)
+__device__ __forceinline__ bool p2m_column_ok(const P2MArgs& m, int c, int n, int kw, int park_end)
 {
-    return p2_column_ok(m.a, c, n, kw);
+    return p2_column_ok(m.a, c, n, kw, park_end);
 }
 
 // One class: forward transform of the class's columns, product with its
@@ -974,7 +976,7 @@ __global__ void __launch_bounds__(C::TH, C::MINB) p2_multiclass(const __grid_con
     const P2Args& a = M.a;
     const int c0 = blockIdx.x * NT;
     for (int cl = 0; cl < NT; ++cl)
-        if (c0 + cl < a.ncols && !p2m_column_ok(M, c0 + cl, Ge::N, KREAL ? 1 : 2)) return;
+        if (c0 + cl < a.ncols && !p2m_column_ok(M, c0 + cl, Ge::N, KREAL ? 1 : 2, c0 + NT)) return;
     const float2* F = PARKG ? a.park + (size_t)c0 * Ge::N : lp_dsmem + Ge::W1 + C::WORK;
     load_w1<Ge>(lp_dsmem, a.tw.w1, threadIdx.x, C::TH);
 #pragma unroll 1

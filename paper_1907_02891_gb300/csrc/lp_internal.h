@@ -38,6 +38,7 @@ struct SizeKernels {
     int batch;           // several spectra: one forward column transform, parked
     int park_multi;      // the batched pass parks its column in global memory
     int park_class;      // the Eq. (4) pass keeps its sums in global memory
+    int park_cols;       // columns side by side in a block's parked set
     cudaError_t (*set_attrs)();
     cudaError_t (*p1)(const P1Args&, cudaStream_t);
     cudaError_t (*p2)(const P2Args&, bool kreal, cudaStream_t);
