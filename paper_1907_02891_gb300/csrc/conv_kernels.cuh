@@ -300,46 +300,30 @@ extern __shared__ __align__(16) float2 lp_dsmem[];
 // spectra of a and b need each frequency k = m + R0 (k1 + R1 k2) together
 // with N - k.  That partner lies in sub-transform R0 - m (m = 0: in itself),
 // at k1' = R1 - 1 - k1, k2' = R2 - 1 - k2 (m = 0: k1' = (R1 - k1) mod R1, and
-// for k1 = 0 the run's own element (R2 - k2) mod R2).  Where a sub-transform
-// takes half a warp or less, a warp handles m and R0 - m side by side (RowSub)
-// and the partners are exchanged by shuffles, each lane handing over the
-// upper half of its run; else a sweep through shared memory combines them.
+// for k1 = 0 the run's own element (R2 - k2) mod R2).  Where a transform is
+// one sub-transform (R0 = 1) its lanes exchange the partners by shuffles
+// (RowSub), each handing over the upper half of its run; else a sweep through
+// shared memory combines them (shuffles between the lanes of m and R0 - m were
+// slower at 4704: forward 44 -> 58-65, inverse 41 -> 43-50 us, T and U then
+// being accessed in 16-byte pieces of distinct lines).
 // ---------------------------------------------------------------------------
+// A lane's place in round `round` of the transforms of a block, R0 = 1
 template <class C>
 struct RowSub {
     using Ge = typename C::Ge;
-    static constexpr int R0 = Ge::R0, G = Ge::G;
-    static constexpr bool SHUFFLE = R0 == 1;
-    static constexpr int LANES = R0 == 1 ? G : 2 * G;             // lanes of a unit
-    static constexpr int PU = R0 == 1 ? 1 : R0 / 2 + R0 % 2;      // units of a transform: {m, R0 - m}, {0, R0 / 2}
-    static constexpr int UNITS = PU * C::NT;
-    static constexpr int FLIGHT = SHUFFLE ? C::TH / LANES : 1;
-    static constexpr int ROUNDS = (UNITS + FLIGHT - 1) / FLIGHT;
-    int tr, m, li, partner;  // transform, sub-transform, lane in the group, partner's lane in the warp
-    bool live, origin;       // origin: the run k1 = 0 of m = 0
+    static constexpr int G = Ge::G;
+    static constexpr int FLIGHT = C::TH / G;  // transforms at a time
+    static constexpr int ROUNDS = (C::NT + FLIGHT - 1) / FLIGHT;
+    int tr, li, partner;  // transform, lane in the group, partner's lane in the warp
+    bool live, origin;    // origin: the run k1 = 0
     __device__ __forceinline__ RowSub(int t, int round)
     {
-        const int q = t / LANES + round * FLIGHT;
+        tr = t / G + round * FLIGHT;
         li = t % G;
-        tr = C::NT == 1 ? 0 : q / PU;
-        const int pu = q - tr * PU, half = R0 == 1 ? 0 : (t / G) & 1;
-        live = ROUNDS * FLIGHT == UNITS || q < UNITS;
-        bool self;
-        if (R0 == 1) {
-            m = 0;
-            self = true;
-        } else if (pu == 0) {
-            m = half ? R0 / 2 : 0;
-            if (R0 % 2 && half) live = false;  // odd R0: sub-transform 0 has the warp's half for itself
-            self = true;
-        } else {
-            m = half ? R0 - pu : pu;
-            self = false;
-        }
-        const int kp = m == 0 ? (li == 0 ? 0 : Ge::R1 - li) : Ge::R1 - 1 - li;
+        live = ROUNDS * FLIGHT == C::NT || tr < C::NT;
+        origin = li == 0;
         const int lane = t & 31;
-        partner = ((lane - li) ^ (self ? 0 : G)) + (li < Ge::R1 ? kp : li);
-        origin = m == 0 && li == 0;
+        partner = lane - li + (origin || li >= Ge::R1 ? li : Ge::R1 - li);
     }
 };
 
@@ -414,22 +398,17 @@ __global__ void __launch_bounds__(C::TH, C::MINB) p1_rows(const __grid_constant_
     }
     const long long ldq = a.ldT / 2;
     float4* Tq = reinterpret_cast<float4*>(a.T + blockIdx.y * a.specT);
-    if constexpr (RS::SHUFFLE) {
+    if constexpr (R0 == 1) {
 #pragma unroll 1
         for (int e = 0; e < RS::ROUNDS; ++e) {
             const RS s(t, e);
-            float2* b = work + s.tr * La::ELEMS + s.m * La::S0;
+            float2* b = work + s.tr * La::ELEMS;
             if (s.live && s.li < R2) {
                 float2 x[R1];
-                if constexpr (R0 > 1) {
+                const RowInput in(a, pair0 + s.tr);
 #pragma unroll
-                    for (int l = 0; l < R1; ++l) x[l] = b[s.li + l * La::S1];
-                } else {
-                    const RowInput in(a, pair0 + s.tr);
-#pragma unroll
-                    for (int l = 0; l < R1; ++l) x[l] = in(s.li + l * R2);
-                }
-                stage2_fwd<Ge>(x, b, s.m, s.li, lp_dsmem, a.tw.w2);
+                for (int l = 0; l < R1; ++l) x[l] = in(s.li + l * R2);
+                stage2_fwd<Ge>(x, b, 0, s.li, lp_dsmem, a.tw.w2);
             }
             __syncwarp();
             float2 f[R2];
@@ -439,7 +418,7 @@ __global__ void __launch_bounds__(C::TH, C::MINB) p1_rows(const __grid_constant_
             }
             const int pair = pair0 + s.tr;
             const bool store = s.live && s.li < R1 && pair < a.npairs;
-            const int u = s.m + R0 * s.li;
+            const int u = s.li;
             float4* dst = Tq + t_index4(u, pair, ldq);
 #pragma unroll
             for (int k = 0; k <= R2 / 2; ++k) {
@@ -1034,16 +1013,15 @@ __global__ void __launch_bounds__(C::TH, C::MINB) p3_rows(const __grid_constant_
         }
     };
     if constexpr (R0 > 1) load_w1<Ge>(lp_dsmem, a.tw.w1, t, C::TH);
-    if constexpr (RS::SHUFFLE) {
-        if constexpr (R0 > 1) __syncthreads();  // w1
+    if constexpr (R0 == 1) {
 #pragma unroll 1
         for (int e = 0; e < RS::ROUNDS; ++e) {
             const RS s(t, e);
-            float2* b = work + s.tr * La::ELEMS + s.m * La::S0;
+            float2* b = work + s.tr * La::ELEMS;
             const int pair = pair0 + s.tr;
             const bool load = s.live && s.li < R1 && pair < a.npairs;
             const bool vb = 2 * pair + 1 < a.Hout;
-            const int u = s.m + R0 * s.li;
+            const int u = s.li;
             const float4* src = Uq + u_index4(u, pair, ldq);
             float4 q[R2 / 2 + 1];
 #pragma unroll
@@ -1078,7 +1056,7 @@ __global__ void __launch_bounds__(C::TH, C::MINB) p3_rows(const __grid_constant_
                 store_run<Ge>(f, b, s.li);
             }
             __syncwarp();
-            if (s.live && s.li < R2) finish(s.tr, s.m, s.li, b);
+            if (s.live && s.li < R2) finish(s.tr, 0, s.li, b);
         }
     } else {
 #pragma unroll 1
