@@ -5,9 +5,10 @@ each with one candidate factorisation N = R0 R1 R2 and one launch shape of
 the passes (transforms per block, threads, resident blocks per SM), times
 the three passes of a map whose padded size is N x N on the GPU, and keeps,
 for the factorisation whose best passes sum lowest, the best shape of each
-pass.  With several spectra per map it times the shapes of the batched column
-pass (and its groups per block) at that factorisation, against one
-single-spectrum pass per spectrum.  The result is written to
+pass.  With several spectra per map (--nspec) it times the shapes of the
+batched column pass (and its groups per block), against one single-spectrum
+pass per spectrum, at the two best factorisations, and weighs maps of one
+spectrum and of several together.  The result is written to
 ``tuned_plans.json`` beside this file (or to the file $LP_TUNE_CACHE names)
 as the entry's "geo"; ``build.py`` uses it for every length it lists.
 
@@ -86,6 +87,7 @@ def candidate_shapes(r: Sequence[int], limit: int, parked: bool = False) -> List
 
 def _compile_common(jobs: int) -> List[str]:
     os.makedirs(os.path.join(TUNE_DIR, "common"), exist_ok=True)
+    os.makedirs(B.OBJ, exist_ok=True)
     deps = max(os.path.getmtime(h) for h in B._headers())
     srcs = [os.path.join(B.CSRC, f) for f in COMMON_SRCS]
     with cf.ThreadPoolExecutor(jobs) as ex:
@@ -219,27 +221,37 @@ def tune_size(n: int, quick: bool, jobs: int, common: List[str], log, side: int 
     got = run(plans)
     if not got:
         raise RuntimeError(f"no variant of {n} ran")
-    best = None
+    geos = []
     for r in {tuple(p["geo"]["r"]) for p, _ in got}:
         rs = [(p, t) for p, t in got if tuple(p["geo"]["r"]) == r]
         pick = [min(rs, key=lambda x, k=k: x[1][k]) for k in PASSES]
         total = sum(t[k] for k, (_, t) in zip(PASSES, pick))
-        if best is None or total < best[0]:
-            best = (total, r, [p["geo"][k] for k, (p, _) in zip(("p1", "p2", "p3"), pick)])
-    total, r, (s1, s2, s3) = best
-    out = dict(base, packed=True, geo=dict(B.geo_plan(r), p1=s1, p2=s2, p3=s3))
+        shapes = [p["geo"][k] for k, (p, _) in zip(("p1", "p2", "p3"), pick)]
+        geos.append((total, dict(base, packed=True, geo=dict(B.geo_plan(r), p1=shapes[0], p2=shapes[1], p3=shapes[2]))))
+    geos.sort(key=lambda x: x[0])
+    scored = []
+    # with several spectra: the two best factorisations (the second where it is
+    # within 4 %), by the passes of a map of one spectrum plus 2 / nspec of
+    # those of a map of nspec
+    for total, out in geos[:2] if nspec > 1 else geos[:1]:
+        if total > 1.04 * geos[0][0]:
+            break
+        score = total
+        if nspec > 1:
+            multi = [dict(out, batch=False)]
+            for s in candidate_shapes(out["geo"]["r"], 4 if quick else 8, parked=True):
+                for grp in (1, 2, 3):
+                    if s[1] * grp <= 1024:
+                        multi.append(dict(out, batch=True, geo=dict(out["geo"], pm=s, grp=grp)))
+            out, t = min(run(multi, ns=nspec), key=lambda x: x[1]["p2_cols"])
+            score = total + 2.0 / nspec * sum(t[k] for k in PASSES)
+        scored.append((score, total, out))
+    _, total, out = min(scored, key=lambda x: x[0])
     # packed FP32x2 arithmetic, and the trigger of the next pass: whole maps
     late = list(base.get("late", B.DEFAULT_LATE))
     whole = run([dict(out, packed=pk, late=l) for pk in (True, False) for l in (late, [0, 0, 0])], whole=True)
     pick = min(whole, key=lambda x: x[1]["map"])
     out = dict(pick[0], tuned_total_us=total * 1e3, tuned_map_us=pick[1]["map"] * 1e3)
-    if nspec > 1:
-        multi = [dict(out, batch=False)]
-        for s in candidate_shapes(r, 4 if quick else 8, parked=True):
-            for grp in (1, 2, 3):
-                if s[1] * grp <= 1024:
-                    multi.append(dict(out, batch=True, geo=dict(out["geo"], pm=s, grp=grp)))
-        out = min(run(multi, ns=nspec), key=lambda x: x[1]["p2_cols"])[0]
     log(f"N={n}: chose {out['geo']} packed={out['packed']} late={out.get('late')} batch={out.get('batch')} "
         f"(passes {out['tuned_total_us']:.1f} us, map {out['tuned_map_us']:.1f} us)")
     return out
