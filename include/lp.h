@@ -89,7 +89,12 @@ lp_status lp_create(lp_ctx** ctx, int device, size_t hbm_budget_bytes);
 /* Release everything the context owns (waits for its work to finish). */
 void lp_destroy(lp_ctx* ctx);
 
-/* Device bytes currently held by the context. */
+/*
+ * Device bytes currently held by the context.  Not counted: scratch of spectrum
+ * builds, and up to 256 MB of freed spectrum memory that a context without a
+ * budget keeps for the next build; that is given back when one of the context's
+ * allocations fails, and by lp_destroy.
+ */
 size_t lp_bytes_in_use(const lp_ctx* ctx);
 
 /*
